@@ -13,6 +13,7 @@
 #include <cstdio>
 #include <cstring>
 #include <fstream>
+#include <map>
 #include <mutex>
 #include <sstream>
 #include <string>
@@ -92,6 +93,8 @@ struct gbmd_system {
   double* d_thermo = nullptr;
 };
 
+constexpr int TEAM_SIDES = 4;   // cluster sizes 16, 8, 4, 2, 1: the first on the group's stream
+
 struct Group {
   int device = 0;
   std::vector<gbmd_system*> members;   // may contain nullptr (free slots of a batch)
@@ -108,14 +111,15 @@ struct Group {
   Tile* d_te = nullptr;   // energy/virial launches: EV_TILE_P particles per tile, whatever
                           // the tuning, so the FP64 sums do not depend on it
   Tile* d_tt = nullptr;   // tree-list systems: tiles over their trees' leaves
-  int ntp = 0, ntf = 0, ntc = 0, nts = 0, ntb = 0, ntbk = 0, nte = 0, ntt = 0;
+  Tile* d_tn = nullptr;   // list build by four warps per cell (few cells): (cell, part) items
+  int ntp = 0, ntf = 0, ntc = 0, nts = 0, ntb = 0, ntbk = 0, nte = 0, ntt = 0, ntn = 0;
   size_t cap_desc = 0, cap_tp = 0, cap_tf = 0, cap_tc = 0, cap_ts = 0, cap_part = 0;
-  size_t cap_tb = 0, cap_tbk = 0, cap_te = 0, cap_tt = 0;
+  size_t cap_tb = 0, cap_tbk = 0, cap_te = 0, cap_tt = 0, cap_tn = 0;
   bool any_cell = true;   // some member builds its list from cells
   int window_cap = 0;                        // largest staged window among members
   bool nvt = false;                          // the members integrate NVT (all or none)
   int eval = EVAL_LJ;                        // the members' pair evaluator (all the same)
-  double* d_nhpart = nullptr;                // NVT: per-step-tile v.v partial sums
+  double* d_nhpart = nullptr;                // NVT: v.v partial sums per chunk of a system
   size_t cap_nhpart = 0;
   double* d_partials = nullptr;
   GroupCtl* d_ctl = nullptr;
@@ -127,6 +131,17 @@ struct Group {
   bool layout_dirty = true;
   bool graphs_dirty = true;
   bool use_graphs = true;
+  // the members that the team kernel steps (positions among the live members, the
+  // largest first); the others, if any, are stepped by the graph of `rest`
+  std::vector<int> team;
+  int* d_team = nullptr;
+  size_t cap_team = 0;
+  std::vector<int> team_n;             // their particles
+  int team_max_n = 0;
+  cudaStream_t side[TEAM_SIDES] = {};
+  cudaEvent_t side_ev[TEAM_SIDES + 1] = {};
+  Group* rest = nullptr;
+  bool is_rest = false;
 };
 
 namespace {
@@ -157,6 +172,23 @@ int grow(T** p, size_t* cap, size_t need) {
   return GBMD_OK;
 }
 
+void destroy_graphs(Group* g);
+
+// the group's device tables and graphs
+void free_group(Group* g) {
+  if (g->rest) free_group(g->rest);
+  destroy_graphs(g);
+  for (cudaStream_t st : g->side)
+    if (st) cudaStreamDestroy(st);
+  for (cudaEvent_t e : g->side_ev)
+    if (e) cudaEventDestroy(e);
+  for (void* p : {(void*)g->d_desc, (void*)g->d_tp, (void*)g->d_tf, (void*)g->d_tc, (void*)g->d_te,
+                  (void*)g->d_nhpart, (void*)g->d_ts, (void*)g->d_tb, (void*)g->d_tbk, (void*)g->d_tt,
+                  (void*)g->d_tn, (void*)g->d_team, (void*)g->d_partials, (void*)g->d_ctl})
+    cudaFree(p);
+  delete g;
+}
+
 void destroy_graphs(Group* g) {
   if (g->exec_many) cudaGraphExecDestroy(g->exec_many);
   if (g->exec_one) cudaGraphExecDestroy(g->exec_one);
@@ -167,12 +199,75 @@ void destroy_graphs(Group* g) {
   g->graphs_dirty = true;
 }
 
+// Which list builder serves the rebuild's own launch (the rows are the same): four warps
+// per cell (k_nlist_split) while a launch has few cells, else one warp per cell (k_nlist).
+// One build, ncu: 8 cells (N = 500) 25 against 107 us; 2,744 cells (N = 64,000) 81 against
+// 51 us; the lines cross near the cells of a 20,000-particle system (729: 40.4 against
+// 43.6 us a step with a build every eighth).
+constexpr int SPLIT_MAX_CELLS = 1024;
+bool use_split(const std::vector<gbmd_system*>& m) {
+  long long cells = 0;
+  for (auto* s : m) {
+    if (s->h.staged) return false;   // staged rows hold window indices: k_nlist's
+    if (!s->h.tree) cells += s->h.ncells;
+  }
+  return cells > 0 && cells <= SPLIT_MAX_CELLS;
+}
+// blocks per cell: one for every 32 particles of the mean occupation
+int split_parts(const SysDev& d) { return std::max(1, (d.n / d.ncells + 31) / 32); }
+
+// Systems that the team kernel may step: the cell list on the global force path,
+// without ghosts (their rebuilds are the caller's).  Alone it pays while a step is short
+// beside the launches it saves: up to TEAM_ALONE_N particles (64,000, mixed: 27.7 us a
+// step against 28.2 by the step kernel and k_rebuild; 200,000: 73 against 66; FP64 at
+// 64,000: 223 against 223).  In a batch, where a shared launch makes every member wait
+// for any member's rebuild, up to what one cluster steps in about 50 us.
+constexpr int TEAM_ALONE_N = 49152;
+constexpr int TEAM_CLUSTER_N = 32768;
+constexpr int TEAM_STEPS = 64;   // steps of one launch
+bool team_member(const Group* g, const SysDev& d) {
+  return !d.tree && !d.staged && d.n_ghost == 0 && d.n <= (g->is_batch ? TEAM_CLUSTER_N : TEAM_ALONE_N);
+}
+
 // Rebuild descriptor copies and tile tables for the group's current members.
 int sync_layout(Group* g) {
   if (!g->layout_dirty) return GBMD_OK;
   std::vector<gbmd_system*> m = live(g);
+  g->team.clear();
+  g->team_max_n = 0;
+  std::vector<gbmd_system*> others;
+  if (g->use_graphs && !g->is_rest)
+    for (size_t k = 0; k < m.size(); ++k) {
+      if (team_member(g, m[k]->h)) {
+        g->team.push_back((int)k);
+        g->team_max_n = std::max(g->team_max_n, m[k]->h.n);
+      } else {
+        others.push_back(m[k]);
+      }
+    }
+  std::stable_sort(g->team.begin(), g->team.end(), [&](int a, int b) { return m[a]->h.n > m[b]->h.n; });
+  g->team_n.clear();
+  for (int k : g->team) g->team_n.push_back(m[k]->h.n);
+  if (!g->team.empty() && !others.empty()) {
+    if (!g->rest) {
+      g->rest = new Group();
+      g->rest->is_rest = true;
+      g->rest->is_batch = true;
+    }
+    Group* r = g->rest;
+    r->device = g->device;
+    r->precision = g->precision;
+    r->stream = g->stream;
+    r->tpp = g->tpp;
+    r->fblock = g->fblock;
+    r->members = others;
+    r->layout_dirty = true;
+  } else if (g->rest) {
+    g->rest->members.clear();
+    g->rest->layout_dirty = true;
+  }
   std::vector<SysDev> desc;
-  std::vector<Tile> tp, tf, tc, ts, tb, tbk, te, tt;
+  std::vector<Tile> tp, tf, tc, ts, tb, tbk, te, tt, tn;
   const int per_f = g->fblock / g->tpp;
   g->multi = 0;
   g->rel = true;
@@ -180,6 +275,8 @@ int sync_layout(Group* g) {
   g->nvt = !m.empty() && m[0]->h.nvt;
   g->eval = m.empty() ? EVAL_LJ : m[0]->h.eval;
   g->any_cell = false;
+  const bool split = use_split(m);
+  int nh_chunks = 0;
   for (size_t k = 0; k < m.size(); ++k) {
     SysDev d = m[k]->h;
     const int n = d.n;
@@ -191,15 +288,20 @@ int sync_layout(Group* g) {
       for (int b = 0; b < d.nblocks; b += 8) tbk.push_back({(int)k, b, std::min(8, d.nblocks - b), 0});
       g->window_cap = std::max(g->window_cap, d.window_cap);
     } else {
-      d.tile_first_s = (int)tf.size();
       for (int f = 0; f < n; f += per_f) tf.push_back({(int)k, f, std::min(per_f, n - f), 0});
-      d.tile_count_s = (int)tf.size() - d.tile_first_s;
+      d.nh_first = nh_chunks;
+      d.nh_count = (int)(((long long)n * g->tpp + 31) / 32);
+      nh_chunks += d.nh_count;
       d.tile_first_f = (int)te.size();   // partial sums come from the energy launches
       for (int f = 0; f < n; f += EV_TILE_P) te.push_back({(int)k, f, std::min(EV_TILE_P, n - f), 0});
       d.tile_count_f = (int)te.size() - d.tile_first_f;
     }
     for (int c = 0; c < d.nbins; c += CELLS_PER_TILE)
       tc.push_back({(int)k, c, std::min(CELLS_PER_TILE, d.nbins - c), 0});
+    if (split && !d.tree) {
+      const int parts = split_parts(d);
+      for (int c = 0; c < d.nbins * parts; ++c) tn.push_back({(int)k, c / parts, c % parts, parts});
+    }
     ts.push_back({(int)k, 0, 0, 0});
     if (d.tree)
       for (int f = 0; f < d.tree_leaves_total; f += TILE_P)
@@ -214,7 +316,7 @@ int sync_layout(Group* g) {
   for (auto& d : desc)
     if (d.staged) d.tile_first_f += (int)te.size();   // staged partial sums follow the global ones
   RET(grow(&g->d_partials, &g->cap_part, 8 * std::max<size_t>(te.size() + tb.size(), 1)));
-  RET(grow(&g->d_nhpart, &g->cap_nhpart, std::max<size_t>(tf.size(), 1)));
+  RET(grow(&g->d_nhpart, &g->cap_nhpart, std::max<size_t>(nh_chunks, 1)));
   for (auto& d : desc) {
     d.partials = g->d_partials;
     d.nh_part = g->d_nhpart;
@@ -228,6 +330,8 @@ int sync_layout(Group* g) {
   RET(grow(&g->d_tbk, &g->cap_tbk, tbk.size()));
   RET(grow(&g->d_te, &g->cap_te, te.size()));
   RET(grow(&g->d_tt, &g->cap_tt, tt.size()));
+  RET(grow(&g->d_tn, &g->cap_tn, tn.size()));
+  RET(grow(&g->d_team, &g->cap_team, g->team.size()));
   if (!g->d_ctl) {
     CK(cudaMalloc(&g->d_ctl, sizeof(GroupCtl)));
     CK(cudaMemsetAsync(g->d_ctl, 0, sizeof(GroupCtl), g->stream));
@@ -245,6 +349,9 @@ int sync_layout(Group* g) {
   CK(up(g->d_tbk, tbk));
   CK(up(g->d_te, te));
   CK(up(g->d_tt, tt));
+  CK(up(g->d_tn, tn));
+  if (!g->team.empty())
+    CK(cudaMemcpyAsync(g->d_team, g->team.data(), g->team.size() * sizeof(int), cudaMemcpyHostToDevice, g->stream));
   CK(cudaStreamSynchronize(g->stream));   // host vectors die here
   g->ntp = (int)tp.size();
   g->ntf = (int)tf.size();
@@ -254,6 +361,7 @@ int sync_layout(Group* g) {
   g->ntbk = (int)tbk.size();
   g->nte = (int)te.size();
   g->ntt = (int)tt.size();
+  g->ntn = (int)tn.size();
   g->layout_dirty = false;
   destroy_graphs(g);
   return GBMD_OK;
@@ -279,7 +387,9 @@ std::vector<KernelCall> rebuild_calls(const Group* g) {
                                permute_call(g->d_desc, g->d_tp, g->ntp, g->d_ctl),
                                copyback_call(g->d_desc, g->d_tp, g->ntp, g->d_ctl)};
   if (g->ntbk > 0) v.push_back(blocks_call(g->d_desc, g->d_tbk, g->ntbk, g->d_ctl));
-  if (g->any_cell)
+  if (g->ntn > 0)
+    v.push_back(nlist_split_call(g->d_desc, g->d_tn, g->ntn, g->d_ctl, g->multi > 0));
+  else if (g->any_cell)
     v.push_back(nlist_call(g->d_desc, g->d_tc, g->ntc, g->d_ctl, g->rel, g->multi, g->ntbk > 0));
   if (g->ntt > 0) {
     v.push_back(tree_build_call(g->d_desc, g->d_tt, g->ntt, g->d_ctl));
@@ -343,6 +453,58 @@ std::vector<KernelCall> step_calls(const Group* g, cudaGraphConditionalHandle co
   return v;
 }
 
+// what a team kernel may use of the device, asked once per kernel and device
+struct TeamFit { int sms = 0, blocks_per_sm = 0, max_cluster = 0; };
+int team_fit(void* f, int threads, size_t smem, int dev, TeamFit* out) {
+  static std::mutex mu;
+  static std::map<std::pair<int, void*>, TeamFit> known;
+  std::lock_guard<std::mutex> lock(mu);
+  auto it = known.find({dev, f});
+  if (it != known.end()) {
+    *out = it->second;
+    return GBMD_OK;
+  }
+  TeamFit t;
+  CK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  CK(cudaDeviceGetAttribute(&t.sms, cudaDevAttrMultiProcessorCount, dev));
+  CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&t.blocks_per_sm, f, threads, smem));
+  CK(cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  for (int c = TEAM_MAX_CLUSTER; c >= 1 && !t.max_cluster; c /= 2) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(c);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim = {(unsigned)c, 1, 1};
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    int num = 0;
+    if (cudaOccupancyMaxActiveClusters(&num, f, &cfg) == cudaSuccess && num > 0) t.max_cluster = c;
+    else cudaGetLastError();
+  }
+  known[{dev, f}] = t;
+  *out = t;
+  return GBMD_OK;
+}
+
+// The rebuild of a step of one system alone as one cooperative kernel after the step
+// kernel (no conditional node); null func: the group does not take it.  Up to COOP_MAX_N
+// particles: the separate kernels of a big rebuild balance better over the SMs than
+// resident warps do (KA 10^6: 312 us a step with the conditional node, 357 with this;
+// N = 200,000: 70 and 66).
+constexpr int COOP_MAX_N = 400000;
+int coop_rebuild(const Group* g, KernelCall* out) {
+  out->func = nullptr;
+  std::vector<gbmd_system*> m = live(g);
+  if (m.size() != 1 || m[0]->h.staged || m[0]->h.tree || m[0]->h.n > COOP_MAX_N) return GBMD_OK;
+  TeamFit fit;
+  RET(team_fit(rebuild_func(g->multi > 0), REBUILD_T, REBUILD_SMEM, g->device, &fit));
+  if (fit.blocks_per_sm < 1) return GBMD_OK;
+  *out = rebuild_call(g->d_desc, fit.sms, g->d_ctl, g->multi > 0);
+  return GBMD_OK;
+}
+
 int add_kernel(cudaGraph_t graph, const cudaGraphNode_t* dep, const KernelCall& k,
                cudaGraphNode_t* out) {
   cudaKernelNodeParams p{};
@@ -355,6 +517,11 @@ int add_kernel(cudaGraph_t graph, const cudaGraphNode_t* dep, const KernelCall& 
   p.kernelParams = a;
   p.extra = nullptr;
   CK(cudaGraphAddKernelNode(out, graph, dep, dep ? 1 : 0, &p));
+  if (k.cooperative) {
+    cudaKernelNodeAttrValue v{};
+    v.cooperative = 1;
+    CK(cudaGraphKernelNodeSetAttribute(*out, cudaLaunchAttributeCooperative, &v));
+  }
   return GBMD_OK;
 }
 
@@ -363,11 +530,12 @@ int build_graph(Group* g, int nsteps, cudaGraphExec_t* exec) {
   CK(cudaGraphCreate(&graph, 0));
   const bool events = nsteps == 1 && g->ev_begin && g->ev_end;
   cudaGraphNode_t prev = nullptr;
-  const int nsys = (int)live(g).size();
-  int rc = GBMD_OK;
+  KernelCall coop;
+  int rc = coop_rebuild(g, &coop);
   for (int st = 0; st < nsteps && rc == GBMD_OK; ++st) {
-    cudaGraphConditionalHandle h;
-    cudaError_t e = cudaGraphConditionalHandleCreate(&h, graph, 0, cudaGraphCondAssignDefault);
+    cudaGraphConditionalHandle h = 0;
+    cudaError_t e = coop.func ? cudaSuccess
+                              : cudaGraphConditionalHandleCreate(&h, graph, 0, cudaGraphCondAssignDefault);
     if (e != cudaSuccess) { rc = fail(GBMD_ERR_CUDA, "conditional handle: %s", cudaGetErrorString(e)); break; }
     // force + integrate (event nodes around them when asked), then IF(rebuild){lists}
     cudaGraphNode_t before = prev;
@@ -377,7 +545,7 @@ int build_graph(Group* g, int nsteps, cudaGraphExec_t* exec) {
       if (e != cudaSuccess) { rc = fail(GBMD_ERR_CUDA, "event node: %s", cudaGetErrorString(e)); break; }
       before = g->node_ev_begin;
     }
-    for (const KernelCall& k : step_calls(g, h, 1)) {
+    for (const KernelCall& k : step_calls(g, h, coop.func ? 0 : 1)) {
       cudaGraphNode_t n5;
       rc = add_kernel(graph, before ? &before : nullptr, k, &n5);
       if (rc) break;
@@ -388,6 +556,13 @@ int build_graph(Group* g, int nsteps, cudaGraphExec_t* exec) {
       e = cudaGraphAddEventRecordNode(&g->node_ev_end, graph, &before, 1, g->ev_end);
       if (e != cudaSuccess) { rc = fail(GBMD_ERR_CUDA, "event node: %s", cudaGetErrorString(e)); break; }
       before = g->node_ev_end;
+    }
+    if (coop.func) {
+      cudaGraphNode_t nr;
+      rc = add_kernel(graph, &before, coop, &nr);
+      if (rc) break;
+      prev = nr;
+      continue;
     }
     cudaGraphNodeParams cp{};
     cp.type = cudaGraphNodeTypeConditional;
@@ -426,10 +601,109 @@ int ensure_graphs(Group* g) {
   return GBMD_OK;
 }
 
-// enqueue n steps of the group (graphs, or direct launches when graphs are off)
+// the streams that a batch's classes run on beside the group's own, and their events
+// (event 0: the fork)
+int team_stream(Group* g, size_t q) {
+  if (!g->side_ev[0]) CK(cudaEventCreateWithFlags(&g->side_ev[0], cudaEventDisableTiming));
+  if (g->side[q - 1]) return GBMD_OK;
+  CK(cudaEventCreateWithFlags(&g->side_ev[q], cudaEventDisableTiming));
+  CK(cudaStreamCreateWithFlags(&g->side[q - 1], cudaStreamNonBlocking));
+  return GBMD_OK;
+}
+
+// n steps of the group's team members, one launch per TEAM_STEPS steps.  A system
+// alone takes one cluster up to TEAM_CLUSTER_CHUNKS warps' work a step (FP64, bound by
+// the SMs' FP64 pipes: one block's warps), and every SM beyond that (N = 2,000, mixed: 8.1
+// us a step either way; N = 4,000: 12 on a cluster of 16, 9 on the grid).  A batch's
+// members take clusters of 16, 8, .. 1 blocks by their own size, one launch a size, side
+// by side on streams of their own, the largest first.  A step is shortest with few warps
+// on an SM, the SMs' throughput best with many: a block gets two warps' work while all
+// clusters then fit the SMs at once, else up to four turns of its warps.
+constexpr int TEAM_CLUSTER_CHUNKS = 128;
+int team_cluster(int chunks, int per_block, int most) {
+  int c = 1;
+  while (c < most && (long long)c * per_block < chunks) c *= 2;
+  return c;
+}
+int launch_team(Group* g, long long n) {
+  void* f = k_team_variant(g->eval, g->precision, g->tpp, g->multi);
+  TeamFit fit;
+  RET(team_fit(f, TEAM_T, TEAM_SMEM, g->device, &fit));
+  if (fit.max_cluster < 1) return fail(GBMD_ERR_CUDA, "the team kernel does not fit the device");
+  const int warps = TEAM_T / 32;
+  auto chunks_of = [&](int nn) { return (int)(((long long)nn * g->tpp + 31) / 32); };
+  TeamArgs a{};
+  a.desc = g->d_desc;
+  a.ctl = g->d_ctl;
+  cudaLaunchConfig_t cfg{};
+  cfg.blockDim = dim3(TEAM_T);
+  cfg.dynamicSmemBytes = TEAM_SMEM;
+  cudaLaunchAttribute at{};
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  void* args[1] = {&a};
+  // the classes: [first, last) of the list, blocks per team
+  struct Class { int first, last, cluster; };
+  std::vector<Class> cls;
+  const int most = g->precision == GBMD_FP64 ? warps : TEAM_CLUSTER_CHUNKS;
+  if (!g->is_batch && chunks_of(g->team_max_n) > most) {
+    cls.push_back({0, 1, 0});
+  } else {
+    int per_block = 2;
+    for (; per_block < 4 * warps; per_block *= 2) {
+      long long blocks = 0;
+      for (int nn : g->team_n) blocks += team_cluster(chunks_of(nn), per_block, fit.max_cluster);
+      if (blocks <= fit.sms) break;
+    }
+    for (int k = 0; k < (int)g->team.size(); ++k) {
+      const int c = team_cluster(chunks_of(g->team_n[k]), per_block, fit.max_cluster);
+      if (cls.empty() || cls.back().cluster != c) cls.push_back({k, k, c});
+      cls.back().last = k + 1;
+    }
+  }
+  for (long long k = 0; k < n; k += TEAM_STEPS) {
+    a.nsteps = (int)std::min<long long>(TEAM_STEPS, n - k);
+    for (size_t q = 0; q < cls.size(); ++q) {
+      const Class& c = cls[q];
+      a.list = g->d_team + c.first;
+      a.cluster = c.cluster;
+      cfg.stream = g->stream;
+      if (q > 0) {
+        RET(team_stream(g, q));
+        if (k == 0) CK(cudaStreamWaitEvent(g->side[q - 1], g->side_ev[0], 0));
+        cfg.stream = g->side[q - 1];
+      } else if (k == 0 && cls.size() > 1) {
+        RET(team_stream(g, 1));
+        CK(cudaEventRecord(g->side_ev[0], g->stream));
+      }
+      if (c.cluster) {
+        cfg.gridDim = dim3((unsigned)(c.last - c.first) * c.cluster);
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim = {(unsigned)c.cluster, 1, 1};
+      } else {
+        cfg.gridDim = dim3(fit.blocks_per_sm * fit.sms);
+        at.id = cudaLaunchAttributeCooperative;
+        at.val.cooperative = 1;
+      }
+      CK(cudaLaunchKernelExC(&cfg, f, args));
+    }
+  }
+  for (size_t q = 1; q < cls.size(); ++q) {
+    CK(cudaEventRecord(g->side_ev[q], g->side[q - 1]));
+    CK(cudaStreamWaitEvent(g->stream, g->side_ev[q], 0));
+  }
+  return GBMD_OK;
+}
+
+// enqueue n steps of the group: by the team kernel, and (members it does not take; event
+// records around the force kernel; graphs switched off) graphs or direct launches
 int enqueue_steps(Group* g, long long n) {
   if (n <= 0 || live(g).empty()) return GBMD_OK;
   RET(sync_layout(g));
+  if (!g->team.empty() && !(g->ev_begin && g->ev_end)) {
+    RET(launch_team(g, n));
+    return g->rest ? enqueue_steps(g->rest, n) : GBMD_OK;
+  }
   if (g->use_graphs) {
     RET(ensure_graphs(g));
     for (long long k = 0; k < n / STEPS_PER_GRAPH; ++k) CK(cudaGraphLaunch(g->exec_many, g->stream));
@@ -525,6 +799,13 @@ int sync_system(gbmd_system* s) {
       RET(write_flags(s, &f, st));
       RET(rebuild_and_force(s, 0));   // finishes the interrupted step
       continue;
+    }
+    if (f.error == DEV_TEAM) {   // arrivals may be left over: the next launch starts clean
+      for (Group* g : {s->own, s->batch})
+        if (g && g->d_ctl)
+          CK(cudaMemsetAsync(&g->d_ctl->team_arrive, 0, sizeof(g->d_ctl->team_arrive), g->stream));
+      CK(cudaStreamSynchronize(st));
+      return fail(GBMD_ERR_TIMEOUT, "a wait between thread blocks ran out (step %lld)", f.step);
     }
     if (f.error == DEV_TREE)
       return fail(GBMD_ERR_TIMEOUT, "a tree traversal passed its node bound (step %lld)", f.step);
@@ -1408,12 +1689,7 @@ int gbmd_destroy(gbmd_system* s) {
   if (s->own) cudaStreamSynchronize(s->own->stream);
   for (void* p : s->allocs) cudaFree(p);
   if (s->own) {
-    Group* g = s->own;
-    destroy_graphs(g);
-    cudaFree(g->d_desc); cudaFree(g->d_tp); cudaFree(g->d_tf); cudaFree(g->d_tc); cudaFree(g->d_te); cudaFree(g->d_nhpart);
-    cudaFree(g->d_ts); cudaFree(g->d_tb); cudaFree(g->d_tbk); cudaFree(g->d_tt); cudaFree(g->d_partials);
-    cudaFree(g->d_ctl);
-    delete g;
+    free_group(s->own);
   }
   delete s;
   return GBMD_OK;
@@ -1869,11 +2145,7 @@ int gbmd_batch_destroy(gbmd_batch* bh) {
     s->batch_slot = -1;
     s->own->stream = s->stream;
   }
-  destroy_graphs(b);
-  cudaFree(b->d_desc); cudaFree(b->d_tp); cudaFree(b->d_tf); cudaFree(b->d_tc); cudaFree(b->d_te); cudaFree(b->d_nhpart);
-  cudaFree(b->d_ts); cudaFree(b->d_tb); cudaFree(b->d_tbk); cudaFree(b->d_tt); cudaFree(b->d_partials);
-  cudaFree(b->d_ctl);
-  delete b;
+  free_group(b);
   return GBMD_OK;
 }
 

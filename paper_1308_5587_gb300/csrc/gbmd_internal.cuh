@@ -35,11 +35,14 @@ constexpr int MAXT2 = MAXT * MAXT;
 
 // error codes stored in Flags::error (positive on the device)
 enum DevError : int { DEV_OK = 0, DEV_OVERFLOW = 1, DEV_NONFINITE = 2, DEV_BADTYPE = 3, DEV_WINDOW = 4,
-                      DEV_TREE = 5 /* a tree traversal ran past its node bound */ };
+                      DEV_TREE = 5 /* a tree traversal ran past its node bound */,
+                      DEV_TEAM = 6 /* a wait of the team kernel ran out */ };
 
 // staged force tiles: aligned 2x2x2 blocks of cells; their 4x4x4-cell window is
 // staged in shared memory (at most window_cap particles)
 constexpr int WIN_CELLS = 64;
+
+constexpr int CPOS_TYPE_SHIFT = 30;   // n <= 2^30, at most 4 types
 
 struct Flags {
   int rebuild_req;          // set by the step kernel when r_buff/2 is exceeded
@@ -126,7 +129,8 @@ struct SysDev {
   unsigned* tree_arrive;   // per node: children arrived during the build (reset to 0)
   unsigned* fkey;          // [N] the particle's fine Morton code at the last build (every
                            // system: the order inside a cell)
-  int4* cpos;              // [N] position shadow of member m (cell order) at the last build
+  int4* cpos;              // [N] position shadow of member m (cell order) at the last build,
+                           // w = its index | type << CPOS_TYPE_SHIFT
   int4* tree_q;            // [N] the leaves' particles in leaf order: (x, y, z, index)
   // the list kernel visits the types in decreasing order of their expected query work
   // (sum over t of n_t r_list(type, t)^3): launch positions tree_qpos[k] .. belong to
@@ -149,13 +153,13 @@ struct SysDev {
   int sort_period;
   double dt, h;            // h = dt / (2 m)
   // NVT (Nose-Hoover, MTK form): nh = {xi, eta, exp(-xi dt/2), 0} on the device;
-  // nh_part: the group's per-step-tile partial sums of v.v; tile_first_s /
-  // tile_count_s: this system's tiles of the step's force launch
+  // nh_part: the group's partial sums of v.v, one per chunk of 32 / TPP particles, this
+  // system's from nh_first on
   int nvt;
   double kT, tau, gdof;    // gdof = 3N - 3
   double* nh;
   double* nh_part;
-  int tile_first_s, tile_count_s;
+  int nh_first, nh_count;
   double dtq[3];           // dt * 2^32 / L: the drift in box-fraction units
   double mass;
   int eval;                // PairEval of the system's potential
@@ -194,6 +198,9 @@ struct GroupCtl {
   unsigned int blocks_done_a;   // last-block counter of the NVT force half
   int any_rebuild;
   unsigned long long launches;
+  // barrier of a team that is a whole grid (k_team.cuh): arrivals with their votes, and
+  // the generation that releases the waiting blocks
+  unsigned long long team_arrive, team_release;
 };
 
 struct Tile { int sys, first, count, pad; };

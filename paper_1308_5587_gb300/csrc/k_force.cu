@@ -204,6 +204,24 @@ __global__ void __launch_bounds__(STAGED_BLOCK) k_force_staged(const SysDev* __r
 }
 
 
+#define TEAM_DECL(e) \
+  void* k_team_##e##_mixed(int tpp, int mt); \
+  void* k_team_##e##_fp64(int tpp, int mt);
+TEAM_DECL(lj)
+TEAM_DECL(mie)
+TEAM_DECL(yukawa)
+TEAM_DECL(gauss)
+#undef TEAM_DECL
+void* k_team_variant(int eval, int prec, int tpp, int mt) {
+  const bool d = prec == GBMD_FP64;
+  switch (eval) {
+    case EVAL_MIE: return d ? k_team_mie_fp64(tpp, mt) : k_team_mie_mixed(tpp, mt);
+    case EVAL_YUKAWA: return d ? k_team_yukawa_fp64(tpp, mt) : k_team_yukawa_mixed(tpp, mt);
+    case EVAL_GAUSS: return d ? k_team_gauss_fp64(tpp, mt) : k_team_gauss_mixed(tpp, mt);
+    default: return d ? k_team_lj_fp64(tpp, mt) : k_team_lj_mixed(tpp, mt);
+  }
+}
+
 bool tpp_supported(int tpp) { return tpp == 1 || tpp == 2 || tpp == 4; }
 
 // multi: 0 = one type, 1 = at most two types, 2 = up to MAXT types

@@ -206,6 +206,169 @@ __device__ __forceinline__ void pair2(const int4& qi, const int4& qa, const int4
   }
 }
 
+// The sums over the neighbour row of particle i, particle's lane h of TPP: slot groups
+// h, h + TPP, .. in order, U of them in flight (4 U gathers), pairs two at a time.  The
+// order of the sums does not depend on U.  COH: the positions and the list may have
+// been written by this kernel (plain loads), else they are read-only here.
+template <bool COH, typename T>
+__device__ __forceinline__ T load_ro(const T* p) {
+  if constexpr (COH) return *p;
+  else return __ldg(p);
+}
+// four list entries: read once, so they do not push the neighbours' positions out of L1
+template <bool COH>
+__device__ __forceinline__ int4 load_list(const int4* p) {
+  int4 v;
+  if constexpr (COH)
+    asm volatile("ld.global.L1::no_allocate.v4.s32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  else
+    asm("ld.global.nc.L1::no_allocate.v4.s32 {%0, %1, %2, %3}, [%4];"
+        : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
+  return v;
+}
+template <int TPP, int MT, int EVAL, bool EV, bool COH, int U>
+__device__ __forceinline__ void gather_mixed(const SysDev& s, const int4* qv, const int4& qi, int i,
+                                             int h, int n, const PairF* tabf, float2& fx,
+                                             float2& fy, float2& fz, float2& e, float2* w) {
+  const int nt = s.ntypes;
+  const int groups = (n + 3) >> 2;
+  const int4* nl4 = reinterpret_cast<const int4*>(s.nl) + i;
+  const size_t stride = (size_t)s.nl_stride;
+  const int cap_groups = s.cap >> 2;
+  // the first slot groups of this lane, fetched before the count is known
+  int4 jn[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u)
+    jn[u] = h + u * TPP < cap_groups ? load_list<COH>(nl4 + (size_t)(h + u * TPP) * stride)
+                                     : make_int4(i, i, i, i);
+  const float2 sc0 = make_float2(s.fscale[0], s.fscale[0]);
+  const float2 sc1 = make_float2(s.fscale[1], s.fscale[1]);
+  const float2 sc2 = make_float2(s.fscale[2], s.fscale[2]);
+  const PairF p0 = s.pf[0];
+  // two types: particle i's row of the pair table stays in registers, so a
+  // neighbour's parameters are a select, not a shared-memory load per pair
+  const PairF r0 = MT == 1 ? s.pf[qi.w * nt] : p0;
+  const PairF r1 = MT == 1 ? s.pf[qi.w * nt + nt - 1] : p0;
+  auto par = [&](int tj) -> PairF {
+    if (MT == 0) return p0;
+    if (MT == 1) return tj ? r1 : r0;
+    return tabf[qi.w * nt + tj];
+  };
+  fx = fy = fz = e = make_float2(0.f, 0.f);
+  for (int c = 0; c < 6; ++c) w[c] = fx;
+  for (int gg = h; gg < groups; gg += U * TPP) {
+    int4 q[U][4];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int k0 = (gg + u * TPP) << 2;
+      const int4 jc = jn[u];
+      q[u][0] = load_ro<COH>(qv + (k0 < n ? jc.x : i));
+      q[u][1] = load_ro<COH>(qv + (k0 + 1 < n ? jc.y : i));
+      q[u][2] = load_ro<COH>(qv + (k0 + 2 < n ? jc.z : i));
+      q[u][3] = load_ro<COH>(qv + (k0 + 3 < n ? jc.w : i));
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int g2 = gg + (U + u) * TPP;
+      if (g2 < groups) jn[u] = load_list<COH>(nl4 + (size_t)g2 * stride);
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int k0 = (gg + u * TPP) << 2;
+      const bool o0 = k0 < n, o1 = k0 + 1 < n, o2 = k0 + 2 < n, o3 = k0 + 3 < n;
+      const int4 q0 = q[u][0], q1 = q[u][1], q2 = q[u][2], q3 = q[u][3];
+      const PairF P0 = par(q0.w), P1 = par(q1.w), P2 = par(q2.w), P3 = par(q3.w);
+      pair2<EVAL, EV>(qi, q0, q1, o0, o1, sc0, sc1, sc2, P0, P1, fx, fy, fz, e, w);
+      pair2<EVAL, EV>(qi, q2, q3, o2, o3, sc0, sc1, sc2, P2, P3, fx, fy, fz, e, w);
+    }
+  }
+}
+
+template <int TPP, int MT, int EVAL, bool EV, bool COH>
+__device__ __forceinline__ void gather_fp64(const SysDev& s, const double4_32a* pv, const int4* qv,
+                                            const double4_32a& pi, int i, int h, int n,
+                                            const PairF* tabf, const PairD* tabd, double& fx,
+                                            double& fy, double& fz, double& e, double* w) {
+  const int nt = s.ntypes, ti = (int)__double_as_longlong(pi.w);
+  const int groups = (n + 3) >> 2;
+  const int4* nl4 = reinterpret_cast<const int4*>(s.nl) + i;
+  const size_t stride = (size_t)s.nl_stride;
+  int4 jn = h < (s.cap >> 2) ? load_list<COH>(nl4 + (size_t)h * stride) : make_int4(i, i, i, i);
+  // the FP32 pre-test reads the fixed-point shadow qv of the same positions
+  const int4 qi = qv[i];
+  const float fs0 = s.fscale[0], fs1 = s.fscale[1], fs2 = s.fscale[2];
+  const float cut0 = s.pf[0].rc2 * FP64_PRETEST_MARGIN;
+  const double L0 = s.L[0], L1 = s.L[1], L2 = s.L[2];
+  const int h0 = __double2hiint(s.halfL[0]), h1 = __double2hiint(s.halfL[1]),
+            h2 = __double2hiint(s.halfL[2]);
+  const PairD p0 = s.pd[0];
+  fx = fy = fz = e = 0.0;
+  for (int c = 0; c < 6; ++c) w[c] = 0.0;
+  for (int gg = h; gg < groups; gg += TPP) {
+    const int4 jc = jn;
+    if (gg + TPP < groups) jn = load_list<COH>(nl4 + (size_t)(gg + TPP) * stride);
+    const int k0 = gg << 2;
+    const int jj[4] = {jc.x, jc.y, jc.z, jc.w};
+    double4_32a pp[4];
+    int4 qq[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int j = k0 + u < n ? jj[u] : i;   // own slot: unused
+      pp[u] = pv[j];
+      qq[u] = load_ro<COH>(qv + j);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      // FP32 pre-test on the fixed-point difference (the exact minimum image): a
+      // pair beyond r_cut by more than the margin skips the FP64 work, which it
+      // would not pass; every other pair is decided in FP64 below
+      const float ex = (float)min_image_fixed(qi.x, qq[u].x) * fs0;
+      const float ey = (float)min_image_fixed(qi.y, qq[u].y) * fs1;
+      const float ez = (float)min_image_fixed(qi.z, qq[u].z) * fs2;
+      const float r2f = fmaf(ex, ex, fmaf(ey, ey, ez * ez));
+      const float cut = MT ? tabf[ti * nt + qq[u].w].rc2 * FP64_PRETEST_MARGIN : cut0;
+      if (!(k0 + u < n) || !(r2f < cut)) continue;
+      const double4_32a pj = pp[u];
+      double dx = pi.x - pj.x, dy = pi.y - pj.y, dz = pi.z - pj.z;
+      // minimum image: |d| < L; the test on the high words is exact except within
+      // 2^-20 of L/2, where either choice leaves |d| ~ L/2 > r_cut.  Only pairs
+      // across a box face need it, so a warp takes the correction (FP64 adds on
+      // every lane once the compiler turns it into selects) only when one of its
+      // pairs does
+      const bool wx = (__double2hiint(dx) & 0x7fffffff) > h0;
+      const bool wy = (__double2hiint(dy) & 0x7fffffff) > h1;
+      const bool wz = (__double2hiint(dz) & 0x7fffffff) > h2;
+      if (__any_sync(__activemask(), wx || wy || wz)) {
+        if (wx) dx -= copysign(L0, dx);
+        if (wy) dy -= copysign(L1, dy);
+        if (wz) dz -= copysign(L2, dz);
+      }
+      const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
+      const PairD P = MT ? tabd[ti * nt + (int)__double_as_longlong(pj.w)] : p0;
+      // both positive, so the bit patterns order like the values
+      const bool in = k0 + u < n && __double_as_longlong(r2) < __double_as_longlong(P.rc2);
+      if (in) {
+        double v;
+        const double f = eval_f64<EVAL, EV>(r2, P, v);
+        fx = fma(f, dx, fx);
+        fy = fma(f, dy, fy);
+        fz = fma(f, dz, fz);
+        if (EV) {
+          e += 0.5 * v;
+          const double hf = 0.5 * f;
+          w[0] = fma(hf * dx, dx, w[0]);
+          w[1] = fma(hf * dx, dy, w[1]);
+          w[2] = fma(hf * dx, dz, w[2]);
+          w[3] = fma(hf * dy, dy, w[3]);
+          w[4] = fma(hf * dy, dz, w[4]);
+          w[5] = fma(hf * dz, dz, w[5]);
+        }
+      }
+    }
+  }
+}
+
 // MODE_FORCE: forces at the current positions (readouts); MODE_EV: also the
 // energy / virial / v.v partial sums; MODE_STEP: the step kernel -- forces, then each
 // particle's velocity Verlet update into the next shadow buffer (step_core.cuh), then
@@ -248,44 +411,11 @@ __device__ __forceinline__ void force_body(const SysDev* __restrict__ sysv,
   if (active) {
   const int n = valid ? s.nn[i] : 0;
   if (STEP && valid && h == 0) prefetch_particle(s, i);   // in flight during the gathers
-  const int groups = (n + 3) >> 2;
-  const int4* __restrict__ nl4 = reinterpret_cast<const int4*>(s.nl) + i;
-  const size_t stride = (size_t)s.nl_stride;
-  const int cap_groups = s.cap >> 2;
-  // first slot group of this lane, fetched before the count is known
-  int4 jn = h < cap_groups ? __ldg(nl4 + (size_t)h * stride) : make_int4(i, i, i, i);
-
   if (PREC == GBMD_MIXED) {
     const int4* __restrict__ qv = q_at(s, step);
     const int4 qi = qv[i];
-    const float2 sc0 = make_float2(s.fscale[0], s.fscale[0]);
-    const float2 sc1 = make_float2(s.fscale[1], s.fscale[1]);
-    const float2 sc2 = make_float2(s.fscale[2], s.fscale[2]);
-    const PairF p0 = s.pf[0];
-    // two types: particle i's row of the pair table stays in registers, so a
-    // neighbour's parameters are a select, not a shared-memory load per pair
-    const PairF r0 = MT == 1 ? s.pf[qi.w * nt] : p0;
-    const PairF r1 = MT == 1 ? s.pf[qi.w * nt + nt - 1] : p0;
-    auto par = [&](int tj) -> PairF {
-      if (MT == 0) return p0;
-      if (MT == 1) return tj ? r1 : r0;
-      return tabf[qi.w * nt + tj];
-    };
-    float2 fx = make_float2(0.f, 0.f), fy = fx, fz = fx, e = fx;
-    float2 w[6] = {fx, fx, fx, fx, fx, fx};
-    for (int gg = h; gg < groups; gg += TPP) {
-      const int4 jc = jn;
-      if (gg + TPP < groups) jn = __ldg(nl4 + (size_t)(gg + TPP) * stride);
-      const int k0 = gg << 2;
-      const bool o0 = k0 < n, o1 = k0 + 1 < n, o2 = k0 + 2 < n, o3 = k0 + 3 < n;
-      const int4 q0 = __ldg(qv + (o0 ? jc.x : i));
-      const int4 q1 = __ldg(qv + (o1 ? jc.y : i));
-      const int4 q2 = __ldg(qv + (o2 ? jc.z : i));
-      const int4 q3 = __ldg(qv + (o3 ? jc.w : i));
-      const PairF P0 = par(q0.w), P1 = par(q1.w), P2 = par(q2.w), P3 = par(q3.w);
-      pair2<EVAL, EV>(qi, q0, q1, o0, o1, sc0, sc1, sc2, P0, P1, fx, fy, fz, e, w);
-      pair2<EVAL, EV>(qi, q2, q3, o2, o3, sc0, sc1, sc2, P2, P3, fx, fy, fz, e, w);
-    }
+    float2 fx, fy, fz, e, w[6];
+    gather_mixed<TPP, MT, EVAL, EV, false, 1>(s, qv, qi, i, h, n, tabf, fx, fy, fz, e, w);
     // the two halves of each packed accumulator, then the TPP lanes
     const float Fx = group_sum<TPP>(fx.x + fx.y);
     const float Fy = group_sum<TPP>(fy.x + fy.y);
@@ -304,7 +434,7 @@ __device__ __forceinline__ void force_body(const SysDev* __restrict__ sysv,
     } else if (NVTA) {   // closing half kick and scaling; the second half reads F
       if (valid && h == 0) {
         const double f[3] = {widen_f32(Fx, bad), widen_f32(Fy, bad), widen_f32(Fz, bad)};
-        uu = nvt_close(s, i, f, fw.v_full);
+        uu = nvt_close(s, i, f, fw.v_full, s.nh[2]);
         s.f32[i] = make_float4(Fx, Fy, Fz, 0.f);
       }
     } else if (valid && h == 0) {
@@ -324,86 +454,15 @@ __device__ __forceinline__ void force_body(const SysDev* __restrict__ sysv,
     const double4_32a* __restrict__ pv = p64_at(s, step);
     const double4_32a pi = pv[i];
     const int ti = (int)__double_as_longlong(pi.w);
-    // the FP32 pre-test reads the fixed-point shadow of the same positions
-    const int4* __restrict__ qv = q_at(s, step);
-    const int4 qi = qv[i];
-    const float fs0 = s.fscale[0], fs1 = s.fscale[1], fs2 = s.fscale[2];
-    const float cut0 = s.pf[0].rc2 * FP64_PRETEST_MARGIN;
-    const double L0 = s.L[0], L1 = s.L[1], L2 = s.L[2];
-    const int h0 = __double2hiint(s.halfL[0]), h1 = __double2hiint(s.halfL[1]),
-              h2 = __double2hiint(s.halfL[2]);
-    const PairD p0 = s.pd[0];
-    double fx = 0, fy = 0, fz = 0, e = 0;
-    double w0 = 0, w1 = 0, w2 = 0, w3 = 0, w4 = 0, w5 = 0;
-    for (int gg = h; gg < groups; gg += TPP) {
-      const int4 jc = jn;
-      if (gg + TPP < groups) jn = __ldg(nl4 + (size_t)(gg + TPP) * stride);
-      const int k0 = gg << 2;
-      const int jj[4] = {jc.x, jc.y, jc.z, jc.w};
-      double4_32a pp[4];
-      int4 qq[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int j = k0 + u < n ? jj[u] : i;   // own slot: unused
-        pp[u] = pv[j];
-        qq[u] = __ldg(qv + j);
-      }
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        // FP32 pre-test on the fixed-point difference (the exact minimum image): a
-        // pair beyond r_cut by more than the margin skips the FP64 work, which it
-        // would not pass; every other pair is decided in FP64 below
-        const float ex = (float)min_image_fixed(qi.x, qq[u].x) * fs0;
-        const float ey = (float)min_image_fixed(qi.y, qq[u].y) * fs1;
-        const float ez = (float)min_image_fixed(qi.z, qq[u].z) * fs2;
-        const float r2f = fmaf(ex, ex, fmaf(ey, ey, ez * ez));
-        const float cut = MT ? tabf[ti * nt + qq[u].w].rc2 * FP64_PRETEST_MARGIN : cut0;
-        if (!(k0 + u < n) || !(r2f < cut)) continue;
-        const double4_32a pj = pp[u];
-        double dx = pi.x - pj.x, dy = pi.y - pj.y, dz = pi.z - pj.z;
-        // minimum image: |d| < L; the test on the high words is exact except within
-        // 2^-20 of L/2, where either choice leaves |d| ~ L/2 > r_cut.  Only pairs
-        // across a box face need it, so a warp takes the correction (FP64 adds on
-        // every lane once the compiler turns it into selects) only when one of its
-        // pairs does
-        const bool wx = (__double2hiint(dx) & 0x7fffffff) > h0;
-        const bool wy = (__double2hiint(dy) & 0x7fffffff) > h1;
-        const bool wz = (__double2hiint(dz) & 0x7fffffff) > h2;
-        if (__any_sync(__activemask(), wx || wy || wz)) {
-          if (wx) dx -= copysign(L0, dx);
-          if (wy) dy -= copysign(L1, dy);
-          if (wz) dz -= copysign(L2, dz);
-        }
-        const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
-        const PairD P = MT ? tabd[ti * nt + (int)__double_as_longlong(pj.w)] : p0;
-        // both positive, so the bit patterns order like the values
-        const bool in = k0 + u < n && __double_as_longlong(r2) < __double_as_longlong(P.rc2);
-        if (in) {
-          double v;
-          const double f = eval_f64<EVAL, EV>(r2, P, v);
-          fx = fma(f, dx, fx);
-          fy = fma(f, dy, fy);
-          fz = fma(f, dz, fz);
-          if (EV) {
-            e += 0.5 * v;
-            const double hf = 0.5 * f;
-            w0 = fma(hf * dx, dx, w0);
-            w1 = fma(hf * dx, dy, w1);
-            w2 = fma(hf * dx, dz, w2);
-            w3 = fma(hf * dy, dy, w3);
-            w4 = fma(hf * dy, dz, w4);
-            w5 = fma(hf * dz, dz, w5);
-          }
-        }
-      }
-    }
+    double fx, fy, fz, e, w[6];
+    gather_fp64<TPP, MT, EVAL, EV, false>(s, pv, q_at(s, step), pi, i, h, n, tabf, tabd, fx, fy, fz,
+                                          e, w);
     fx = group_sum<TPP>(fx);
     fy = group_sum<TPP>(fy);
     fz = group_sum<TPP>(fz);
     if (EV) {
       e = group_sum<TPP>(e);
-      w0 = group_sum<TPP>(w0); w1 = group_sum<TPP>(w1); w2 = group_sum<TPP>(w2);
-      w3 = group_sum<TPP>(w3); w4 = group_sum<TPP>(w4); w5 = group_sum<TPP>(w5);
+      for (int c = 0; c < 6; ++c) w[c] = group_sum<TPP>(w[c]);
     }
     if (STEP) {
       if (valid && h == 0) {
@@ -415,16 +474,16 @@ __device__ __forceinline__ void force_body(const SysDev* __restrict__ sysv,
     } else if (NVTA) {
       if (valid && h == 0) {
         const double f[3] = {fx, fy, fz};
-        uu = nvt_close(s, i, f, fw.v_full);
+        uu = nvt_close(s, i, f, fw.v_full, s.nh[2]);
         s.f64[i] = make_double4_32a(fx, fy, fz, 0.0);
       }
     } else if (valid && h == 0) {
       s.f64[i] = make_double4_32a(fx, fy, fz, EV ? e : 0.0);
     }
     if (EV) {
-      double vals[NPART] = {valid ? e : 0.0,  valid ? w0 : 0.0, valid ? w1 : 0.0, valid ? w2 : 0.0,
-                            valid ? w3 : 0.0, valid ? w4 : 0.0, valid ? w5 : 0.0,
-                            valid ? vsq(s, i, fx, fy, fz, fw.v_full) : 0.0};
+      double vals[NPART] = {valid ? e : 0.0};
+      for (int c = 0; c < 6; ++c) vals[c + 1] = valid ? w[c] : 0.0;
+      vals[7] = valid ? vsq(s, i, fx, fy, fz, fw.v_full) : 0.0;
       if (valid && h == 0 && s.pp_u) {
         s.pp_u[i] = vals[0];
         for (int c = 0; c < 6; ++c) s.pp_w[6 * (size_t)i + c] = vals[c + 1];
@@ -436,7 +495,9 @@ __device__ __forceinline__ void force_body(const SysDev* __restrict__ sysv,
   if (STEP) step_tail(s, sysv, ctl, nsys, total_blocks, cond, use_cond, need, bad);
   if (NVTA) {
     if (bad) atomicCAS(&s.flags->error, 0, (int)DEV_NONFINITE);
-    nvt_half_tail(s, sysv, ctl, nsys, total_blocks, uu);
+    const int p0 = (int)(threadIdx.x & ~31u) / TPP;   // this warp's first particle of the tile
+    nvt_half_tail(s, sysv, ctl, nsys, total_blocks, uu,
+                  p0 < t.count ? (t.first + p0) / (32 / TPP) : -1);
   }
 }
 

@@ -1,0 +1,8 @@
+// k_team_lj_fp64.cu -- the LJ (and WCA) instances of the team kernel (k_team.cuh), FP64.
+#include "k_team.cuh"
+
+namespace gbmd {
+
+void* k_team_lj_fp64(int tpp, int mt) { return k_team_tpp<EVAL_LJ, GBMD_FP64>(tpp, mt); }
+
+}  // namespace gbmd

@@ -1,0 +1,8 @@
+// k_team_yukawa_mixed.cu -- the yukawa instances of the team kernel (k_team.cuh), mixed precision.
+#include "k_team.cuh"
+
+namespace gbmd {
+
+void* k_team_yukawa_mixed(int tpp, int mt) { return k_team_tpp<EVAL_YUKAWA, GBMD_MIXED>(tpp, mt); }
+
+}  // namespace gbmd

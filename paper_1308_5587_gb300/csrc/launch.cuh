@@ -18,6 +18,7 @@ struct KernelCall {
   void* func;
   dim3 grid, block;
   size_t smem;
+  bool cooperative;
   int nargs;
   alignas(16) unsigned char store[10][16];
 };
@@ -38,6 +39,12 @@ KernelCall copyback_call(const SysDev* d, const Tile* tiles_p, int ntiles, Group
 KernelCall blocks_call(const SysDev* d, const Tile* tiles_b, int ntiles, GroupCtl* ctl);
 KernelCall nlist_call(const SysDev* d, const Tile* tiles_c, int ntiles, GroupCtl* ctl, bool rel,
                       bool multi, bool staged);
+// all of the above for the single system d[0], by the grid of a cooperative launch (no
+// staged window, no tree); returns at once when the step asked for no rebuild
+void* rebuild_func(bool multi);
+KernelCall rebuild_call(const SysDev* d, int blocks, GroupCtl* ctl, bool multi);
+// the same rows built by four warps per cell (tiles over (cell, part) items)
+KernelCall nlist_split_call(const SysDev* d, const Tile* tiles_n, int ntiles, GroupCtl* ctl, bool multi);
 // tree neighbour list (k_tree.cu): the boxes of every type's tree (one thread per
 // leaf; tiles over the system's leaves), then the list (one thread per particle in
 // cell order; tiles over particles)
@@ -89,6 +96,24 @@ KernelCall nlist_export_call(const SysDev* d, const Tile* tiles_p, int ntiles, i
                              int* idx, int cap_out, int* too_many);
 
 cudaError_t launch(const KernelCall& k, cudaStream_t st);
+
+// the team kernel (k_team.cuh): many steps of one or more systems in one launch
+// one block an SM, 128 registers a thread: no spills, and the warps a small system fills;
+// the rest of the SM's 256 KB stays L1 for the force phase's gathers
+constexpr int TEAM_T = 512;
+constexpr size_t TEAM_SMEM = 112 * 1024;
+// the rebuild alone: more warps, 80 registers each
+constexpr int REBUILD_T = 768;
+constexpr size_t REBUILD_SMEM = 220 * 1024;
+constexpr int TEAM_MAX_CLUSTER = 16;
+struct TeamArgs {
+  const SysDev* desc;
+  const int* list;   // the systems of the launch (positions in desc), the largest first
+  GroupCtl* ctl;
+  int nsteps;
+  int cluster;       // blocks of a team; 0: the grid is one team
+};
+void* k_team_variant(int eval, int prec, int tpp, int mt);
 
 // arithmetic throughput probe (k_probe.cu): one timed launch over every SM
 cudaError_t probe_run(int kind, cudaStream_t st, int iters, double* ops, float* ms);

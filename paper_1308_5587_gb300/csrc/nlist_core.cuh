@@ -5,11 +5,42 @@
 // NL_BAND of r_list^2 is decided again in FP64, exactly as the reference
 // definition computes it (the FP32 error is below 2e-6 relative).
 #pragma once
+#include <type_traits>
+
 #include "launch.cuh"
 
 namespace gbmd {
 
 constexpr float NL_BAND = 1e-5f;
+constexpr int NL_TYPE_SHIFT = CPOS_TYPE_SHIFT;   // a candidate's word: j | type << 30
+// a culled candidate is at least this factor beyond the largest r_list^2 (1 + band)
+// from the warp's box, far above the FP32 rounding of the box distance
+constexpr float NL_CULL_MARGIN = 1e-4f;
+
+// fixed-point coordinate of the centre of cell c of nc along an axis
+__device__ __forceinline__ int cell_centre_fixed(int c, int nc) {
+  const unsigned long long u = ((2ull * (unsigned long long)c + 1ull) << 32) / (2ull * (unsigned long long)nc);
+  return (int)((unsigned int)u ^ 0x80000000u);
+}
+
+__device__ __forceinline__ float warp_min(float v) {
+  for (int o = 16; o > 0; o >>= 1) v = fminf(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
+}
+__device__ __forceinline__ float warp_max(float v) {
+  for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+  return v;
+}
+// distance of c from the interval [lo, hi] (0 inside)
+__device__ __forceinline__ float gap_to(float c, float lo, float hi) {
+  return fmaxf(fmaxf(lo - c, c - hi), 0.0f);
+}
+// shift the sign bit of v into the low end of m (candidate k of a chunk of mm
+// ends at bit mm - 1 - k)
+__device__ __forceinline__ unsigned push_sign(unsigned m, float v) {
+  return __funnelshift_l(__float_as_uint(v), m, 1);
+}
+
 
 // this step rebuilds the system's lists (decided by the last block of the step)
 __device__ __forceinline__ bool rebuilding(const SysDev& s) {

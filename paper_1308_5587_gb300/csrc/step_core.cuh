@@ -58,6 +58,7 @@ struct ParticleState {
   double v[3], xq[3];
   int4 qb;   // shadow at the last list build
 };
+template <bool COH = false>   // COH: q_build may have been written by this kernel
 __device__ __forceinline__ ParticleState load_particle(const SysDev& s, int i) {
   ParticleState p;
   const int n = s.n;
@@ -66,7 +67,7 @@ __device__ __forceinline__ ParticleState load_particle(const SysDev& s, int i) {
     p.v[a] = s.v[a * n + i];
     p.xq[a] = s.x[a * n + i];
   }
-  p.qb = __ldg(s.q_build + i);
+  p.qb = COH ? s.q_build[i] : __ldg(s.q_build + i);
   return p;
 }
 
@@ -131,10 +132,10 @@ __device__ __forceinline__ void integrate_one(const SysDev& s, int i, int ty, co
 // thermostat scaling of the previous step, u = (v + h F) exp(-xi dt/2) (just u = v
 // right after create / set_state, when v holds full-step velocities); u is stored
 // as the velocity and u.u returned for the kinetic energy.  The scale factor
-// exp(-xi dt/2) is the one the previous step's opening half used (nh[2]).
-__device__ __forceinline__ double nvt_close(const SysDev& s, int i, const double f[3], int vfull) {
+// exp(-xi dt/2) is the one the previous step's opening half used (`sc`, nh[2]).
+__device__ __forceinline__ double nvt_close(const SysDev& s, int i, const double f[3], int vfull,
+                                            double sc) {
   const int n = s.n;
-  const double sc = s.nh[2];
   double uu = 0.0;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
@@ -146,34 +147,72 @@ __device__ __forceinline__ double nvt_close(const SysDev& s, int i, const double
   return uu;
 }
 
-// FP64 sum over the block in a fixed order (warp shuffles, then the warps in order);
-// the result is valid in thread 0
-__device__ __forceinline__ double block_sum_fixed(double v) {
-  __shared__ double wsum[32];
+// The sum of v.v over a system, in an order that depends on the lanes per particle alone
+// and not on how the particles are spread over blocks or kernels: a warp's particles
+// (32 / TPP consecutive ones, a chunk) by shuffles, the chunks' sums in NH_SLOTS strided
+// slots, the slots in a tree.
+constexpr int NH_SLOTS = 256;
+__device__ __forceinline__ double nh_warp_sum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  if (l == 0) wsum[w] = v;
+  return v;   // lane 0
+}
+// every thread of the block calls it; the sum is returned to all
+__device__ __forceinline__ double nh_total(const double* part, int count, double* slots) {
+  for (int v = threadIdx.x; v < NH_SLOTS; v += blockDim.x) {
+    double a = 0.0;
+    int k = v;
+    for (; k + 3 * NH_SLOTS < count; k += 4 * NH_SLOTS) {   // four loads in flight (from L2:
+      double p[4];                                          // other blocks wrote them)
+#pragma unroll
+      for (int u = 0; u < 4; ++u) p[u] = __ldcg(part + k + u * NH_SLOTS);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) a += p[u];
+    }
+    for (; k < count; k += NH_SLOTS) a += __ldcg(part + k);
+    slots[v] = a;
+  }
   __syncthreads();
-  double t = 0.0;
-  if (threadIdx.x == 0)
-    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) t += wsum[k];
+  for (int w = NH_SLOTS / 2; w > 0; w >>= 1) {
+    for (int v = threadIdx.x; v < w; v += blockDim.x) slots[v] += slots[v + w];
+    __syncthreads();
+  }
+  const double r = slots[0];
   __syncthreads();
-  return t;
+  return r;
 }
 
-// End of the NVT force half, every block: publish this block's v.v partial sum and
-// count the arrival; the last block updates every NVT system's thermostat
-// (closing half of the previous step, then opening half of this one, with
-// G = (2K/(g kT) - 1)/tau^2 at the kinetic energy K of the closing velocities):
+// The thermostat (xi, eta) between two steps, from the sum of v.v of the closing
+// velocities: the closing half of the previous step, then the opening half of this one,
+// with G = (2K/(g kT) - 1)/tau^2 at their kinetic energy K:
 //   eta += dt/2 xi;  xi += dt/2 G;     (skipped right after create / set_state)
-//   xi += dt/2 G;    eta += dt/2 xi;   exp(-xi dt/2) for the opening scaling
+//   xi += dt/2 G;    eta += dt/2 xi;   returns exp(-xi dt/2) for the opening scaling
+__device__ __forceinline__ double nh_update(const SysDev& s, double sum, int vfull, double& xi,
+                                            double& eta) {
+  const double K = 0.5 * s.mass * sum;
+  const double G = (2.0 * K / (s.gdof * s.kT) - 1.0) / (s.tau * s.tau);
+  const double hdt = 0.5 * s.dt;
+  if (!vfull) {
+    eta += hdt * xi;
+    xi += hdt * G;
+  }
+  xi += hdt * G;
+  eta += hdt * xi;
+  return exp(-hdt * xi);
+}
+
+// End of the NVT force half, every block: publish the warps' v.v sums (chunk `chunk` of
+// the system for this warp, -1: none) and count the arrival; the last block updates
+// every NVT system's thermostat.
 __device__ __forceinline__ void nvt_half_tail(const SysDev& s, const SysDev* __restrict__ sysv,
                                               GroupCtl* ctl, int nsys, int total_blocks,
-                                              double uu) {
-  const double part = block_sum_fixed(uu);
+                                              double uu, int chunk) {
+  const double part = nh_warp_sum(uu);
+  if ((threadIdx.x & 31) == 0 && chunk >= 0) s.nh_part[s.nh_first + chunk] = part;
   __shared__ int last;
+  __shared__ double slots[NH_SLOTS];
+  __threadfence();
+  __syncthreads();
   if (threadIdx.x == 0) {
-    s.nh_part[blockIdx.x] = part;
     __threadfence();
     last = (atomicAdd(&ctl->blocks_done_a, 1u) == (unsigned)total_blocks - 1u);
   }
@@ -186,24 +225,12 @@ __device__ __forceinline__ void nvt_half_tail(const SysDev& s, const SysDev* __r
     const FlagWords w = load_flag_words(sk.flags);
     const longlong2 sl = load_flag_pair(&sk.flags->step);
     if (!(w.error == 0 && (sl.y < 0 || sl.x < sl.y))) continue;
-    double a = 0.0;   // this system's tiles, strided over the block in a fixed order
-    for (int t = threadIdx.x; t < sk.tile_count_s; t += blockDim.x)
-      a += ((const volatile double*)sk.nh_part)[sk.tile_first_s + t];
-    const double sum = block_sum_fixed(a);
+    const double sum = nh_total(sk.nh_part + sk.nh_first, sk.nh_count, slots);
     if (threadIdx.x == 0) {
-      const double K = 0.5 * sk.mass * sum;
-      const double G = (2.0 * K / (sk.gdof * sk.kT) - 1.0) / (sk.tau * sk.tau);
-      const double hdt = 0.5 * sk.dt;
       double xi = sk.nh[0], eta = sk.nh[1];
-      if (!w.v_full) {
-        eta += hdt * xi;
-        xi += hdt * G;
-      }
-      xi += hdt * G;
-      eta += hdt * xi;
+      sk.nh[2] = nh_update(sk, sum, w.v_full, xi, eta);
       sk.nh[0] = xi;
       sk.nh[1] = eta;
-      sk.nh[2] = exp(-hdt * xi);
     }
   }
   if (threadIdx.x == 0) ctl->blocks_done_a = 0;
