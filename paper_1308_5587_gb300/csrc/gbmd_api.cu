@@ -110,11 +110,12 @@ struct Group {
   Tile *d_tb = nullptr, *d_tbk = nullptr;   // staged force blocks; their window kernel
   Tile* d_te = nullptr;   // energy/virial launches: EV_TILE_P particles per tile, whatever
                           // the tuning, so the FP64 sums do not depend on it
-  Tile* d_tt = nullptr;   // tree-list systems: tiles over their trees' leaves
+  Tile *d_tt = nullptr, *d_tg = nullptr;   // tree-list systems: tiles over their trees'
+                                           // leaves, and over the groups that query them
   Tile* d_tn = nullptr;   // list build by four warps per cell (few cells): (cell, part) items
-  int ntp = 0, ntf = 0, ntc = 0, nts = 0, ntb = 0, ntbk = 0, nte = 0, ntt = 0, ntn = 0;
+  int ntp = 0, ntf = 0, ntc = 0, nts = 0, ntb = 0, ntbk = 0, nte = 0, ntt = 0, ntg = 0, ntn = 0;
   size_t cap_desc = 0, cap_tp = 0, cap_tf = 0, cap_tc = 0, cap_ts = 0, cap_part = 0;
-  size_t cap_tb = 0, cap_tbk = 0, cap_te = 0, cap_tt = 0, cap_tn = 0;
+  size_t cap_tb = 0, cap_tbk = 0, cap_te = 0, cap_tt = 0, cap_tg = 0, cap_tn = 0;
   bool any_cell = true;   // some member builds its list from cells
   int window_cap = 0;                        // largest staged window among members
   bool nvt = false;                          // the members integrate NVT (all or none)
@@ -184,7 +185,7 @@ void free_group(Group* g) {
     if (e) cudaEventDestroy(e);
   for (void* p : {(void*)g->d_desc, (void*)g->d_tp, (void*)g->d_tf, (void*)g->d_tc, (void*)g->d_te,
                   (void*)g->d_nhpart, (void*)g->d_ts, (void*)g->d_tb, (void*)g->d_tbk, (void*)g->d_tt,
-                  (void*)g->d_tn, (void*)g->d_team, (void*)g->d_partials, (void*)g->d_ctl})
+                  (void*)g->d_tg, (void*)g->d_tn, (void*)g->d_team, (void*)g->d_partials, (void*)g->d_ctl})
     cudaFree(p);
   delete g;
 }
@@ -215,6 +216,11 @@ bool use_split(const std::vector<gbmd_system*>& m) {
 }
 // blocks per cell: one for every 32 particles of the mean occupation
 int split_parts(const SysDev& d) { return std::max(1, (d.n / d.ncells + 31) / 32); }
+
+// the query groups of type ty of a tree-list system
+int tree_groups(const SysDev& d, int ty) {
+  return d.tree_single[ty] ? d.tree_n[ty] : (d.tree_n[ty] + TREE_G - 1) / TREE_G;
+}
 
 // Systems that the team kernel may step: the cell list on the global force path,
 // without ghosts (their rebuilds are the caller's).  Alone it pays while a step is short
@@ -267,7 +273,7 @@ int sync_layout(Group* g) {
     g->rest->layout_dirty = true;
   }
   std::vector<SysDev> desc;
-  std::vector<Tile> tp, tf, tc, ts, tb, tbk, te, tt, tn;
+  std::vector<Tile> tp, tf, tc, ts, tb, tbk, te, tt, tg, tn;
   const int per_f = g->fblock / g->tpp;
   g->multi = 0;
   g->rel = true;
@@ -306,6 +312,11 @@ int sync_layout(Group* g) {
     if (d.tree)
       for (int f = 0; f < d.tree_leaves_total; f += TILE_P)
         tt.push_back({(int)k, f, std::min(TILE_P, d.tree_leaves_total - f), 0});
+    for (int q = 0; d.tree && q < d.ntypes; ++q) {
+      const int ty = d.tree_qtype[q], groups = tree_groups(d, ty);
+      for (int f = 0; f < groups; f += TREE_WARPS)
+        tg.push_back({(int)k, f, std::min(TREE_WARPS, groups - f), ty | (d.tree_single[ty] ? 256 : 0)});
+    }
     desc.push_back(d);
     if (d.ntypes > 1) g->multi = std::max(g->multi, d.ntypes > 2 ? 2 : 1);
     if (!d.tree) {
@@ -330,6 +341,7 @@ int sync_layout(Group* g) {
   RET(grow(&g->d_tbk, &g->cap_tbk, tbk.size()));
   RET(grow(&g->d_te, &g->cap_te, te.size()));
   RET(grow(&g->d_tt, &g->cap_tt, tt.size()));
+  RET(grow(&g->d_tg, &g->cap_tg, tg.size()));
   RET(grow(&g->d_tn, &g->cap_tn, tn.size()));
   RET(grow(&g->d_team, &g->cap_team, g->team.size()));
   if (!g->d_ctl) {
@@ -349,6 +361,7 @@ int sync_layout(Group* g) {
   CK(up(g->d_tbk, tbk));
   CK(up(g->d_te, te));
   CK(up(g->d_tt, tt));
+  CK(up(g->d_tg, tg));
   CK(up(g->d_tn, tn));
   if (!g->team.empty())
     CK(cudaMemcpyAsync(g->d_team, g->team.data(), g->team.size() * sizeof(int), cudaMemcpyHostToDevice, g->stream));
@@ -361,6 +374,7 @@ int sync_layout(Group* g) {
   g->ntbk = (int)tbk.size();
   g->nte = (int)te.size();
   g->ntt = (int)tt.size();
+  g->ntg = (int)tg.size();
   g->ntn = (int)tn.size();
   g->layout_dirty = false;
   destroy_graphs(g);
@@ -393,7 +407,7 @@ std::vector<KernelCall> rebuild_calls(const Group* g) {
     v.push_back(nlist_call(g->d_desc, g->d_tc, g->ntc, g->d_ctl, g->rel, g->multi, g->ntbk > 0));
   if (g->ntt > 0) {
     v.push_back(tree_build_call(g->d_desc, g->d_tt, g->ntt, g->d_ctl));
-    v.push_back(tree_nlist_call(g->d_desc, g->d_tp, g->ntp, g->d_ctl));
+    v.push_back(tree_nlist_call(g->d_desc, g->d_tg, g->ntg, g->d_ctl));
   }
   return v;
 }
@@ -497,7 +511,7 @@ constexpr int COOP_MAX_N = 400000;
 int coop_rebuild(const Group* g, KernelCall* out) {
   out->func = nullptr;
   std::vector<gbmd_system*> m = live(g);
-  if (m.size() != 1 || m[0]->h.staged || m[0]->h.tree || m[0]->h.n > COOP_MAX_N) return GBMD_OK;
+  if (m.size() != 1 || m[0]->h.staged || m[0]->h.n > COOP_MAX_N) return GBMD_OK;
   TeamFit fit;
   RET(team_fit(rebuild_func(g->multi > 0), REBUILD_T, REBUILD_SMEM, g->device, &fit));
   if (fit.blocks_per_sm < 1) return GBMD_OK;
@@ -1190,13 +1204,15 @@ int create_impl(const gbmd_desc* d, gbmd_system** out, bool device) {
       ord[t] = t;
     }
     std::stable_sort(ord, ord + nt, [&](int a, int b) { return work[a] > work[b]; });
-    int qpos = 0;
+    const double vol = d->box[0] * d->box[1] * d->box[2];
     for (int k = 0; k < nt; ++k) {
       h.tree_qtype[k] = ord[k];
-      h.tree_qpos[k] = qpos;
-      qpos += (int)tcount[ord[k]];
+      // a group of 8 spans about two spacings of its type: where that is more than the
+      // type's reach, the group's box would mostly hold strangers
+      double reach = 0;
+      for (int u = 0; u < nt; ++u) reach = std::max(reach, cut_of(d, k * nt + u) + d->r_buff);
+      h.tree_single[k] = tcount[k] > 0 && 2.0 * std::cbrt(vol / (double)tcount[k]) > reach;
     }
-    h.tree_qpos[nt] = qpos;
   }
   h.nvt = d->integrator == GBMD_NVT;
   h.kT = d->kT;

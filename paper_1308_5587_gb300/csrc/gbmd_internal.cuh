@@ -133,9 +133,9 @@ struct SysDev {
                            // w = its index | type << CPOS_TYPE_SHIFT
   int4* tree_q;            // [N] the leaves' particles in leaf order: (x, y, z, index)
   // the list kernel visits the types in decreasing order of their expected query work
-  // (sum over t of n_t r_list(type, t)^3): launch positions tree_qpos[k] .. belong to
-  // type tree_qtype[k]
-  int tree_qpos[MAXT + 1], tree_qtype[MAXT];
+  // (sum over t of n_t r_list(type, t)^3); tree_single[t]: a query of type t is for one
+  // particle, else for a group of neighbours
+  int tree_qtype[MAXT], tree_single[MAXT];
   int n, ntypes, cap, precision;
   // domain decomposition: the last n_ghost tags are ghosts (not integrated; their
   // positions are set from outside every step); such a system leaves its rebuilds to

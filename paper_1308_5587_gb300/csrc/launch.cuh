@@ -46,10 +46,12 @@ KernelCall rebuild_call(const SysDev* d, int blocks, GroupCtl* ctl, bool multi);
 // the same rows built by four warps per cell (tiles over (cell, part) items)
 KernelCall nlist_split_call(const SysDev* d, const Tile* tiles_n, int ntiles, GroupCtl* ctl, bool multi);
 // tree neighbour list (k_tree.cu): the boxes of every type's tree (one thread per
-// leaf; tiles over the system's leaves), then the list (one thread per particle in
-// cell order; tiles over particles)
+// leaf; tiles over the system's leaves), then the list (one warp per group of particles;
+// tiles over groups)
+constexpr int TREE_WARPS = 8;   // groups a block
+constexpr int TREE_G = 8;       // particles of a group: TREE_G x 4 lanes
 KernelCall tree_build_call(const SysDev* d, const Tile* tiles_l, int ntiles, GroupCtl* ctl);
-KernelCall tree_nlist_call(const SysDev* d, const Tile* tiles_p, int ntiles, GroupCtl* ctl);
+KernelCall tree_nlist_call(const SysDev* d, const Tile* tiles_g, int ntiles, GroupCtl* ctl);
 // pair force kernels.  MODE_FORCE: forces at the current positions (readouts);
 // MODE_EV: also energy / virial / v.v partial sums (+ per-particle arrays when the
 // descriptor has them); MODE_STEP: the step kernel -- forces, the velocity Verlet

@@ -14,6 +14,7 @@
 #include "nlist_warp.cuh"
 #include "sort_core.cuh"
 #include "step_core.cuh"
+#include "tree_rows.cuh"
 
 namespace gbmd {
 
@@ -25,6 +26,7 @@ template <int T, int SLOTS>
 union TeamSmem {
   SplitCell split[T / NS_T];
   WarpRing<false, SLOTS> warp[T / 32];
+  struct { TreeWarp warp[T / 32]; TreeTable tab; } tree;
   int scan[32];
   double slots[NH_SLOTS];
 };
@@ -167,23 +169,48 @@ __device__ __noinline__ unsigned team_rebuild(const SysDev& s, Team& tm, TeamSme
   }
   unsigned long long nb = 0;
   int over = 0;
-  // Four warps a cell (nlist_split) while that keeps every group of four warps to one
-  // item; with more cells the team is busy anyway and a warp a cell needs fewer
-  // instructions (N = 20,011 on the whole grid, 729 cells: 37 us by four warps in two
-  // turns, 35 by one)
-  const int g = threadIdx.x / NS_T, groups = tm.size * (T / NS_T);
-  const int split = max(1, (n / s.ncells + 31) / 32);   // parts of a cell, 32 particles each
-  if ((long long)s.nbins * split <= groups) {
-    for (int k = tm.rank + g * tm.size; k < s.nbins * split; k += groups)
-      over = max(over, nlist_split<MULTI>(s, k / split, k % split, split, g, sm.split[g], tab, nb));
-  } else {
-    // cells of uneven cost: after its first, a warp takes the next free cell
-    int* const next = s.cell_cursor + s.nbins;   // set to 0 by the scan
-    for (int r = w0; r < s.nbins;) {
+  int* const next = s.cell_cursor + s.nbins;   // work counter, set to 0 by the scan
+  const int lane = threadIdx.x & 31;
+  if (s.tree) {
+    for (int g = t0; g < s.tree_leaves_total; g += nt) tree_leaf(s, qv, g);
+    if (tm.vote(0u) & VOTE_LOST) return VOTE_LOST;
+    tree_table(s, sm.tree.tab);
+    __syncthreads();
+    for (int k = w0;;) {   // query groups, the types with the longest queries first
       int q = 0;
-      if ((threadIdx.x & 31) == 0) q = nw + atomicAdd(next, 1);   // in flight during the build
-      over = max(over, nlist_cell<MULTI, false, false>(s, r, sm.warp[threadIdx.x >> 5], nb));
-      r = __shfl_sync(0xffffffffu, q, 0);
+      if (lane == 0) q = nw + atomicAdd(next, 1);   // in flight during the query
+      int at = k, o = 0, ty = 0, per = 1, groups = 0;
+      for (; o < s.ntypes; ++o, at -= groups) {
+        ty = s.tree_qtype[o];
+        per = s.tree_single[ty] ? 1 : TREE_G;
+        groups = (s.tree_n[ty] + per - 1) / per;
+        if (at < groups) break;
+      }
+      if (o == s.ntypes) break;
+      const int r = tree_rows(s, ty, at * per, min(per, s.tree_n[ty] - at * per), per,
+                              sm.tree.warp[threadIdx.x >> 5], sm.tree.tab, nb);
+      if (r < 0) atomicCAS(&s.flags->error, 0, (int)DEV_TREE);
+      over = max(over, r);
+      k = __shfl_sync(0xffffffffu, q, 0);
+    }
+  } else {
+    // Four warps a cell (nlist_split) while that keeps every group of four warps to one
+    // item; with more cells the team is busy anyway and a warp a cell needs fewer
+    // instructions (N = 20,011 on the whole grid, 729 cells: 37 us by four warps in two
+    // turns, 35 by one)
+    const int g = threadIdx.x / NS_T, groups = tm.size * (T / NS_T);
+    const int split = max(1, (n / s.ncells + 31) / 32);   // parts of a cell, 32 particles each
+    if ((long long)s.nbins * split <= groups) {
+      for (int k = tm.rank + g * tm.size; k < s.nbins * split; k += groups)
+        over = max(over, nlist_split<MULTI>(s, k / split, k % split, split, g, sm.split[g], tab, nb));
+    } else {
+      // cells of uneven cost: after its first, a warp takes the next free cell
+      for (int r = w0; r < s.nbins;) {
+        int q = 0;
+        if (lane == 0) q = nw + atomicAdd(next, 1);   // in flight during the build
+        over = max(over, nlist_cell<MULTI, false, false>(s, r, sm.warp[threadIdx.x >> 5], nb));
+        r = __shfl_sync(0xffffffffu, q, 0);
+      }
     }
   }
   if (over > 0) {

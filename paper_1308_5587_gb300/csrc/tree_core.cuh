@@ -73,6 +73,14 @@ GBMD_HD uint32_t tree_axis_gap(uint32_t u, uint32_t lo, uint32_t hi) {
   return up < down ? up : down;
 }
 
+// Periodic distance between the intervals [a, b] and [lo, hi] (none wraps): zero where
+// they overlap, else the shorter way round between their nearer ends
+GBMD_HD uint32_t tree_box_gap(uint32_t a, uint32_t b, uint32_t lo, uint32_t hi) {
+  if (lo - a <= b - a || a - lo <= hi - lo) return 0u;
+  const uint32_t up = lo - b, down = a - hi;
+  return up < down ? up : down;
+}
+
 // squared distance (FP32, in length units) from the point to the node box
 GBMD_HD float tree_gap2(const TreeBox& b, uint32_t ux, uint32_t uy, uint32_t uz, float fs0,
                         float fs1, float fs2) {
