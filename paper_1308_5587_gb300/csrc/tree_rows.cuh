@@ -63,7 +63,8 @@ __device__ __forceinline__ void tree_leaf(const SysDev& s, const int4* qv, int g
 // Popping only one level at a time keeps the leaves in ascending order, so a row holds
 // its neighbours in (type, cell order) order as the thread's walk did.  Each particle's
 // lanes then test the leaves' particles from a ring of 32.
-// WCA 1:10, N = 100,100: a build 1,405 us with a walk per thread, 587 this way (ncu).
+// WCA 1:10, N = 100,100: a build 1,405 us with a walk per thread, 243 this way (ncu; 587
+// before groups that span much of the box query one by one).
 constexpr int TREE_STACK = 1088;   // 32 entries a level stay (at most 30 levels), 64 on top
 
 struct TreeWarp {
@@ -87,11 +88,11 @@ __device__ __forceinline__ void tree_table(const SysDev& s, TreeTable& t) {
 }
 
 // The rows of members first .. first + count - 1 (count <= per) of type ty, per = TREE_G
-// or 1 particles a group.  Returns the longest row past the capacity (0: none; -1: the
+// or 1 particles at a time.  Returns the longest row past the capacity (0: none; -1: the
 // traversal ran past its bound).  Every lane of the warp calls it.
-__device__ __forceinline__ int tree_rows(const SysDev& s, int ty, int first, int count, int per,
-                                         TreeWarp& sm, const TreeTable& tab,
-                                         unsigned long long& nb) {
+__device__ __forceinline__ int tree_query_rows(const SysDev& s, int ty, int first, int count,
+                                               int per, TreeWarp& sm, const TreeTable& tab,
+                                               unsigned long long& nb) {
   const int lane = threadIdx.x & 31;
   // lanes of a particle: 32 / per; this lane's particle p and place c among its lanes
   const int lanes = 32 / per, shift = per == 1 ? 5 : 2;
@@ -215,7 +216,38 @@ __device__ __forceinline__ int tree_rows(const SysDev& s, int ty, int first, int
     nb += (unsigned long long)cnt;
     if (cnt > cap) over = cnt;
   }
-  return bad ? -1 : over;
+  return bad ? -1 : over;   // `bad` is the same in every lane
+}
+
+// The same for a group of up to TREE_G particles.  Where the sort order jumps, a group
+// can span much of the box, and its query would then visit every leaf in between (one
+// such warp outlives the rest of the build): its particles query one by one when the
+// space within reach of the group's box is more than TREE_SPREAD times one particle's.
+constexpr float TREE_SPREAD = 16.0f;
+__device__ __forceinline__ int tree_rows(const SysDev& s, int ty, int first, int count, int per,
+                                         TreeWarp& sm, const TreeTable& tab,
+                                         unsigned long long& nb) {
+  int step = count;
+  if (per > 1) {
+    const int lane = threadIdx.x & 31;
+    const int4 q = s.tree_q[s.tree_first[ty] + first + (lane < count ? lane : 0)];
+    auto extent = [](int v, float fs) {
+      const uint32_t u = tree_u(v);
+      return (float)(__reduce_max_sync(0xffffffffu, u) - __reduce_min_sync(0xffffffffu, u)) * fs;
+    };
+    const float ex = extent(q.x, s.fscale[0]), ey = extent(q.y, s.fscale[1]), ez = extent(q.z, s.fscale[2]);
+    float hi = 3e38f;
+    for (int t = 0; t < s.ntypes; ++t) hi = fminf(hi, tab.hi[ty * s.ntypes + t]);
+    const float d = 2.0f * sqrtf(hi);
+    if ((ex + d) * (ey + d) * (ez + d) > TREE_SPREAD * d * d * d) step = per = 1;
+  }
+  int over = 0;
+  for (int k = 0; k < count; k += step) {
+    const int r = tree_query_rows(s, ty, first + k, step, per, sm, tab, nb);
+    if (r < 0) return -1;
+    over = max(over, r);
+  }
+  return over;
 }
 
 }  // namespace gbmd
