@@ -90,7 +90,7 @@ struct gbmd_system {
   double *d_pos = nullptr, *d_vel = nullptr, *d_frc = nullptr;
   int *d_img = nullptr, *d_type = nullptr, *d_misc = nullptr;
   double *d_ppu = nullptr, *d_ppw = nullptr;   // per-particle readout staging (lazy)
-  double* d_thermo = nullptr;
+  std::vector<char> bounce;   // host side of a small readout
 };
 
 constexpr int TEAM_SIDES = 4;   // cluster sizes 16, 8, 4, 2, 1: the first on the group's stream
@@ -750,13 +750,31 @@ int write_flags(gbmd_system* s, const Flags* f, cudaStream_t st) {
   return GBMD_OK;
 }
 
+// the Snapshot that the last readout kernel left
+int read_snapshot(gbmd_system* s, Snapshot* o, cudaStream_t st) {
+  CK(cudaMemcpyAsync(o, s->h.thermo, sizeof(Snapshot), cudaMemcpyDeviceToHost, st));
+  CK(cudaStreamSynchronize(st));
+  return GBMD_OK;
+}
+
+// no error to recover from and no steps owed: what a readout enqueued behind the steps
+// has read is the state they end in
+bool settled(const gbmd_system* s, const Flags& f) {
+  const long long want = s->step_limit >= 0 ? std::min(s->target_step, s->step_limit) : s->target_step;
+  return f.error == 0 && f.step >= want;
+}
+
 cudaStream_t cur_stream(gbmd_system* s) { return s->own->stream; }
 
 // rebuild lists (when flags->do_rebuild) + forces, outside any graph, for the system alone
 int rebuild_and_force(gbmd_system* s, int ev) {
   Group* g = s->own;
   RET(sync_layout(g));
-  for (const KernelCall& c : rebuild_calls(g)) CK(launch(c, g->stream));
+  KernelCall coop;
+  coop.func = nullptr;
+  if (g->use_graphs) RET(coop_rebuild(g, &coop));
+  if (coop.func) CK(launch(coop, g->stream));
+  else for (const KernelCall& c : rebuild_calls(g)) CK(launch(c, g->stream));
   for (const KernelCall& c : force_calls(g, ev)) CK(launch(c, g->stream));
   return GBMD_OK;
 }
@@ -790,9 +808,8 @@ int grow_nlist(gbmd_system* s, int need) {
 int sync_system(gbmd_system* s) {
   cudaStream_t st = cur_stream(s);
   for (int round = 0; round < 64; ++round) {
-    CK(cudaStreamSynchronize(st));
     Flags f;
-    RET(read_flags(s, &f, st));
+    RET(read_flags(s, &f, st));   // waits for the stream
     if (f.error == DEV_NONFINITE)
       return fail(GBMD_ERR_NONFINITE, "non-finite coordinate or a particle moved more than L/2 in one step (step %lld)", f.step);
     if (f.error == DEV_WINDOW) {   // a staged window outgrew shared memory
@@ -1266,7 +1283,6 @@ int create_impl(const gbmd_desc* d, gbmd_system** out, bool device) {
   A((void**)&h.type_alt, N * 4); A((void**)&h.tag_alt, N * 4); A((void**)&h.q_alt, N * 16);
   A((void**)&h.fkey, N * 4);   // fine Morton keys: the order inside a cell
   A((void**)&h.cpos, N * 16);  // positions in cell order (the list build's candidates)
-  A((void**)&h.thermo, 16 * 8);
   A((void**)&h.nh, 4 * 8);
   if (tree) {
     A((void**)&h.tree_box, (size_t)nodes * sizeof(TreeBox));
@@ -1274,10 +1290,15 @@ int create_impl(const gbmd_desc* d, gbmd_system** out, bool device) {
     A((void**)&h.tree_q, N * 16);
   }
   A((void**)&s->d_flags, sizeof(Flags));
-  A((void**)&s->d_pos, N * 24); A((void**)&s->d_vel, N * 24); A((void**)&s->d_frc, N * 24);
-  A((void**)&s->d_img, N * 12); A((void**)&s->d_type, N * 4); A((void**)&s->d_misc, 64);
+  // import/export staging behind the snapshot: a small readout comes back in one copy
+  A((void**)&h.thermo, SNAPSHOT_BYTES + N * 84);
+  s->d_frc = h.thermo + SNAPSHOT_BYTES / 8;
+  s->d_vel = s->d_frc + 3 * N;
+  s->d_pos = s->d_vel + 3 * N;
+  s->d_img = (int*)(s->d_pos + 3 * N);
+  s->d_misc = h.thermo ? &((Snapshot*)h.thermo)->bad : nullptr;
+  A((void**)&s->d_type, N * 4);
   h.flags = s->d_flags;
-  s->d_thermo = h.thermo;
   if (rc != GBMD_OK) { gbmd_destroy(s); return rc; }
   cudaStream_t st = s->stream;
   rc = setup_cells(s, geo.nc, st);
@@ -1285,6 +1306,7 @@ int create_impl(const gbmd_desc* d, gbmd_system** out, bool device) {
   {
     const double nh0[4] = {0.0, 0.0, 1.0, 0.0};   // xi, eta, exp(-xi dt/2)
     cudaError_t e5 = cudaMemsetAsync(s->d_flags, 0, sizeof(Flags), st);
+    if (!e5) e5 = cudaMemsetAsync(h.thermo, 0, SNAPSHOT_BYTES, st);
     cudaError_t e6 = cudaMemsetAsync(h.nn, 0, N * 4, st);
     if (tree && e6 == cudaSuccess) e6 = cudaMemsetAsync(h.tree_arrive, 0, (size_t)nodes * 4, st);
     cudaError_t e7 = cudaMemcpyAsync(h.nh, nh0, sizeof(nh0), cudaMemcpyHostToDevice, st);
@@ -1314,9 +1336,10 @@ int create_impl(const gbmd_desc* d, gbmd_system** out, bool device) {
 }
 
 // Upload positions/velocities/types/images (tag order, host or device memory),
-// then build the lists (with the initial Morton sort) and compute the forces.
+// then build the lists (with the initial Morton sort) and compute the forces.  bad (on
+// the device): the state is refused when it is set, and nothing of the system changes.
 int load_state(gbmd_system* s, const double* pos, const double* vel, const int32_t* type,
-               const int32_t* image, bool device, long long step) {
+               const int32_t* image, bool device, long long step, const int* bad = nullptr) {
   cudaStream_t st = cur_stream(s);
   const size_t N = (size_t)s->h.n;
   const double *dp = pos, *dv = vel;
@@ -1337,28 +1360,16 @@ int load_state(gbmd_system* s, const double* pos, const double* vel, const int32
   }
   Group* g = s->own;
   RET(sync_layout(g));
-  CK(launch(import_call(g->d_desc, g->d_tp, g->ntp, dp, dv, dt, di), st));
-  Flags f{};
-  f.do_rebuild = 1;
-  f.do_sort = 1;
-  f.v_full = 1;
-  f.active = 1;
-  f.step = step;
-  f.step_limit = s->step_limit;
-  f.last_sort = step;
-  Flags old{};
-  CK(cudaMemcpyAsync(&old, s->d_flags, sizeof(Flags), cudaMemcpyDeviceToHost, st));
-  CK(cudaStreamSynchronize(st));
-  if (old.error == DEV_BADTYPE) return fail(GBMD_ERR_BAD_ARG, "type id out of range in the device type array");
-  f.n_rebuilds = old.n_rebuilds;
-  f.n_sorts = old.n_sorts + 1;
-  f.launches = old.launches;
-  RET(write_flags(s, &f, st));
-  s->target_step = step;
+  CK(launch(load_flags_call(g->d_desc, bad, step, s->step_limit), st));
+  CK(launch(import_call(g->d_desc, g->d_tp, g->ntp, dp, dv, dt, di, bad), st));
   RET(rebuild_and_force(s, 0));
-  CK(cudaStreamSynchronize(st));
-  Flags after;
-  RET(read_flags(s, &after, st));
+  CK(launch(snapshot_call(g->d_desc), st));
+  Snapshot snap;
+  RET(read_snapshot(s, &snap, st));
+  if (bad && snap.bad) return fail(GBMD_ERR_BAD_ARG, "non-finite state");
+  Flags after = snap.flags;
+  if (after.error == DEV_BADTYPE) return fail(GBMD_ERR_BAD_ARG, "type id out of range in the device type array");
+  s->target_step = step;
   if (after.error == DEV_WINDOW) {
     s->h.staged = 0;
     RET(refresh_desc(s));
@@ -1385,15 +1396,11 @@ int load_state(gbmd_system* s, const double* pos, const double* vel, const int32
 // stored xi / eta are those of the step's opening half; the closing half adds
 // dt/2 G(K) to xi and dt/2 xi to eta (nothing right after create / set_state).
 // h_ext = K + U (+ g kT (tau^2 xi^2 / 2 + eta) for NVT) is the conserved quantity.
-int fill_thermostat(gbmd_system* s, const Flags& f, gbmd_thermo* out) {
+void fill_thermostat(gbmd_system* s, const Flags& f, const double* nh, gbmd_thermo* out) {
   out->xi = 0.0;
   out->eta = 0.0;
   out->h_ext = out->ke + out->pe;
-  if (!s->h.nvt) return GBMD_OK;
-  double nh[2];
-  cudaStream_t st = cur_stream(s);
-  CK(cudaMemcpyAsync(nh, s->h.nh, sizeof(nh), cudaMemcpyDeviceToHost, st));
-  CK(cudaStreamSynchronize(st));
+  if (!s->h.nvt) return;
   const SysDev& h = s->h;
   double xi = nh[0], eta = nh[1];
   if (!f.v_full) {
@@ -1404,43 +1411,98 @@ int fill_thermostat(gbmd_system* s, const Flags& f, gbmd_thermo* out) {
   out->xi = xi;
   out->eta = eta;
   out->h_ext += h.gdof * h.kT * (0.5 * h.tau * h.tau * xi * xi + eta);
-  return GBMD_OK;
 }
 
-int thermo_impl(gbmd_system* s, double out[8]) {
+// the thermodynamic state from a snapshot whose sums are of the current positions
+void fill_thermo(gbmd_system* s, const Snapshot& snap, gbmd_thermo* out) {
+  const double* t = snap.thermo;
+  const double n = (double)s->h.n;
+  const double vol = s->h.L[0] * s->h.L[1] * s->h.L[2];
+  out->step = snap.flags.step;
+  out->pe = t[0];
+  out->ke = 0.5 * s->h.mass * t[1];
+  out->temperature = n > 1 ? 2.0 * out->ke / (3.0 * n - 3.0) : 0.0;
+  for (int c = 0; c < 6; ++c) out->virial[c] = t[2 + c];
+  out->w = t[2] + t[5] + t[7];
+  out->pressure = (n * out->temperature + out->w / 3.0) / vol;
+  out->n_rebuilds = snap.flags.n_rebuilds;
+  fill_thermostat(s, snap.flags, snap.nh, out);
+}
+
+// Readouts are enqueued behind the steps without waiting for them, with a snapshot of
+// the flags as their last kernel saw them; what they read counts once the snapshot says
+// that the steps ended well.  Otherwise the system is recovered and they run once more.
+// So a readout costs one round trip to the device (two where its arrays are too big for
+// one copy through `bounce`), not one for each thing it must know.
+constexpr size_t BOUNCE_MAX = 256 * 1024;
+
+int thermo_impl(gbmd_system* s, Snapshot* snap) {
   Group* g = s->own;
-  RET(sync_layout(g));
   cudaStream_t st = cur_stream(s);
-  for (const KernelCall& c : force_calls(g, 1)) CK(launch(c, st));
-  CK(launch(thermo_call(g->d_desc, g->d_ts, g->nts, g->d_ctl), st));
-  CK(cudaMemcpyAsync(out, s->d_thermo, 8 * sizeof(double), cudaMemcpyDeviceToHost, st));
-  CK(cudaStreamSynchronize(st));
-  return GBMD_OK;
+  for (int turn = 0; turn < 2; ++turn) {
+    RET(sync_layout(g));
+    for (const KernelCall& c : force_calls(g, 1)) CK(launch(c, st));
+    CK(launch(thermo_call(g->d_desc, g->d_ts, g->nts, g->d_ctl), st));
+    RET(read_snapshot(s, snap, st));
+    if (settled(s, snap->flags)) return GBMD_OK;
+    RET(sync_system(s));
+  }
+  return fail(GBMD_ERR_STATE, "the system does not settle");
 }
 
 int export_impl(gbmd_system* s, double* pos, double* vel, int32_t* image, double* force,
-                double* pp_u, double* pp_w) {
+                double* pp_u, double* pp_w, int64_t* step = nullptr) {
   Group* g = s->own;
-  RET(sync_layout(g));
   cudaStream_t st = cur_stream(s);
   const size_t N = (size_t)s->h.n;
   if ((pp_u || pp_w) && !s->d_ppw) return fail(GBMD_ERR_STATE, "per-particle arrays not allocated");
-  // forces and full-step velocities need F at the current positions: the step kernel
-  // does not store its force, so evaluate it here
-  if (vel || force)
-    for (const KernelCall& c : force_calls(g, 0)) CK(launch(c, st));
-  CK(launch(export_call(g->d_desc, g->d_tp, g->ntp, pos ? s->d_pos : nullptr,
-                        vel ? s->d_vel : nullptr, image ? s->d_img : nullptr,
-                        force ? s->d_frc : nullptr, pp_u ? s->d_ppu : nullptr,
-                        pp_w ? s->d_ppw : nullptr), st));
-  if (pos) CK(cudaMemcpyAsync(pos, s->d_pos, N * 24, cudaMemcpyDeviceToHost, st));
-  if (vel) CK(cudaMemcpyAsync(vel, s->d_vel, N * 24, cudaMemcpyDeviceToHost, st));
-  if (image) CK(cudaMemcpyAsync(image, s->d_img, N * 12, cudaMemcpyDeviceToHost, st));
-  if (force) CK(cudaMemcpyAsync(force, s->d_frc, N * 24, cudaMemcpyDeviceToHost, st));
-  if (pp_u) CK(cudaMemcpyAsync(pp_u, s->d_ppu, N * 8, cudaMemcpyDeviceToHost, st));
-  if (pp_w) CK(cudaMemcpyAsync(pp_w, s->d_ppw, N * 48, cudaMemcpyDeviceToHost, st));
-  CK(cudaStreamSynchronize(st));
-  return GBMD_OK;
+  for (int turn = 0; turn < 2; ++turn) {
+    RET(sync_layout(g));
+    // forces and full-step velocities need F at the current positions: the step kernel
+    // does not store its force, so evaluate it here (per-particle arrays: the energy pass)
+    if (pp_u || pp_w)
+      for (const KernelCall& c : force_calls(g, 1)) CK(launch(c, st));
+    else if (vel || force)
+      for (const KernelCall& c : force_calls(g, 0)) CK(launch(c, st));
+    CK(launch(export_call(g->d_desc, g->d_tp, g->ntp, pos ? s->d_pos : nullptr,
+                          vel ? s->d_vel : nullptr, image ? s->d_img : nullptr,
+                          force ? s->d_frc : nullptr, pp_u ? s->d_ppu : nullptr,
+                          pp_w ? s->d_ppw : nullptr), st));
+    // snapshot, force, velocity, position and image lie one after the other
+    const size_t bytes = SNAPSHOT_BYTES + N * (image ? 84 : pos ? 72 : vel ? 48 : force ? 24 : 0);
+    Snapshot snap;
+    const bool one = !pp_u && !pp_w && bytes <= BOUNCE_MAX;
+    if (one) {
+      s->bounce.resize(bytes);
+      CK(cudaMemcpyAsync(s->bounce.data(), s->h.thermo, bytes, cudaMemcpyDeviceToHost, st));
+      CK(cudaStreamSynchronize(st));
+      memcpy(&snap, s->bounce.data(), sizeof(snap));
+    } else {
+      RET(read_snapshot(s, &snap, st));
+    }
+    if (!settled(s, snap.flags)) {
+      RET(sync_system(s));
+      continue;
+    }
+    if (step) *step = snap.flags.step;
+    if (one) {
+      const char* b = s->bounce.data() + SNAPSHOT_BYTES;
+      if (force) memcpy(force, b, N * 24);
+      if (vel) memcpy(vel, b + N * 24, N * 24);
+      if (pos) memcpy(pos, b + N * 48, N * 24);
+      if (image) memcpy(image, b + N * 72, N * 12);
+      return GBMD_OK;
+    }
+    if (pos) CK(cudaMemcpyAsync(pos, s->d_pos, N * 24, cudaMemcpyDeviceToHost, st));
+    if (vel) CK(cudaMemcpyAsync(vel, s->d_vel, N * 24, cudaMemcpyDeviceToHost, st));
+    if (image) CK(cudaMemcpyAsync(image, s->d_img, N * 12, cudaMemcpyDeviceToHost, st));
+    if (force) CK(cudaMemcpyAsync(force, s->d_frc, N * 24, cudaMemcpyDeviceToHost, st));
+    if (pp_u) CK(cudaMemcpyAsync(pp_u, s->d_ppu, N * 8, cudaMemcpyDeviceToHost, st));
+    if (pp_w) CK(cudaMemcpyAsync(pp_w, s->d_ppw, N * 48, cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
+    return GBMD_OK;
+  }
+  return fail(GBMD_ERR_STATE, "the system does not settle");
 }
 
 int time_force(Group* g, float* ms) {
@@ -1731,7 +1793,6 @@ int gbmd_get_forces(gbmd_system* s, double* out) {
   Range nvtx_range("gbmd_get_forces");
   if (!s || !out) return fail(GBMD_ERR_BAD_ARG, "NULL argument");
   RET(use_device(s->device));
-  RET(sync_system(s));
   return export_impl(s, nullptr, nullptr, nullptr, out, nullptr, nullptr);
 }
 
@@ -1739,30 +1800,18 @@ int gbmd_get_thermo(gbmd_system* s, gbmd_thermo* out) {
   Range nvtx_range("gbmd_get_thermo");
   if (!s || !out) return fail(GBMD_ERR_BAD_ARG, "NULL argument");
   RET(use_device(s->device));
-  RET(sync_system(s));
-  double t[8];
-  RET(thermo_impl(s, t));
-  Flags f;
-  RET(read_flags(s, &f, cur_stream(s)));
-  const double n = (double)s->h.n;
-  const double vol = s->h.L[0] * s->h.L[1] * s->h.L[2];
-  out->step = f.step;
-  out->pe = t[0];
-  out->ke = 0.5 * s->h.mass * t[1];
-  out->temperature = n > 1 ? 2.0 * out->ke / (3.0 * n - 3.0) : 0.0;
-  for (int c = 0; c < 6; ++c) out->virial[c] = t[2 + c];
-  out->w = t[2] + t[5] + t[7];
-  out->pressure = (n * out->temperature + out->w / 3.0) / vol;
-  out->n_rebuilds = f.n_rebuilds;
-  return fill_thermostat(s, f, out);
+  Snapshot snap;
+  RET(thermo_impl(s, &snap));
+  fill_thermo(s, snap, out);
+  return GBMD_OK;
 }
 
 int gbmd_get_per_particle(gbmd_system* s, double* energy, double* virial) {
   Range nvtx_range("gbmd_get_per_particle");
   if (!s) return fail(GBMD_ERR_BAD_ARG, "system is NULL");
   RET(use_device(s->device));
-  RET(sync_system(s));
   if (!s->h.pp_u) {
+    RET(sync_system(s));
     const size_t N = (size_t)s->h.n;
     RET(dalloc(s, (void**)&s->h.pp_u, N * 8));
     RET(dalloc(s, (void**)&s->h.pp_w, N * 48));
@@ -1770,8 +1819,8 @@ int gbmd_get_per_particle(gbmd_system* s, double* energy, double* virial) {
     RET(dalloc(s, (void**)&s->d_ppw, N * 48));
     RET(refresh_desc(s));
   }
-  double t[8];
-  RET(thermo_impl(s, t));   // the energy pass fills the per-particle arrays
+  if (!energy && !virial) return sync_system(s);
+  // the energy pass fills the per-particle arrays
   return export_impl(s, nullptr, nullptr, nullptr, nullptr, energy, virial);
 }
 
@@ -1779,14 +1828,7 @@ int gbmd_get_state(gbmd_system* s, double* pos, double* vel, int32_t* image, int
   Range nvtx_range("gbmd_get_state");
   if (!s) return fail(GBMD_ERR_BAD_ARG, "system is NULL");
   RET(use_device(s->device));
-  RET(sync_system(s));
-  RET(export_impl(s, pos, vel, image, nullptr, nullptr, nullptr));
-  if (step) {
-    Flags f;
-    RET(read_flags(s, &f, cur_stream(s)));
-    *step = f.step;
-  }
-  return GBMD_OK;
+  return export_impl(s, pos, vel, image, nullptr, nullptr, nullptr, step);
 }
 
 int gbmd_set_state(gbmd_system* s, const double* pos, const double* vel, const int32_t* image,
@@ -1809,11 +1851,7 @@ int gbmd_set_state(gbmd_system* s, const double* pos, const double* vel, const i
   CK(cudaMemsetAsync(s->d_misc, 0, 4, st));
   CK(launch(prep_state_call(g->d_desc, g->d_tp, g->ntp, s->d_pos, s->d_vel, s->d_type, s->d_misc),
             st));
-  int bad = 0;
-  CK(cudaMemcpyAsync(&bad, s->d_misc, 4, cudaMemcpyDeviceToHost, st));
-  CK(cudaStreamSynchronize(st));
-  if (bad) return fail(GBMD_ERR_BAD_ARG, "non-finite state");
-  return load_state(s, s->d_pos, s->d_vel, s->d_type, image ? s->d_img : nullptr, true, step);
+  return load_state(s, s->d_pos, s->d_vel, s->d_type, image ? s->d_img : nullptr, true, step, s->d_misc);
 }
 
 int gbmd_get_neighbors(gbmd_system* s, int32_t* counts, int32_t* idx, int64_t cap) {
@@ -2244,18 +2282,8 @@ extern "C" int gbmd_get_thermo_noalloc(gbmd_system* s, gbmd_thermo* out) {
     CK(launch(force_staged_call(g->multi, MODE_EV, addr.desc, g->d_tb, g->ntb, g->d_ctl, 0,
                                 g->window_cap, StepArgs{}), st));
   CK(launch(thermo_call(addr.desc, g->d_ts, g->nts, g->d_ctl), st));
-  double t[8];
-  CK(cudaMemcpyAsync(t, s->d_thermo, sizeof(t), cudaMemcpyDeviceToHost, st));
-  CK(cudaStreamSynchronize(st));   // `d` and `t` are host stack memory
-  const double n = (double)s->h.n;
-  const double vol = s->h.L[0] * s->h.L[1] * s->h.L[2];
-  out->step = f.step;
-  out->pe = t[0];
-  out->ke = 0.5 * s->h.mass * t[1];
-  out->temperature = n > 1 ? 2.0 * out->ke / (3.0 * n - 3.0) : 0.0;
-  for (int c = 0; c < 6; ++c) out->virial[c] = t[2 + c];
-  out->w = t[2] + t[5] + t[7];
-  out->pressure = (n * out->temperature + out->w / 3.0) / vol;
-  out->n_rebuilds = f.n_rebuilds;
-  return fill_thermostat(s, f, out);
+  Snapshot snap;
+  RET(read_snapshot(s, &snap, st));   // waits: `d` is host stack memory
+  fill_thermo(s, snap, out);
+  return GBMD_OK;
 }

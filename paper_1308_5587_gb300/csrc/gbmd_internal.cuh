@@ -64,6 +64,17 @@ struct Flags {
 
 static_assert(sizeof(Flags) == 88 && offsetof(Flags, step) == 32, "Flags layout");
 
+// What a readout brings back in one copy, at SysDev::thermo: the sums, the thermostat
+// and the flags as the readout's last kernel found them, and `bad` of a new state
+struct Snapshot {
+  double thermo[8];   // pe, sum v.v, W (6)
+  double nh[4];
+  Flags flags;
+  int bad, pad[9];
+};
+static_assert(sizeof(Snapshot) == 224, "Snapshot layout");
+constexpr size_t SNAPSHOT_BYTES = 256;
+
 // Device reads of a system's flags, which other blocks and kernels of the step
 // write: volatile vector loads, so that the fields a kernel needs arrive in one
 // round trip instead of one dependent load each.  Flags sit at the start of their
@@ -187,7 +198,7 @@ struct SysDev {
   // thermo scratch: per-force-tile partial sums (pe, virial[6], pad) and output
   double *partials;
   int tile_first_f, tile_count_f;   // this system's tiles in the force tile table
-  double *thermo;                   // 16 doubles: pe, ke, virial[6], ...
+  double *thermo;                   // a Snapshot
   double *pp_u, *pp_w;              // optional per-particle energy / virial (N, N x 6)
   Flags *flags;
 };

@@ -33,6 +33,16 @@ __device__ double block_sum(double v, double* sh) {
   return r;
 }
 
+// one thread: the system's flags and thermostat into its Snapshot
+__device__ __forceinline__ void take_snapshot(const SysDev& s) {
+  Snapshot* o = reinterpret_cast<Snapshot*>(s.thermo);
+  const volatile long long* f = reinterpret_cast<const volatile long long*>(s.flags);
+  long long* to = reinterpret_cast<long long*>(&o->flags);
+  for (int k = 0; k < (int)(sizeof(Flags) / 8); ++k) to[k] = f[k];
+  for (int k = 0; k < 3; ++k) o->nh[k] = s.nh[k];
+}
+__global__ void k_snapshot(const SysDev* __restrict__ d) { take_snapshot(*d); }
+
 // U, sum v.v and W (6) of one system from the per-tile partial sums that the
 // energy variant of the force kernel wrote just before (fixed order: each thread
 // sums tiles t, t + 256, ... in order, then a fixed tree over the threads)
@@ -52,6 +62,25 @@ __global__ void __launch_bounds__(256) k_thermo(const SysDev* __restrict__ sysv,
     r = block_sum<double>(acc[c], sh);
     if (threadIdx.x == 0) s.thermo[c == 0 ? 0 : c + 1] = r;
   }
+  if (threadIdx.x == 0) take_snapshot(s);
+}
+
+// The flags of a newly loaded state (step and limit given), unless *bad: then only no
+// rebuild is due
+__global__ void k_load_flags(const SysDev* __restrict__ d, const int* bad, long long step,
+                             long long limit) {
+  Flags* f = d->flags;
+  if (bad && *bad) {
+    f->do_rebuild = f->do_sort = 0;
+    return;
+  }
+  f->rebuild_req = 0;
+  f->do_rebuild = f->do_sort = f->active = f->v_full = 1;
+  f->error = f->overflow_need = f->max_window = 0;
+  f->step = f->last_sort = step;
+  f->step_limit = limit;
+  f->n_sorts += 1;
+  f->nb_total = 0;
 }
 
 // ---------------------------------------------------------------------------
@@ -81,10 +110,11 @@ __global__ void __launch_bounds__(TILE_P) k_import(const SysDev* __restrict__ sy
                                                    const double* __restrict__ pos,
                                                    const double* __restrict__ vel,
                                                    const int* __restrict__ type,
-                                                   const int* __restrict__ image) {
+                                                   const int* __restrict__ image,
+                                                   const int* __restrict__ bad) {
   const Tile t = tiles[blockIdx.x];
   const SysDev& s = sysv[t.sys];
-  if (threadIdx.x >= t.count) return;
+  if (threadIdx.x >= t.count || (bad && *bad)) return;   // a refused state replaces nothing
   const int i = t.first + threadIdx.x, n = s.n;
   int q[3];
   for (int a = 0; a < 3; ++a) {
@@ -132,6 +162,7 @@ __global__ void __launch_bounds__(TILE_P) k_export(const SysDev* __restrict__ sy
                                                    double* pp_u, double* pp_w) {
   const Tile t = tiles[blockIdx.x];
   const SysDev& s = sysv[t.sys];
+  if (blockIdx.x == 0 && threadIdx.x == 0) take_snapshot(s);
   if (threadIdx.x >= t.count) return;
   const int tg = t.first + threadIdx.x, n = s.n;
   const int i = s.rtag[tg];
@@ -298,9 +329,21 @@ KernelCall thermo_call(const SysDev* d, const Tile* tiles_s, int nsys, GroupCtl*
 }
 
 KernelCall import_call(const SysDev* d, const Tile* tiles_p, int ntiles, const double* pos,
-                       const double* vel, const int* type, const int* image) {
+                       const double* vel, const int* type, const int* image, const int* bad) {
   KernelCall k = mk((void*)k_import, ntiles, TILE_P);
-  put(k, d); put(k, tiles_p); put(k, pos); put(k, vel); put(k, type); put(k, image);
+  put(k, d); put(k, tiles_p); put(k, pos); put(k, vel); put(k, type); put(k, image); put(k, bad);
+  return k;
+}
+
+KernelCall load_flags_call(const SysDev* d, const int* bad, long long step, long long limit) {
+  KernelCall k = mk((void*)k_load_flags, 1, 1);
+  put(k, d); put(k, bad); put(k, step); put(k, limit);
+  return k;
+}
+
+KernelCall snapshot_call(const SysDev* d) {
+  KernelCall k = mk((void*)k_snapshot, 1, 1);
+  put(k, d);
   return k;
 }
 

@@ -85,7 +85,11 @@ KernelCall thermo_call(const SysDev* d, const Tile* tiles_s, int nsys, GroupCtl*
 KernelCall prep_state_call(const SysDev* d, const Tile* tiles_p, int ntiles, const double* pos,
                            const double* vel, int* type_by_tag, int* bad);
 KernelCall import_call(const SysDev* d, const Tile* tiles_p, int ntiles, const double* pos,
-                       const double* vel, const int* type, const int* image);
+                       const double* vel, const int* type, const int* image, const int* bad);
+// the flags of a state being loaded into system *d, and the Snapshot of *d; with `bad`
+// (may be null) set the load changes nothing
+KernelCall load_flags_call(const SysDev* d, const int* bad, long long step, long long limit);
+KernelCall snapshot_call(const SysDev* d);
 KernelCall export_call(const SysDev* d, const Tile* tiles_p, int ntiles, double* pos,
                        double* vel, int* image, double* force, double* pp_u, double* pp_w);
 // domain decomposition (one system, d pointing at its descriptor): ghost positions
