@@ -108,8 +108,9 @@ struct Group {
   SysDev* d_desc = nullptr;
   Tile *d_tp = nullptr, *d_tf = nullptr, *d_tc = nullptr, *d_ts = nullptr;
   Tile *d_tb = nullptr, *d_tbk = nullptr;   // staged force blocks; their window kernel
-  Tile* d_te = nullptr;   // energy/virial launches: EV_TILE_P particles per tile, whatever
+  Tile* d_te = nullptr;   // energy/virial launches: ev_tile(n) particles per tile, whatever
                           // the tuning, so the FP64 sums do not depend on it
+  int ev_tile = EV_TILE_P;   // the largest of them
   Tile *d_tt = nullptr, *d_tg = nullptr;   // tree-list systems: tiles over their trees'
                                            // leaves, and over the groups that query them
   Tile* d_tn = nullptr;   // list build by four warps per cell (few cells): (cell, part) items
@@ -286,6 +287,7 @@ int sync_layout(Group* g) {
   for (size_t k = 0; k < m.size(); ++k) {
     SysDev d = m[k]->h;
     const int n = d.n;
+    g->ev_tile = std::max(k ? g->ev_tile : 0, ev_tile(n));
     for (int f = 0; f < n; f += TILE_P) tp.push_back({(int)k, f, std::min(TILE_P, n - f), 0});
     if (d.staged) {   // one force tile per 2x2x2 block of cells
       d.tile_first_f = (int)tb.size();   // shifted past the global tiles below
@@ -299,7 +301,7 @@ int sync_layout(Group* g) {
       d.nh_count = (int)(((long long)n * g->tpp + 31) / 32);
       nh_chunks += d.nh_count;
       d.tile_first_f = (int)te.size();   // partial sums come from the energy launches
-      for (int f = 0; f < n; f += EV_TILE_P) te.push_back({(int)k, f, std::min(EV_TILE_P, n - f), 0});
+      for (int f = 0; f < n; f += ev_tile(n)) te.push_back({(int)k, f, std::min(ev_tile(n), n - f), 0});
       d.tile_count_f = (int)te.size() - d.tile_first_f;
     }
     for (int c = 0; c < d.nbins; c += CELLS_PER_TILE)
@@ -419,9 +421,9 @@ KernelCall plain_force_call(const Group* g) {
 }
 
 // energy/virial launch of the global-list systems: the step's threads per particle
-// (so the FP32 forces it writes are bitwise the step's), EV_TILE_P particles per block
+// (so the FP32 forces it writes are bitwise the step's), ev_tile particles per block
 KernelCall ev_force_call(const Group* g, const SysDev* desc) {
-  return force_call(g->precision, g->multi, MODE_EV, g->tpp, EV_TILE_P * g->tpp, desc, g->d_te,
+  return force_call(g->precision, g->multi, MODE_EV, g->tpp, g->ev_tile * g->tpp, desc, g->d_te,
                     g->nte, g->d_ctl, StepArgs{}, g->eval);
 }
 

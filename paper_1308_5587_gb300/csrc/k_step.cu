@@ -19,20 +19,6 @@ namespace gbmd {
 // the kinetic term sum v^2 at full-step velocities, in a fixed order.
 // thermo[0] = pe, thermo[1] = sum v^2, thermo[2..7] = W.
 // ---------------------------------------------------------------------------
-template <typename T>
-__device__ double block_sum(double v, double* sh) {
-  // fixed-order tree reduction over the block (deterministic)
-  sh[threadIdx.x] = v;
-  __syncthreads();
-  for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-    if (threadIdx.x < w) sh[threadIdx.x] += sh[threadIdx.x + w];
-    __syncthreads();
-  }
-  double r = sh[0];
-  __syncthreads();
-  return r;
-}
-
 // one thread: the system's flags and thermostat into its Snapshot
 __device__ __forceinline__ void take_snapshot(const SysDev& s) {
   Snapshot* o = reinterpret_cast<Snapshot*>(s.thermo);
@@ -44,25 +30,32 @@ __device__ __forceinline__ void take_snapshot(const SysDev& s) {
 __global__ void k_snapshot(const SysDev* __restrict__ d) { take_snapshot(*d); }
 
 // U, sum v.v and W (6) of one system from the per-tile partial sums that the
-// energy variant of the force kernel wrote just before (fixed order: each thread
-// sums tiles t, t + 256, ... in order, then a fixed tree over the threads)
-__global__ void __launch_bounds__(256) k_thermo(const SysDev* __restrict__ sysv,
-                                                const Tile* __restrict__ tiles) {
-  __shared__ double sh[256];
+// energy variant of the force kernel wrote just before, in a fixed order: each thread
+// sums tiles t, t + THERMO_T, ... (four tiles in flight), then the warps by shuffles,
+// then the warps' sums in order
+constexpr int THERMO_T = 512;
+__global__ void __launch_bounds__(THERMO_T) k_thermo(const SysDev* __restrict__ sysv,
+                                                     const Tile* __restrict__ tiles) {
+  __shared__ double sh[THERMO_T / 32][8];
   const SysDev& s = sysv[tiles[blockIdx.x].sys];
   if (threadIdx.x == 0) atomicAdd(&s.flags->launches, 1ull);
   double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  for (int k = threadIdx.x; k < s.tile_count_f; k += blockDim.x) {
-    const double* p = s.partials + 8 * (size_t)(s.tile_first_f + k);
-    for (int c = 0; c < 8; ++c) acc[c] += p[c];
+  const double* p = s.partials + 8 * (size_t)s.tile_first_f;
+#pragma unroll 4
+  for (int k = threadIdx.x; k < s.tile_count_f; k += THERMO_T)
+    for (int c = 0; c < 8; ++c) acc[c] += p[8 * (size_t)k + c];
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    for (int o = 16; o > 0; o >>= 1) acc[c] += __shfl_down_sync(0xffffffffu, acc[c], o);
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5][c] = acc[c];
   }
-  double r = block_sum<double>(acc[7], sh);
-  if (threadIdx.x == 0) s.thermo[1] = r;
-  for (int c = 0; c < 7; ++c) {
-    r = block_sum<double>(acc[c], sh);
-    if (threadIdx.x == 0) s.thermo[c == 0 ? 0 : c + 1] = r;
+  __syncthreads();
+  if (threadIdx.x < 8) {
+    double r = 0;
+    for (int w = 0; w < THERMO_T / 32; ++w) r += sh[w][threadIdx.x];
+    s.thermo[threadIdx.x == 7 ? 1 : threadIdx.x == 0 ? 0 : threadIdx.x + 1] = r;
   }
-  if (threadIdx.x == 0) take_snapshot(s);
+  if (threadIdx.x == 32) take_snapshot(s);
 }
 
 // The flags of a newly loaded state (step and limit given), unless *bad: then only no
@@ -323,7 +316,7 @@ cudaError_t launch(const KernelCall& k, cudaStream_t st) {
 }
 
 KernelCall thermo_call(const SysDev* d, const Tile* tiles_s, int nsys, GroupCtl*) {
-  KernelCall k = mk((void*)k_thermo, nsys, 256);
+  KernelCall k = mk((void*)k_thermo, nsys, THERMO_T);
   put(k, d); put(k, tiles_s);
   return k;
 }

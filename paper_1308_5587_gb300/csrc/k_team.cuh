@@ -109,7 +109,8 @@ __global__ void __launch_bounds__(TEAM_T, 1) k_team(TeamArgs a) {
         const double4_32a* const pv = p64_at(s, step);
         const double4_32a pi = pv[i];
         double fx, fy, fz, e, wv[6];
-        gather_fp64<TPP, MT, EVAL, false, true>(s, pv, qv, pi, i, h, nn, tabf, tabd, fx, fy, fz, e, wv);
+        gather_fp64<TPP, MT, EVAL, false, true>(s, pv, qv, pi, i, h, nn, tabf, tabd,
+                                               sm.queue + threadIdx.x, T, fx, fy, fz, e, wv);
         fx = group_sum<TPP>(fx);
         fy = group_sum<TPP>(fy);
         fz = group_sum<TPP>(fz);

@@ -7,7 +7,12 @@
 namespace gbmd {
 
 constexpr int TILE_P = 256;     // particles per block of the streaming kernels
-constexpr int EV_TILE_P = 128;  // particles per FP64 energy/virial partial sum
+// particles per FP64 energy/virial partial sum (a block of the energy launches), by the
+// system's size alone, so the sums depend on no tuning.  Up to EV_SMALL_N particles a
+// block of 128 leaves SMs idle or unevenly loaded (FP64, N = 4,000: 32 blocks of 512
+// threads, 120 us; the whole readout 177 us with them, 68 with tiles of 32)
+constexpr int EV_TILE_P = 128, EV_TILE_SMALL = 32, EV_SMALL_N = 131072;
+inline int ev_tile(int n) { return n <= EV_SMALL_N ? EV_TILE_SMALL : EV_TILE_P; }
 constexpr int CELLS_PER_TILE = 8;   // warps (= cells) per block of the cell kernels
 constexpr int SCAN_THREADS = 1024;
 

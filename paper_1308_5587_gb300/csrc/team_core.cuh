@@ -29,6 +29,7 @@ union TeamSmem {
   struct { TreeWarp warp[T / 32]; TreeTable tab; } tree;
   int scan[32];
   double slots[NH_SLOTS];
+  int queue[16 * T];   // FP64 force phase (k_force.cuh)
 };
 
 struct Team {
