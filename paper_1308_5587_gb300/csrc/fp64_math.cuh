@@ -1,8 +1,96 @@
-// fp64_math.cuh -- the FP64 reciprocal of the pair force (1/r^2), shared by the
-// force evaluators and the arithmetic probe that prices it.
+// fp64_math.cuh -- the FP64 pair force's arithmetic that is kept off the FP64 pipe, and
+// its reciprocal.
 //
-// The FP64 pipe is the bound of the FP64 force path, and the correctly rounded
-// reciprocal costs ~5.6 FMA slots.  Here the hardware approximation
+// The FP64 pipe is the bound of the FP64 force path: it takes one warp instruction in
+// 16 cycles of an SM (1.99 of 128 lanes a clock, measured), the time of some 30 integer
+// instructions of each SM quarter.
+#pragma once
+
+namespace gbmd {
+
+// ---- displacements and r^2 on the integer pipe ----
+// A position is a 64-bit integer in units of 2^-fix_bits, chosen so that half the longest
+// box edge is at most 2^61 units: an FP64 coordinate is held to 2^-62 of that edge or
+// better, finer than its own last place for all but the smallest.  A displacement and
+// the sum of its squares are then exact integers, and each is rounded to FP64 once.  On
+// the FP64 pipe they are 6 of a pair's 17 instructions (three differences, r^2), each
+// rounded.  20 steps with readouts, LJ 64,000: 3,970 -> 2,831 us; the paper's workload
+// 4,182 -> 3,197.
+
+// an integer below 2^62 with its highest word `hi` != 0, shifted left until its leading
+// bit is bit 62 (`m`), as FP64: rounded to nearest at bit 10; `e` = (the biased exponent
+// that bit 62 stands for) - 1, for the leading bit adds one to it
+__device__ __forceinline__ double fix_pack(unsigned long long m, int e, unsigned sign) {
+  const unsigned long long b = (m + 0x200ull) >> 10;
+  return __hiloint2double((int)(((unsigned)(b >> 32) + ((unsigned)e << 20)) | sign), (int)(unsigned)b);
+}
+
+struct FixDiff {
+  unsigned long long m;   // |d|
+  unsigned sign;          // 0x80000000: d < 0
+  __device__ __forceinline__ unsigned hi() const { return (unsigned)(m >> 32); }
+  // the displacement through the other face: |d| -> L - |d|
+  __device__ __forceinline__ void other_way(long long L) {
+    m = (unsigned long long)L - m;
+    sign ^= 0x80000000u;
+  }
+  __device__ __forceinline__ double value(int fix_bits) const {
+    int sh;
+    if (hi() != 0u) {
+      sh = __clz(hi()) - 1;
+    } else {   // below 2^-29 of half the edge
+      if (m == 0ull) return 0.0;
+      sh = __clzll(m) - 1;
+    }
+    return fix_pack(m << sh, 1022 + 62 - fix_bits - sh, sign);
+  }
+};
+__device__ __forceinline__ FixDiff fix_diff(long long a, long long b) {
+  const long long d = a - b, s = d >> 63;
+  return FixDiff{(unsigned long long)((d ^ s) - s), (unsigned)(d >> 32) & 0x80000000u};
+}
+
+// |d|^2 below 2^96 units: all 128 bits of it
+static __device__ __noinline__ double fix_r2_close(unsigned long long x, unsigned long long y,
+                                                   unsigned long long z, int fix_bits) {
+  using u64 = unsigned long long;
+  const unsigned __int128 r = (unsigned __int128)x * x + (unsigned __int128)y * y + (unsigned __int128)z * z;
+  u64 s = (u64)(r >> 64);   // below 2^32
+  u64 t = (u64)r;
+  int e = 1022 + 126 - 2 * fix_bits;
+  if (s == 0ull) {
+    if (t == 0ull) return 0.0;
+    s = t;
+    t = 0ull;
+    e -= 64;
+  }
+  const int lead = __clzll(s);   // 0: one place too far left already
+  const u64 m = lead == 0 ? s >> 1 : lead == 1 ? s : s << (lead - 1) | t >> (65 - lead);
+  return fix_pack(m, e - (lead - 1), 0u);
+}
+
+// |d|^2 for components up to 2^61
+__device__ __forceinline__ double fix_r2(const FixDiff& x, const FixDiff& y, const FixDiff& z,
+                                         int fix_bits) {
+  using u64 = unsigned long long;
+  const unsigned xl = (unsigned)x.m, yl = (unsigned)y.m, zl = (unsigned)z.m;
+  const unsigned xh = x.hi(), yh = y.hi(), zh = z.hi();   // <= 2^29
+  const u64 high = (u64)xh * xh + (u64)yh * yh + (u64)zh * zh;      // x 2^64
+  const u64 mid = (u64)xh * xl + (u64)yh * yl + (u64)zh * zl;       // x 2^33; below 2^63
+  const u64 low = (u64)__umulhi(xl, xl) + __umulhi(yl, yl) + __umulhi(zl, zl);   // x 2^32
+  // r^2 = (s 2^32 + t) 2^32, short of it by less than 3 2^32 (the low halves of the low
+  // words' squares): 2^-62 of an r^2 of 2^96 and more
+  const u64 a = (mid << 1) + low;
+  const u64 s = high + (a >> 32);
+  const unsigned t = (unsigned)a;
+  // r below 2^-13 of half the longest edge
+  if ((unsigned)(s >> 32) == 0u) return fix_r2_close(x.m, y.m, z.m, fix_bits);
+  const int sh = __clz((unsigned)(s >> 32)) - 1;   // 1 .. 30
+  return fix_pack(s << sh | t >> (32 - sh), 1022 + 126 - 2 * fix_bits - sh, 0u);
+}
+
+// ---- reciprocal ----
+// The correctly rounded reciprocal costs ~5.6 FMA slots.  Here the hardware approximation
 // (rcp.approx.ftz.f64: relative error below 2^-19.9, measured over [0.25, 16)) is
 // refined by one third-order step of the geometric series of 1/(1 - e):
 //   a ~ 1/x,  e = 1 - x a,  1/x = a / (1 - e) = a (1 + e + e^2 + ...)  ->  a (1 + e + e^2)
@@ -11,10 +99,6 @@
 // differ by 1 ulp, none by more), for 3 FMAs plus the approximation (~3.3 slots).
 // x must be positive and normal (r^2 > 0); at x = 0 the result is not finite and
 // the step kernel's non-finite check reports it.
-#pragma once
-
-namespace gbmd {
-
 __device__ __forceinline__ double rcp_f64(double x) {
   double a;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(a) : "d"(x));

@@ -1241,10 +1241,19 @@ int create_impl(const gbmd_desc* d, gbmd_system** out, bool device) {
   h.window_cap = STAGED_WINDOW_CAP;
   for (int a = 0; a < 3; ++a) {
     h.L[a] = d->box[a];
-    h.halfL[a] = 0.5 * d->box[a];
     h.qscale[a] = 4294967296.0 / d->box[a];
     h.dtq[a] = d->dt * h.qscale[a];
     h.fscale[a] = (float)(d->box[a] / 4294967296.0);
+  }
+  // units of the FP64 gather's positions: half the longest edge is at most 2^61 of them
+  int fix_e;
+  const double half_max = 0.5 * std::max({d->box[0], d->box[1], d->box[2]});
+  if (std::frexp(half_max, &fix_e) == 0.5) --fix_e;
+  h.fix_bits = 61 - fix_e;   // half_max <= 2^fix_e
+  for (int a = 0; a < 3; ++a) {
+    h.fix_q[a] = std::ldexp(d->box[a], h.fix_bits - 32);
+    h.fix_L[a] = std::llrint(std::ldexp(d->box[a], h.fix_bits));
+    h.fix_half[a] = (unsigned)((unsigned long long)h.fix_L[a] >> 33);
   }
   const double hb = 0.5 * d->r_buff;
   h.rbuff_half2 = (float)(hb * hb * (1.0 - 1e-5));

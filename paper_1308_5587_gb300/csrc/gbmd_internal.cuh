@@ -14,7 +14,8 @@
 //   q           int4 [N]: x as 32-bit fixed point of x/L (2^32 <-> L, two's
 //               complement, so an int32 difference is the minimum image) + type in w
 //   q_build     int4 [N]: q at the last neighbour-list build (displacement check)
-//   p64         double4_32a [N]: FP64 x, y, z + type bits in w (FP64 force gather only)
+//   p64         longlong4_32a [N]: x, y, z as 62-bit fixed point in units of 2^-fix_bits,
+//               type in w (FP64 force gather only; fp64_math.cuh)
 //   f32 / f64   float4 / double4_32a [N]: force (+ per-particle energy in w when asked)
 //   nn, nl      int32 [N] neighbour counts; ELL4 list: entry k of particle i at
 //               nl[((k / 4) * nl_stride + i) * 4 + k % 4], nl_stride = N rounded up
@@ -120,7 +121,13 @@ inline int eval_of(int potential) {
 
 struct SysDev {
   // geometry
-  double L[3], halfL[3];
+  double L[3];
+  // FP64 gather: positions in units of 2^-fix_bits, at most 2^61 of them to half the
+  // longest edge; per axis the factor from L / 2^32 units, L, and the high word of L / 2
+  int fix_bits;
+  unsigned fix_half[3];
+  double fix_q[3];
+  long long fix_L[3];
   double qscale[3];        // 2^32 / L
   float fscale[3];         // L / 2^32
   float rbuff_half2;       // (r_buff / 2)^2, slightly reduced (conservative)
@@ -184,7 +191,7 @@ struct SysDev {
   // odd steps): the step kernel gathers from one and writes the next step's to the
   // other.  p64 only in FP64 mode.
   int4 *q, *q1, *q_build;
-  double4_32a *p64, *p64b;
+  longlong4_32a *p64, *p64b;
   float4 *f32;
   double4_32a *f64;
   int *nn, *nl;
@@ -228,12 +235,20 @@ __device__ __forceinline__ long long step_of(const Flags* f) {
 __device__ __forceinline__ int4* q_at(const SysDev& s, long long step) {
   return (step & 1) ? s.q1 : s.q;
 }
-__device__ __forceinline__ double4_32a* p64_at(const SysDev& s, long long step) {
+__device__ __forceinline__ longlong4_32a* p64_at(const SysDev& s, long long step) {
   return (step & 1) ? s.p64b : s.p64;
 }
 
 __device__ __forceinline__ void count_launch(const SysDev& s) {
   if (threadIdx.x == 0 && blockIdx.x == 0) atomicAdd(&s.flags->launches, 1ull);
+}
+
+// the FP64 gather's copy of a position given in units of L / 2^32 (fix_q scales by a
+// power of two times L / 2^32, so the product is the position's FP64 value in real units)
+__device__ __forceinline__ longlong4_32a fix_position(const SysDev& s, double xq, double yq,
+                                                      double zq, int type) {
+  return make_longlong4_32a(__double2ll_rn(xq * s.fix_q[0]), __double2ll_rn(yq * s.fix_q[1]),
+                            __double2ll_rn(zq * s.fix_q[2]), type);
 }
 
 // 32-bit fixed point of x/L with wrap-around; x in any image

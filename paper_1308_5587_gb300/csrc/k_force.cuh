@@ -29,8 +29,9 @@
 // displacement exactly; it is converted to FP32 and scaled by L/2^32.  The pair
 // arithmetic runs two neighbours at a time (LJ in packed FP32x2 operations); the
 // per-particle sums are FP32.
-// FP64: positions come from the double4 shadow p64; the minimum image is one
-// conditional correction by L (|d| < L for wrapped coordinates); all arithmetic FP64.
+// FP64: positions come from the 62-bit fixed-point copy p64; the displacement, its
+// minimum image (one conditional correction by L) and r^2 are exact integer arithmetic,
+// rounded once to FP64 (fp64_math.cuh); everything after is FP64.
 #pragma once
 #include "launch.cuh"
 #include "step_core.cuh"
@@ -295,12 +296,12 @@ __device__ __forceinline__ void gather_mixed(const SysDev& s, const int4* qv, co
 // test's branch, 162 from the queue.
 constexpr int FP64_QUEUE = 16;   // entries a lane (a power of two)
 template <int TPP, int MT, int EVAL, bool EV, bool COH>
-__device__ __forceinline__ void gather_fp64(const SysDev& s, const double4_32a* pv, const int4* qv,
-                                            const double4_32a& pi, int i, int h, int n,
+__device__ __forceinline__ void gather_fp64(const SysDev& s, const longlong4_32a* pv, const int4* qv,
+                                            const longlong4_32a& pi, int i, int h, int n,
                                             const PairF* tabf, const PairD* tabd, int* queue,
                                             int qstride, double& fx, double& fy, double& fz,
                                             double& e, double* w) {
-  const int nt = s.ntypes, ti = (int)__double_as_longlong(pi.w);
+  const int nt = s.ntypes, ti = (int)pi.w;
   const int groups = (n + 3) >> 2;
   const int4* nl4 = reinterpret_cast<const int4*>(s.nl) + i;
   const size_t stride = (size_t)s.nl_stride;
@@ -308,9 +309,8 @@ __device__ __forceinline__ void gather_fp64(const SysDev& s, const double4_32a* 
   const int4 qi = qv[i];
   const float fs0 = s.fscale[0], fs1 = s.fscale[1], fs2 = s.fscale[2];
   const float cut0 = s.pf[0].rc2 * FP64_PRETEST_MARGIN;
-  const double L0 = s.L[0], L1 = s.L[1], L2 = s.L[2];
-  const int h0 = __double2hiint(s.halfL[0]), h1 = __double2hiint(s.halfL[1]),
-            h2 = __double2hiint(s.halfL[2]);
+  const int fb = s.fix_bits;
+  const unsigned h0 = s.fix_half[0], h1 = s.fix_half[1], h2 = s.fix_half[2];
   const PairD p0 = s.pd[0];
   fx = fy = fz = e = 0.0;
   for (int c = 0; c < 6; ++c) w[c] = 0.0;
@@ -342,7 +342,7 @@ __device__ __forceinline__ void gather_fp64(const SysDev& s, const double4_32a* 
       gg += TPP;
     }
     // up to four of them in FP64
-    double4_32a pp[4];
+    longlong4_32a pp[4];
     const int m = min(tail - head, 4);
 #pragma unroll
     for (int u = 0; u < 4; ++u)
@@ -351,23 +351,21 @@ __device__ __forceinline__ void gather_fp64(const SysDev& s, const double4_32a* 
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
       if (u >= m) continue;
-      const double4_32a pj = pp[u];
-      double dx = pi.x - pj.x, dy = pi.y - pj.y, dz = pi.z - pj.z;
+      const longlong4_32a pj = pp[u];
+      FixDiff x = fix_diff(pi.x, pj.x), y = fix_diff(pi.y, pj.y), z = fix_diff(pi.z, pj.z);
       // minimum image: |d| < L; the test on the high words is exact except within
-      // 2^-20 of L/2, where either choice leaves |d| ~ L/2 > r_cut.  Only pairs
-      // across a box face need it, so a warp takes the correction (FP64 adds on
-      // every lane once the compiler turns it into selects) only when one of its
+      // 2^-28 of L/2, where either choice leaves |d| ~ L/2 > r_cut.  Only pairs
+      // across a box face need it, so a warp takes the correction only when one of its
       // pairs does
-      const bool wx = (__double2hiint(dx) & 0x7fffffff) > h0;
-      const bool wy = (__double2hiint(dy) & 0x7fffffff) > h1;
-      const bool wz = (__double2hiint(dz) & 0x7fffffff) > h2;
+      const bool wx = x.hi() > h0, wy = y.hi() > h1, wz = z.hi() > h2;
       if (__any_sync(__activemask(), wx || wy || wz)) {
-        if (wx) dx -= copysign(L0, dx);
-        if (wy) dy -= copysign(L1, dy);
-        if (wz) dz -= copysign(L2, dz);
+        if (wx) x.other_way(s.fix_L[0]);
+        if (wy) y.other_way(s.fix_L[1]);
+        if (wz) z.other_way(s.fix_L[2]);
       }
-      const double r2 = fma(dx, dx, fma(dy, dy, dz * dz));
-      const PairD P = MT ? tabd[ti * nt + (int)__double_as_longlong(pj.w)] : p0;
+      const double r2 = fix_r2(x, y, z, fb);
+      const double dx = x.value(fb), dy = y.value(fb), dz = z.value(fb);
+      const PairD P = MT ? tabd[ti * nt + (int)pj.w] : p0;
       // both positive, so the bit patterns order like the values
       if (__double_as_longlong(r2) < __double_as_longlong(P.rc2)) {
         double v;
@@ -472,9 +470,9 @@ __device__ __forceinline__ void force_body(const SysDev* __restrict__ sysv,
       reduce_partials<TPP>(vals, s.partials + 8 * (size_t)blockIdx.x);
     }
   } else {
-    const double4_32a* __restrict__ pv = p64_at(s, step);
-    const double4_32a pi = pv[i];
-    const int ti = (int)__double_as_longlong(pi.w);
+    const longlong4_32a* __restrict__ pv = p64_at(s, step);
+    const longlong4_32a pi = pv[i];
+    const int ti = (int)pi.w;
     double fx, fy, fz, e, w[6];
     extern __shared__ int fp64_queue[];   // FP64_QUEUE ints a thread
     gather_fp64<TPP, MT, EVAL, EV, false>(s, pv, q_at(s, step), pi, i, h, n, tabf, tabd,

@@ -139,8 +139,7 @@ __global__ void __launch_bounds__(TILE_P) k_import(const SysDev* __restrict__ sy
   s.q1[i] = qn;
   s.q_build[i] = qn;
   if (s.precision == GBMD_FP64) {   // the FP64 gather copies exist in FP64 mode only
-    const double4_32a pn = make_double4_32a(s.x[i] * (s.L[0] / 4294967296.0), s.x[n + i] * (s.L[1] / 4294967296.0),
-                                            s.x[2 * n + i] * (s.L[2] / 4294967296.0), __longlong_as_double(ty));
+    const longlong4_32a pn = fix_position(s, s.x[i], s.x[n + i], s.x[2 * n + i], ty);
     s.p64[i] = pn;
     s.p64b[i] = pn;
   }
@@ -266,12 +265,12 @@ __global__ void __launch_bounds__(TILE_P) k_ghost_set(const SysDev* __restrict__
     if (qq >= 0x80000000LL) { xq -= 4294967296.0; qq -= 0x100000000LL; }
     s.x[a * n + i] = xq;
     q[a] = (int)qq;
-    xr[a] = xq * (L / 4294967296.0);
+    xr[a] = xq;
   }
   const int ty = s.type[i];
   q_at(s, step)[i] = make_int4(q[0], q[1], q[2], ty);
   if (s.precision == GBMD_FP64)
-    p64_at(s, step)[i] = make_double4_32a(xr[0], xr[1], xr[2], __longlong_as_double(ty));
+    p64_at(s, step)[i] = fix_position(s, xr[0], xr[1], xr[2], ty);
 }
 
 // out[k] = the wrapped position of the particle with tag tags[k] (NaN for a tag out

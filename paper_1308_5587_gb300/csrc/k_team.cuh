@@ -106,8 +106,8 @@ __global__ void __launch_bounds__(TEAM_T, 1) k_team(TeamArgs a) {
           }
         }
       } else {
-        const double4_32a* const pv = p64_at(s, step);
-        const double4_32a pi = pv[i];
+        const longlong4_32a* const pv = p64_at(s, step);
+        const longlong4_32a pi = pv[i];
         double fx, fy, fz, e, wv[6];
         gather_fp64<TPP, MT, EVAL, false, true>(s, pv, qv, pi, i, h, nn, tabf, tabd,
                                                sm.queue + threadIdx.x, T, fx, fy, fz, e, wv);
@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(TEAM_T, 1) k_team(TeamArgs a) {
           } else {
             bool moved = false;
             bad |= !isfinite(fx) || !isfinite(fy) || !isfinite(fz);
-            integrate_one<PREC>(s, i, (int)__double_as_longlong(pi.w), f, vfull,
+            integrate_one<PREC>(s, i, (int)pi.w, f, vfull,
                                 load_particle<true>(s, i), qn, p64_at(s, step + 1), moved, bad);
             need |= moved;
           }

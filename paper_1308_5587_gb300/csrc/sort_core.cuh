@@ -118,13 +118,13 @@ __device__ __forceinline__ void permute_one(const SysDev& s, const int4* qv, int
 
 __device__ __forceinline__ void copyback_one(const SysDev& s, long long step, int k) {
   const int n = s.n;
-  double xr[3];
+  double xr[3];   // in units of L / 2^32
   for (int a = 0; a < 3; ++a) {
     const double xq = s.x_alt[a * n + k];
     s.x[a * n + k] = xq;
     s.v[a * n + k] = s.v_alt[a * n + k];
     s.img[a * n + k] = s.img_alt[a * n + k];
-    xr[a] = xq * (s.L[a] * (1.0 / 4294967296.0));
+    xr[a] = xq;
   }
   const int ty = s.type_alt[k];
   s.type[k] = ty;
@@ -136,7 +136,7 @@ __device__ __forceinline__ void copyback_one(const SysDev& s, long long step, in
   s.rmember[k] = k;
   s.cpos[k] = with_index(s.q_alt[k], k);
   if (s.precision == GBMD_FP64)
-    p64_at(s, step)[k] = make_double4_32a(xr[0], xr[1], xr[2], __longlong_as_double(ty));
+    p64_at(s, step)[k] = fix_position(s, xr[0], xr[1], xr[2], ty);
 }
 
 }  // namespace gbmd

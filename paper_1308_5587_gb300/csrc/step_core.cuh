@@ -77,7 +77,7 @@ template <int PREC>
 __device__ __forceinline__ void integrate_one(const SysDev& s, int i, int ty, const double f[3],
                                               int vfull, const ParticleState& p0,
                                               int4* __restrict__ q_next,
-                                              double4_32a* __restrict__ p64_next, bool& need,
+                                              longlong4_32a* __restrict__ p64_next, bool& need,
                                               bool& bad) {
   const int n = s.n;
   if (s.n_ghost > 0 && __ldg(s.tag + i) >= n - s.n_ghost) {
@@ -88,10 +88,7 @@ __device__ __forceinline__ void integrate_one(const SysDev& s, int i, int ty, co
                               (int)rint_ll(p0.xq[2]), ty);
     q_next[i] = qg;
     if (PREC == GBMD_FP64)
-      p64_next[i] = make_double4_32a(p0.xq[0] * (s.L[0] * (1.0 / 4294967296.0)),
-                                     p0.xq[1] * (s.L[1] * (1.0 / 4294967296.0)),
-                                     p0.xq[2] * (s.L[2] * (1.0 / 4294967296.0)),
-                                     __longlong_as_double(ty));
+      p64_next[i] = fix_position(s, p0.xq[0], p0.xq[1], p0.xq[2], ty);
     return;
   }
   const double kick = vfull ? s.h : s.h + s.h;
@@ -118,10 +115,7 @@ __device__ __forceinline__ void integrate_one(const SysDev& s, int i, int ty, co
   }
   q_next[i] = make_int4(q[0], q[1], q[2], ty);
   if (PREC == GBMD_FP64)
-    p64_next[i] = make_double4_32a(xq[0] * (s.L[0] * (1.0 / 4294967296.0)),
-                                   xq[1] * (s.L[1] * (1.0 / 4294967296.0)),
-                                   xq[2] * (s.L[2] * (1.0 / 4294967296.0)),
-                                   __longlong_as_double(ty));
+    p64_next[i] = fix_position(s, xq[0], xq[1], xq[2], ty);
   const float dx = (float)min_image_fixed(q[0], p0.qb.x) * s.fscale[0];
   const float dy = (float)min_image_fixed(q[1], p0.qb.y) * s.fscale[1];
   const float dz = (float)min_image_fixed(q[2], p0.qb.z) * s.fscale[2];
