@@ -143,27 +143,27 @@ __device__ __forceinline__ void eval_f32x2(const float2 r2, const PairF& Pa, con
 // one, and the fixed-point shadow within 2^-32 L of the FP64 position.
 constexpr float FP64_PRETEST_MARGIN = 1.0f + 1e-5f;
 
-// FP64, one neighbour
+// FP64, one neighbour at r^2 = q
 template <int EVAL, bool EV>
-__device__ __forceinline__ double eval_f64(double r2, const PairD& P, double& v) {
+__device__ __forceinline__ double eval_f64(const FixR2& q, const PairD& P, double& v) {
   if constexpr (EVAL == EVAL_LJ) {
-    const double r2i = rcp_f64(r2);
-    const double r6i = r2i * r2i * r2i;
+    double r6i, r8i;
+    fix_inv68(q, r6i, r8i);
     if (EV) v = fma(r6i, fma(P.p3, r6i, -P.p4), -P.shift);
-    return r2i * r6i * fma(P.p0, r6i, -P.p1);
+    return r8i * fma(P.p0, r6i, -P.p1);
   } else if constexpr (EVAL == EVAL_MIE) {
-    const double r2i = rcp_f64(r2);
+    const double r2i = fix_inv2(q);
     const double x = P.p0 * r2i;   // (sigma / r)^2
     const double tn = pow(x, P.p1), tm = pow(x, P.p2);
     if (EV) v = P.p3 * (tn - tm) - P.shift;
     return 2.0 * P.p3 * (P.p1 * tn - P.p2 * tm) * r2i;
   } else if constexpr (EVAL == EVAL_YUKAWA) {
-    const double r = sqrt(r2);
+    const double r2 = q.value(), r = sqrt(r2);
     const double e = P.p0 * exp(-P.p1 * r) / r;
     if (EV) v = e - P.shift;
     return e * (1.0 + P.p1 * r) / r2;
   } else {   // EVAL_GAUSS
-    const double e = exp(-P.p1 * r2);
+    const double e = exp(-P.p1 * q.value());
     if (EV) v = P.p0 * e - P.shift;
     return P.p2 * e;
   }
@@ -363,11 +363,11 @@ __device__ __forceinline__ void gather_fp64(const SysDev& s, const longlong4_32a
         if (wy) y.other_way(s.fix_L[1]);
         if (wz) z.other_way(s.fix_L[2]);
       }
-      const double r2 = fix_r2(x, y, z, fb);
+      const FixR2 r2 = fix_r2(x, y, z, fb);
       const double dx = x.value(fb), dy = y.value(fb), dz = z.value(fb);
       const PairD P = MT ? tabd[ti * nt + (int)pj.w] : p0;
       // both positive, so the bit patterns order like the values
-      if (__double_as_longlong(r2) < __double_as_longlong(P.rc2)) {
+      if (__double_as_longlong(r2.value()) < __double_as_longlong(P.rc2)) {
         double v;
         const double f = eval_f64<EVAL, EV>(r2, P, v);
         fx = fma(f, dx, fx);

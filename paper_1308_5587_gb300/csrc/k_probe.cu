@@ -6,8 +6,8 @@
 // the pipe, not latency, sets the rate:
 //   PROBE_DFMA: x <- fma(x, a, b) in FP64          (one FP64 multiply-add)
 //   PROBE_FFMA: x <- fmaf(x, a, b) in FP32         (one FP32 multiply-add)
-//   PROBE_DRCP: x <- rcp_f64(x) in FP64            (the reciprocal the FP64 pair
-//                                                   force takes once per pair)
+//   PROBE_DRCP: x <- rcp_f64(x) in FP64            (a reciprocal on that pipe: what
+//                                                   the pair force would pay there)
 // The grid is the SM count times 8 blocks of 256 threads.  Each thread stores the
 // sum of its chains, so the compiler cannot drop them.
 #include "launch.cuh"
