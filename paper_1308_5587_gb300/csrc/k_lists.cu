@@ -174,7 +174,8 @@ __global__ void __launch_bounds__(CELLS_PER_TILE * 32) k_cellsort(const SysDev* 
   count(s, t, ctl);
   const int w = threadIdx.x >> 5;
   if (!block_rebuilding(s) || w >= t.count) return;
-  cellsort_one(s, q_at(s, step_of(s.flags)), t.first + w);
+  const int b = s.cell_start[t.first + w];
+  cellsort_one(s, q_at(s, step_of(s.flags)), s.members_tmp + b, b, s.cell_start[t.first + w + 1] - b);
 }
 
 // ---- re-sort: gather every per-particle array into cell order ----

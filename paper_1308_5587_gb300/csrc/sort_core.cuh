@@ -23,7 +23,8 @@ __device__ __forceinline__ unsigned fine_morton(const int4& q) {
 }
 
 // ---- binning + histogram ----
-__device__ __forceinline__ void bin_one(const SysDev& s, const int4* qv, int i) {
+// the particle's sort bin, kept with its Morton code
+__device__ __forceinline__ int bin_of(const SysDev& s, const int4* qv, int i) {
   const int4 q = qv[i];
   const int cx = cell_of_fixed(q.x, s.nc[0]);
   const int cy = cell_of_fixed(q.y, s.nc[1]);
@@ -33,10 +34,30 @@ __device__ __forceinline__ void bin_one(const SysDev& s, const int4* qv, int i) 
   const int r = s.lin2rank[(cz * s.nc[1] + cy) * s.nc[0] + cx] + (s.tree ? q.w * s.ncells : 0);
   s.key[i] = r;
   s.fkey[i] = fine_morton(q);
+  return r;
+}
+__device__ __forceinline__ void bin_one(const SysDev& s, const int4* qv, int i) {
+  const int r = bin_of(s, qv, i);
   // consecutive particles mostly share a bin: one atomic per distinct bin of the warp
   const unsigned am = __activemask();
   const unsigned peers = __match_any_sync(am, r);
   if ((int)(threadIdx.x & 31) == __ffs(peers) - 1) atomicAdd(&s.cell_cnt[r], __popc(peers));
+}
+
+// The same, and the particle into the bin's bucket of `cap` entries at the place the
+// histogram's atomic gives it; false: the bucket is full.
+__device__ __forceinline__ bool bin_bucket(const SysDev& s, const int4* qv, int i, int* bucket,
+                                           int cap) {
+  const int r = bin_of(s, qv, i);
+  const int lane = threadIdx.x & 31;
+  const unsigned am = __activemask();
+  const unsigned peers = __match_any_sync(am, r);
+  const int leader = __ffs(peers) - 1;
+  int at = 0;
+  if (lane == leader) at = atomicAdd(&s.cell_cnt[r], __popc(peers));
+  at = __shfl_sync(am, at, leader) + __popc(peers & ((1u << lane) - 1u));
+  if (at < cap) bucket[(size_t)r * cap + at] = i;
+  return at < cap;
 }
 
 // ---- scatter particle indices into their cells (unordered within a cell) ----
@@ -62,9 +83,10 @@ __device__ __forceinline__ int4 with_index(const int4& q, int j) {
 // ---- sort one bin's members (one warp) -> a deterministic order ----
 // By (fine Morton code, index), so that consecutive members of a bin are spatial
 // neighbours (the tree list's leaves; the force kernel's warps).
-__device__ __forceinline__ void cellsort_one(const SysDev& s, const int4* qv, int r) {
+// The bin's n members, in any order at `src`, get the ranks b ..
+__device__ __forceinline__ void cellsort_one(const SysDev& s, const int4* qv, const int* src, int b,
+                                             int n) {
   const int lane = threadIdx.x & 31;
-  const int b = s.cell_start[r], e = s.cell_start[r + 1], n = e - b;
   // the sort key of member m: (fine code, index)
   auto key = [&](int v) -> unsigned long long {
     return ((unsigned long long)s.fkey[v] << 32) | (unsigned)v;
@@ -73,7 +95,7 @@ __device__ __forceinline__ void cellsort_one(const SysDev& s, const int4* qv, in
   // a cell's candidates contiguously, however far the particles have drifted from
   // the order of the last re-sort
   if (n <= 32) {
-    const int v = lane < n ? s.members_tmp[b + lane] : 0x7fffffff;
+    const int v = lane < n ? src[lane] : 0x7fffffff;
     const unsigned long long kv = lane < n ? key(v) : ~0ull;
     int rk = 0;
     for (int k = 0; k < 32; ++k) rk += __shfl_sync(0xffffffffu, kv, k) < kv;
@@ -85,12 +107,12 @@ __device__ __forceinline__ void cellsort_one(const SysDev& s, const int4* qv, in
   } else {   // 32 members against 32 at a time, every key read once per block of 32
     for (int m0 = 0; m0 < n; m0 += 32) {
       const int m = m0 + lane;
-      const int v = m < n ? s.members_tmp[b + m] : 0x7fffffff;
+      const int v = m < n ? src[m] : 0x7fffffff;
       const unsigned long long kv = m < n ? key(v) : ~0ull;
       int rk = 0;
       for (int k0 = 0; k0 < n; k0 += 32) {
         const unsigned long long ko =
-            k0 == m0 ? kv : k0 + lane < n ? key(s.members_tmp[b + k0 + lane]) : ~0ull;
+            k0 == m0 ? kv : k0 + lane < n ? key(src[k0 + lane]) : ~0ull;
         for (int k = 0; k < 32; ++k) rk += __shfl_sync(0xffffffffu, ko, k) < kv;
       }
       if (m < n) {

@@ -21,13 +21,23 @@ namespace gbmd {
 constexpr int TEAM_SPIN = 1 << 22;   // polls of ~0.5 us: two seconds
 enum : unsigned { VOTE_NEED = 1u, VOTE_BAD = 2u, VOTE_LOST = 4u };
 
+// The team's cell sort takes buckets: the histogram's atomic places each particle in its
+// bin's bucket, every block scans the counts for itself, and each bin is sorted out of
+// its bucket into its final place: one barrier where count, scan and scatter take three.
+// For up to SCAN_MAX bins with a mean of at most two thirds of a bucket; a bucket that
+// runs over sends the rebuild to the separate phases.  The buckets lie in the re-sort's
+// scratch.  With the even spread of the cells over the blocks (below), 50 steps with
+// readouts: N = 64,000 1,872 -> 1,789 us; one list build of N = 20,011 with its
+// readouts 464 -> 443.
+constexpr int SCAN_MAX = 12288, BUCKET = 64;
+
 // shared memory of the phases (one at a time; dynamic: more than 48 KB)
 template <int T, int SLOTS>
 union TeamSmem {
   SplitCell split[T / NS_T];
   WarpRing<false, SLOTS> warp[T / 32];
   struct { TreeWarp warp[T / 32]; TreeTable tab; } tree;
-  int scan[32];
+  struct { int start[SCAN_MAX + 1], warp[32]; } scan;
   double slots[NH_SLOTS];
   int queue[16 * T];   // FP64 force phase (k_force.cuh)
 };
@@ -145,6 +155,35 @@ __device__ __forceinline__ void scan_bins(const SysDev& s, int* sh) {
   }
 }
 
+// The same by every block for itself, into shared memory: start[0 .. nbins]
+template <int T>
+__device__ __forceinline__ void scan_own(const SysDev& s, int* start, int* sh) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int nc = s.nbins;
+  for (int c = threadIdx.x; c < nc; c += T) start[c] = __ldcg(s.cell_cnt + c);
+  __syncthreads();
+  const int per = ((nc + T - 1) / T) | 1;   // consecutive bins of a thread (odd: no bank twice)
+  const int c0 = min(nc, (int)threadIdx.x * per), c1 = min(nc, c0 + per);
+  int sum = 0;
+  for (int c = c0; c < c1; ++c) sum += start[c];
+  int x = sum;
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, x, o);
+    if (lane >= o) x += y;
+  }
+  if (lane == 31) sh[w] = x;
+  __syncthreads();
+  int e = x - sum;
+  for (int k = 0; k < w; ++k) e += sh[k];
+  for (int c = c0; c < c1; ++c) {
+    const int m = start[c];
+    start[c] = e;
+    e += m;
+  }
+  if (threadIdx.x == 0) start[nc] = s.n;
+  __syncthreads();
+}
+
 // The list rebuild (and re-sort) of the team's system at the positions of `step`;
 // returns the last vote (BAD: a row passed the capacity, the flags say so).
 template <int T, bool MULTI, int SLOTS>
@@ -152,16 +191,47 @@ __device__ __noinline__ unsigned team_rebuild(const SysDev& s, Team& tm, TeamSme
                                               SplitTable& tab, long long step, bool sort) {
   const int n = s.n;
   const int t0 = tm.rank * T + threadIdx.x, nt = tm.size * T;
-  const int w0 = tm.rank * (T / 32) + (threadIdx.x >> 5), nw = tm.size * (T / 32);
+  const int w = threadIdx.x >> 5, nw = tm.size * (T / 32);
   const int4* qv = q_at(s, step);
-  for (int i = t0; i < n; i += nt) bin_one(s, qv, i);
+  // this block's bins
+  const int r0 = (int)((long long)s.nbins * tm.rank / tm.size);
+  const int r1 = (int)((long long)s.nbins * (tm.rank + 1) / tm.size);
+  int* const bucket = reinterpret_cast<int*>(s.x_alt);   // 6 n entries
+  const int bcap = (int)min((long long)BUCKET, 6ll * n / s.nbins);
+  bool full = s.nbins > SCAN_MAX || bcap < 16 || 3ll * n > 2ll * bcap * s.nbins;
+  if (full) {
+    for (int i = t0; i < n; i += nt) bin_one(s, qv, i);
+  } else {
+    for (int i = t0; i < n; i += nt) full |= !bin_bucket(s, qv, i, bucket, bcap);
+  }
+  const unsigned v = tm.vote(full ? VOTE_NEED : 0u);
+  if (v & VOTE_LOST) return VOTE_LOST;
+  const bool direct = !(v & VOTE_NEED);
+  if (direct) {
+    scan_own<T>(s, sm.scan.start, sm.scan.warp);
+    const int* const start = sm.scan.start;
+    for (int r = r0 + (int)threadIdx.x; r < r1; r += T) s.cell_start[r] = start[r];
+    if (tm.rank == 0 && threadIdx.x == 0) {
+      s.cell_start[s.nbins] = n;
+      s.cell_cursor[s.nbins] = 0;   // the list build's work counter
+      s.flags->nb_total = 0;
+      s.flags->max_window = 0;
+    }
+    for (int r = r0 + w; r < r1; r += T / 32)
+      cellsort_one(s, qv, bucket + (size_t)r * bcap, start[r], start[r + 1] - start[r]);
+  } else {
+    if (tm.rank == 0) scan_bins<T>(s, sm.scan.warp);
+    if (tm.vote(0u) & VOTE_LOST) return VOTE_LOST;
+    for (int i = t0; i < n; i += nt) scatter_one(s, i);
+    if (tm.vote(0u) & VOTE_LOST) return VOTE_LOST;
+    for (int r = r0 + w; r < r1; r += T / 32) {
+      const int b = s.cell_start[r];
+      cellsort_one(s, qv, s.members_tmp + b, b, s.cell_start[r + 1] - b);
+    }
+  }
   if (tm.vote(0u) & VOTE_LOST) return VOTE_LOST;
-  if (tm.rank == 0) scan_bins<T>(s, sm.scan);
-  if (tm.vote(0u) & VOTE_LOST) return VOTE_LOST;
-  for (int i = t0; i < n; i += nt) scatter_one(s, i);
-  if (tm.vote(0u) & VOTE_LOST) return VOTE_LOST;
-  for (int r = w0; r < s.nbins; r += nw) cellsort_one(s, qv, r);
-  if (tm.vote(0u) & VOTE_LOST) return VOTE_LOST;
+  if (direct)   // every block has scanned the counts: empty for the next build
+    for (int r = r0 + (int)threadIdx.x; r < r1; r += T) s.cell_cnt[r] = 0;
   if (sort) {
     for (int k = t0; k < n; k += nt) permute_one(s, qv, k);
     if (tm.vote(0u) & VOTE_LOST) return VOTE_LOST;
@@ -177,7 +247,8 @@ __device__ __noinline__ unsigned team_rebuild(const SysDev& s, Team& tm, TeamSme
     if (tm.vote(0u) & VOTE_LOST) return VOTE_LOST;
     tree_table(s, sm.tree.tab);
     __syncthreads();
-    for (int k = w0;;) {   // query groups, the types with the longest queries first
+    // query groups, the types with the longest queries first and spread over the blocks
+    for (int k = w * tm.size + tm.rank;;) {
       int q = 0;
       if (lane == 0) q = nw + atomicAdd(next, 1);   // in flight during the query
       int at = k, o = 0, ty = 0, per = 1, groups = 0;
@@ -204,9 +275,14 @@ __device__ __noinline__ unsigned team_rebuild(const SysDev& s, Team& tm, TeamSme
     if ((long long)s.nbins * split <= groups) {
       for (int k = tm.rank + g * tm.size; k < s.nbins * split; k += groups)
         over = max(over, nlist_split<MULTI>(s, k / split, k % split, split, g, sm.split[g], tab, nb));
+    } else if (s.nbins <= nw) {
+      // a cell to a warp: every block gets its share of them (before, 729 cells of N =
+      // 20,011 kept 46 of 152 blocks busy, 2,744 of N = 64,000 115)
+      const int r = r0 + w;
+      if (r < r1) over = nlist_cell<MULTI, false, false>(s, r, sm.warp[w], nb);
     } else {
       // cells of uneven cost: after its first, a warp takes the next free cell
-      for (int r = w0; r < s.nbins;) {
+      for (int r = tm.rank * (T / 32) + w; r < s.nbins;) {
         int q = 0;
         if (lane == 0) q = nw + atomicAdd(next, 1);   // in flight during the build
         over = max(over, nlist_cell<MULTI, false, false>(s, r, sm.warp[threadIdx.x >> 5], nb));

@@ -42,6 +42,15 @@ def fluid(n, **kw):
     return lambda: wl.lj_fluid(n, rho, 1.2, seed=300 + n, **kw)
 
 
+def clump(n_side=12):
+    """Soft particles crowded at the centre: some cells hold many times the mean."""
+    u = (np.arange(n_side) - 0.5 * (n_side - 1)) / (0.5 * n_side)
+    pos = np.stack(np.meshgrid(u, u, u, indexing="ij"), -1).reshape(-1, 3)
+    pos = 9.0 * pos * np.abs(pos)
+    return wl.Workload(pos, -0.3 * pos, np.zeros(len(pos), np.int32), np.full(3, 18.0),
+                       wl.gauss_single(), r_buff=0.4)
+
+
 # name: (workload, precision, create options).  Sizes at the edges of the rules: a cluster
 # of one block, of 16, the whole grid, the largest team, the cooperative rebuild alone;
 # two cells an axis (raw fixed point), four warps a cell and one; every pair-table mode.
@@ -64,6 +73,9 @@ CASES = {
     "gauss_700_fp64": (fluid(700, pairs=wl.gauss_single()), "fp64", {}),
     "n49152_team": (fluid(49152), "mixed", {"sort_period": 30}),
     "n49153_coop_rebuild": (fluid(49153), "mixed", {"sort_period": 30}),
+    "clump_1728_buckets_run_over": (clump, "mixed", {"sort_period": 3}),
+    "dilute_1500_no_buckets": (lambda: wl.lj_fluid(1500, 0.02, 1.2, seed=38), "mixed",
+                               {"sort_period": 2}),
     "n33001_fp64_one_lane": (fluid(33001), "fp64", {}),
     "tree_3000": (lambda: wl.colloid_mixture(3000, ratio=5.0, seed=34), "mixed",
                   {"nlist": "tree", "sort_period": 10}),
