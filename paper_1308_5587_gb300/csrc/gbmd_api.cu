@@ -236,6 +236,26 @@ bool team_member(const Group* g, const SysDev& d) {
   return !d.tree && !d.staged && d.n_ghost == 0 && d.n <= (g->is_batch ? TEAM_CLUSTER_N : TEAM_ALONE_N);
 }
 
+// The force tiles of a system, `per` particles each.  The particles of a wide type of a
+// tree-list system (its order is type-major) come first, in wide tiles: one to each 32
+// threads of a block of per * tpp.
+void force_tiles(const SysDev& d, int sys, int prec, int tpp, int per, std::vector<Tile>* out) {
+  auto add = [&](int first, int count, int p, int wide) {
+    for (int f = 0; f < count; f += p) out->push_back({sys, first + f, std::min(p, count - f), wide});
+  };
+  const bool wide = d.tree && !d.nvt && has_wide(prec, tpp);
+  if (!wide) return add(0, d.n, per, 0);
+  for (int t = 0; t < d.ntypes; ++t)
+    if (d.tree_wide[t]) add(d.tree_first[t], d.tree_n[t], std::max(1, per * tpp / 32), 1);
+  for (int t = 0; t < d.ntypes;) {   // the others, across type boundaries
+    if (d.tree_wide[t]) { ++t; continue; }
+    const int first = d.tree_first[t];
+    int count = 0;
+    for (; t < d.ntypes && !d.tree_wide[t]; ++t) count += d.tree_n[t];
+    add(first, count, per, 0);
+  }
+}
+
 // Rebuild descriptor copies and tile tables for the group's current members.
 int sync_layout(Group* g) {
   if (!g->layout_dirty) return GBMD_OK;
@@ -296,12 +316,12 @@ int sync_layout(Group* g) {
       for (int b = 0; b < d.nblocks; b += 8) tbk.push_back({(int)k, b, std::min(8, d.nblocks - b), 0});
       g->window_cap = std::max(g->window_cap, d.window_cap);
     } else {
-      for (int f = 0; f < n; f += per_f) tf.push_back({(int)k, f, std::min(per_f, n - f), 0});
+      force_tiles(d, (int)k, g->precision, g->tpp, per_f, &tf);
       d.nh_first = nh_chunks;
       d.nh_count = (int)(((long long)n * g->tpp + 31) / 32);
       nh_chunks += d.nh_count;
       d.tile_first_f = (int)te.size();   // partial sums come from the energy launches
-      for (int f = 0; f < n; f += ev_tile(n)) te.push_back({(int)k, f, std::min(ev_tile(n), n - f), 0});
+      force_tiles(d, (int)k, g->precision, g->tpp, ev_tile(n), &te);
       d.tile_count_f = (int)te.size() - d.tile_first_f;
     }
     for (int c = 0; c < d.nbins; c += CELLS_PER_TILE)
@@ -1231,6 +1251,8 @@ int create_impl(const gbmd_desc* d, gbmd_system** out, bool device) {
       double reach = 0;
       for (int u = 0; u < nt; ++u) reach = std::max(reach, cut_of(d, k * nt + u) + d->r_buff);
       h.tree_single[k] = tcount[k] > 0 && 2.0 * std::cbrt(vol / (double)tcount[k]) > reach;
+      // few particles with long rows: their lanes' chains would outlive the rest
+      h.tree_wide[k] = work[k] * 4.0 / 3.0 * M_PI / vol >= 64.0 && 32 * tcount[k] <= n;
     }
   }
   h.nvt = d->integrator == GBMD_NVT;

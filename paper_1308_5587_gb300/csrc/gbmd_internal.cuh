@@ -154,6 +154,7 @@ struct SysDev {
   // (sum over t of n_t r_list(type, t)^3); tree_single[t]: a query of type t is for one
   // particle, else for a group of neighbours
   int tree_qtype[MAXT], tree_single[MAXT];
+  int tree_wide[MAXT];   // a type's particles take wide force tiles (a warp each)
   int n, ntypes, cap, precision;
   // domain decomposition: the last n_ghost tags are ghosts (not integrated; their
   // positions are set from outside every step); such a system leaves its rebuilds to

@@ -56,8 +56,8 @@ __device__ __forceinline__ T group_sum(T v) {
 // (fixed order)
 constexpr int NPART = 8;   // energy, virial xx xy xz yy yz zz, sum of v^2
 template <int TPP>
-__device__ void reduce_partials(const double* vals, double* out) {
-  __shared__ double sh[NPART][EV_TILE_P];
+__device__ __forceinline__ void reduce_partials(const double* vals, double (*sh)[EV_TILE_P],
+                                                double* out) {
   const int g = threadIdx.x / TPP, l = threadIdx.x % TPP;
   const int ng = blockDim.x / TPP;
   if (l == 0)
@@ -394,12 +394,11 @@ __device__ __forceinline__ void gather_fp64(const SysDev& s, const longlong4_32a
 // the end-of-step decisions by the last of `total_blocks` blocks.  A system that is
 // frozen (device error) or at its step limit is skipped in step mode.
 template <int PREC, int TPP, int MT, int MODE, int EVAL>
-__device__ __forceinline__ void force_body(const SysDev* __restrict__ sysv,
-                                           const Tile* __restrict__ tiles, GroupCtl* ctl,
+__device__ __forceinline__ void force_body(const SysDev* __restrict__ sysv, const Tile& t,
+                                           double (*part)[EV_TILE_P], GroupCtl* ctl,
                                            int nsys, int total_blocks,
                                            cudaGraphConditionalHandle cond, int use_cond) {
   constexpr bool EV = MODE == MODE_EV, STEP = MODE == MODE_STEP, NVTA = MODE == MODE_NVT_A;
-  const Tile t = tiles[blockIdx.x];
   const SysDev& s = sysv[t.sys];
   if (threadIdx.x == 0 && t.first == 0) atomicAdd(&s.flags->launches, 1ull);
   if (threadIdx.x == 0 && blockIdx.x == 0) atomicAdd(&ctl->launches, 1ull);
@@ -467,7 +466,7 @@ __device__ __forceinline__ void force_body(const SysDev* __restrict__ sysv,
         s.pp_u[i] = vals[0];
         for (int c = 0; c < 6; ++c) s.pp_w[6 * (size_t)i + c] = vals[c + 1];
       }
-      reduce_partials<TPP>(vals, s.partials + 8 * (size_t)blockIdx.x);
+      reduce_partials<TPP>(vals, part, s.partials + 8 * (size_t)blockIdx.x);
     }
   } else {
     const longlong4_32a* __restrict__ pv = p64_at(s, step);
@@ -508,7 +507,7 @@ __device__ __forceinline__ void force_body(const SysDev* __restrict__ sysv,
         s.pp_u[i] = vals[0];
         for (int c = 0; c < 6; ++c) s.pp_w[6 * (size_t)i + c] = vals[c + 1];
       }
-      reduce_partials<TPP>(vals, s.partials + 8 * (size_t)blockIdx.x);
+      reduce_partials<TPP>(vals, part, s.partials + 8 * (size_t)blockIdx.x);
     }
   }
   }   // active
@@ -522,12 +521,23 @@ __device__ __forceinline__ void force_body(const SysDev* __restrict__ sysv,
 }
 
 
+// A wide tile (Tile::pad) gives each of its particles a whole warp: the few particles of
+// a size-disperse mixture with many neighbours (sync_layout has the rule).  WCA 1:10,
+// N = 100,100: the 100 large ones, ~160 neighbours each in a row of 40 slot groups one
+// after another, outlived the other blocks (SMs active 41% of a step kernel); 40 steps with readouts
+// 3,018 us with every particle on TPP lanes, 1,901 with wide tiles.
 template <int PREC, int TPP, int MT, int MODE, int EVAL>
 __global__ void __launch_bounds__(512) k_force(const SysDev* __restrict__ sysv,
                                                const Tile* __restrict__ tiles, GroupCtl* ctl,
                                                int nsys, int total_blocks,
                                                cudaGraphConditionalHandle cond, int use_cond) {
-  force_body<PREC, TPP, MT, MODE, EVAL>(sysv, tiles, ctl, nsys, total_blocks, cond, use_cond);
+  __shared__ double part[MODE == MODE_EV ? NPART : 1][EV_TILE_P];
+  const Tile t = tiles[blockIdx.x];
+  constexpr bool wide = has_wide(PREC, TPP) && MODE != MODE_NVT_A;
+  if (wide && t.pad)
+    force_body<PREC, 32, MT, MODE, EVAL>(sysv, t, part, ctl, nsys, total_blocks, cond, use_cond);
+  else
+    force_body<PREC, TPP, MT, MODE, EVAL>(sysv, t, part, ctl, nsys, total_blocks, cond, use_cond);
 }
 
 // The mixed-precision step kernel with one lane per particle (the large systems)
@@ -540,8 +550,8 @@ template <int MT, int EVAL>
 __global__ void __maxnreg__(STEP1_MAXREG)
     k_force_step1(const SysDev* __restrict__ sysv, const Tile* __restrict__ tiles, GroupCtl* ctl,
                   int nsys, int total_blocks, cudaGraphConditionalHandle cond, int use_cond) {
-  force_body<GBMD_MIXED, 1, MT, MODE_STEP, EVAL>(sysv, tiles, ctl, nsys, total_blocks, cond,
-                                                 use_cond);
+  force_body<GBMD_MIXED, 1, MT, MODE_STEP, EVAL>(sysv, tiles[blockIdx.x], nullptr, ctl, nsys,
+                                                 total_blocks, cond, use_cond);
 }
 
 // the k_force variant for (precision, threads per particle, table mode, mode) with

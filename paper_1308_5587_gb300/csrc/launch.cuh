@@ -67,6 +67,10 @@ KernelCall tree_nlist_call(const SysDev* d, const Tile* tiles_g, int ntiles, Gro
 // the thermostat.  nvt_b_call: the second half (opening scaling and kick, drift,
 // shadow, rebuild check, end-of-step decisions).
 enum { MODE_FORCE = 0, MODE_EV = 1, MODE_STEP = 2, MODE_NVT_A = 3 };
+// which step configurations take wide tiles, a warp a particle (all modes of one do, so
+// that a readout's forces are the step's): not the register-capped step kernel of one
+// lane a particle
+__host__ __device__ constexpr bool has_wide(int prec, int tpp) { return prec == GBMD_FP64 || tpp > 1; }
 struct StepArgs {
   int nsys = 0;             // systems of the group (decisions of the last block)
   int total_blocks = 0;     // blocks of all the step's force launches
