@@ -211,15 +211,19 @@ struct SysDev {
   Flags *flags;
 };
 
+// barrier of a team of resident blocks that is no cluster (team_core.cuh): arrivals with
+// their votes, and the generation that releases the waiting blocks
+struct TeamSync {
+  unsigned long long arrive, release;
+};
+
 // group-level control block (one per single system or batch)
 struct GroupCtl {
   unsigned int blocks_done;  // last-block counter of the step kernel
   unsigned int blocks_done_a;   // last-block counter of the NVT force half
   int any_rebuild;
   unsigned long long launches;
-  // barrier of a team that is a whole grid (k_team.cuh): arrivals with their votes, and
-  // the generation that releases the waiting blocks
-  unsigned long long team_arrive, team_release;
+  TeamSync team;             // of a team that is a whole grid
 };
 
 struct Tile { int sys, first, count, pad; };

@@ -321,8 +321,8 @@ __global__ void __launch_bounds__(REBUILD_T, 1) k_rebuild(const SysDev* __restri
   tm.cluster = 0;
   tm.size = (int)gridDim.x;
   tm.rank = (int)blockIdx.x;
-  tm.ctl = ctl;
-  tm.gen = (unsigned)(*(const volatile unsigned long long*)&ctl->team_release >> 8);
+  tm.sync = &ctl->team;
+  tm.gen = (unsigned)(*(const volatile unsigned long long*)&ctl->team.release >> 8);
   tm.par = 0;
   tm.slot = nullptr;
   tm.word = &word;

@@ -36,18 +36,26 @@ __global__ void __launch_bounds__(TEAM_T, 1) k_team(TeamArgs a) {
   tm.cluster = a.cluster;
   tm.size = a.cluster ? a.cluster : (int)gridDim.x;
   tm.rank = a.cluster ? (int)(blockIdx.x % a.cluster) : (int)blockIdx.x;
-  tm.ctl = a.ctl;
+  tm.sync = &a.ctl->team;
+  int member = a.cluster ? (int)(blockIdx.x / a.cluster) : 0;
+  if (a.share) {
+    const int4 sh = a.share[blockIdx.x];
+    member = sh.x;
+    tm.rank = sh.y;
+    tm.size = sh.z;
+    tm.sync = a.sync + sh.w;
+  }
   tm.gen = 0;
   tm.par = 0;
   tm.slot = slot;
   tm.word = &word;
-  const SysDev& s = a.desc[a.list[a.cluster ? blockIdx.x / a.cluster : 0]];
+  const SysDev& s = a.desc[a.list[member]];
   // The flags change only after the team's first barrier, so every block reads the same.
   const FlagWords fw = load_flag_words(s.flags);
   const longlong2 sl = load_flag_pair(&s.flags->step);        // (step, step_limit)
   const longlong2 lr = load_flag_pair(&s.flags->last_sort);   // (last_sort, n_rebuilds)
   const long long nsort0 = ((const volatile Flags*)s.flags)->n_sorts;
-  if (!a.cluster) tm.gen = (unsigned)(*(const volatile unsigned long long*)&a.ctl->team_release >> 8);
+  if (!a.cluster) tm.gen = (unsigned)(*(const volatile unsigned long long*)&tm.sync->release >> 8);
   if (fw.error != 0 || (sl.y >= 0 && sl.x >= sl.y)) return;
   if (a.cluster) cooperative_groups::this_cluster().sync();   // every block runs: its shared
                                                               // memory may be written
@@ -138,7 +146,7 @@ __global__ void __launch_bounds__(TEAM_T, 1) k_team(TeamArgs a) {
       const unsigned v = tm.vote(bad ? VOTE_BAD : 0u);
       if (v & VOTE_LOST) { error = DEV_TEAM; break; }
       if (v & VOTE_BAD) { error = DEV_NONFINITE; break; }
-      const double sum = nh_total(s.nh_part + s.nh_first, chunks, sm.slots);
+      const double sum = nh_total(s.nh_part + s.nh_first, chunks, sm.sums);
       if (threadIdx.x == 0) nvt_sc = nh_update(s, sum, vfull, xi, eta);
       __syncthreads();
       sc = nvt_sc;

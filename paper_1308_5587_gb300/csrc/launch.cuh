@@ -126,7 +126,11 @@ struct TeamArgs {
   const int* list;   // the systems of the launch (positions in desc), the largest first
   GroupCtl* ctl;
   int nsteps;
-  int cluster;       // blocks of a team; 0: the grid is one team
+  int cluster;       // blocks of a team; 0: the grid is one team, or several by `share`
+  // per block of the grid, or null: (position in list, rank in its team, the team's
+  // blocks, its barrier in sync)
+  const int4* share;
+  TeamSync* sync;
 };
 void* k_team_variant(int eval, int prec, int tpp, int mt);
 

@@ -144,14 +144,18 @@ __device__ __forceinline__ double nvt_close(const SysDev& s, int i, const double
 // The sum of v.v over a system, in an order that depends on the lanes per particle alone
 // and not on how the particles are spread over blocks or kernels: a warp's particles
 // (32 / TPP consecutive ones, a chunk) by shuffles, the chunks' sums in NH_SLOTS strided
-// slots, the slots in a tree.
-constexpr int NH_SLOTS = 256;
+// slots, 32 slots at a time by shuffles, then those sums by shuffles.  In the team kernel
+// every step waits for it: one barrier of the block (a tree in shared memory took eight;
+// 50 NVT steps with readouts, N = 20,011: 1,746 us with it, 1,719 so).
+constexpr int NH_SLOTS = 512, NH_SUMS = NH_SLOTS / 32;
 __device__ __forceinline__ double nh_warp_sum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
   return v;   // lane 0
 }
-// every thread of the block calls it; the sum is returned to all
-__device__ __forceinline__ double nh_total(const double* part, int count, double* slots) {
+// every thread of the block (whole warps) calls it; the sum is returned to all.  `sums`
+// (shared) may be written again after the block's next barrier.
+__device__ __forceinline__ double nh_total(const double* part, int count, double* sums) {
+  const int lane = threadIdx.x & 31;
   for (int v = threadIdx.x; v < NH_SLOTS; v += blockDim.x) {
     double a = 0.0;
     int k = v;
@@ -162,16 +166,17 @@ __device__ __forceinline__ double nh_total(const double* part, int count, double
 #pragma unroll
       for (int u = 0; u < 4; ++u) a += p[u];
     }
-    for (; k < count; k += NH_SLOTS) a += __ldcg(part + k);
-    slots[v] = a;
+    double p[3];
+#pragma unroll
+    for (int u = 0; u < 3; ++u) p[u] = k + u * NH_SLOTS < count ? __ldcg(part + k + u * NH_SLOTS) : 0.0;
+#pragma unroll
+    for (int u = 0; u < 3; ++u) a += p[u];
+    a = nh_warp_sum(a);
+    if (lane == 0) sums[v >> 5] = a;
   }
   __syncthreads();
-  for (int w = NH_SLOTS / 2; w > 0; w >>= 1) {
-    for (int v = threadIdx.x; v < w; v += blockDim.x) slots[v] += slots[v + w];
-    __syncthreads();
-  }
-  const double r = slots[0];
-  __syncthreads();
+  double r = sums[lane & (NH_SUMS - 1)];
+  for (int o = NH_SUMS / 2; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
   return r;
 }
 
@@ -203,7 +208,7 @@ __device__ __forceinline__ void nvt_half_tail(const SysDev& s, const SysDev* __r
   const double part = nh_warp_sum(uu);
   if ((threadIdx.x & 31) == 0 && chunk >= 0) s.nh_part[s.nh_first + chunk] = part;
   __shared__ int last;
-  __shared__ double slots[NH_SLOTS];
+  __shared__ double sums[NH_SUMS];
   __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -219,7 +224,8 @@ __device__ __forceinline__ void nvt_half_tail(const SysDev& s, const SysDev* __r
     const FlagWords w = load_flag_words(sk.flags);
     const longlong2 sl = load_flag_pair(&sk.flags->step);
     if (!(w.error == 0 && (sl.y < 0 || sl.x < sl.y))) continue;
-    const double sum = nh_total(sk.nh_part + sk.nh_first, sk.nh_count, slots);
+    __syncthreads();   // the previous system's sums have been read
+    const double sum = nh_total(sk.nh_part + sk.nh_first, sk.nh_count, sums);
     if (threadIdx.x == 0) {
       double xi = sk.nh[0], eta = sk.nh[1];
       sk.nh[2] = nh_update(sk, sum, w.v_full, xi, eta);

@@ -5,7 +5,8 @@
 //   * a thread-block cluster (hardware barrier, votes through distributed shared
 //     memory): one per system, so a launch steps any number of systems side by side; or
 //   * the whole grid of a cooperative launch (one system), for systems with more work
-//     than one cluster's SMs should carry: arrivals on one counter, the last one
+//     than one cluster's SMs should carry, or a share of that grid (a batch whose
+//     clusters would not all run at once): arrivals on one counter, the last one
 //     publishes the outcome.  Waits are bounded; one that runs out sets DEV_TEAM.
 #pragma once
 #include <cooperative_groups.h>
@@ -38,13 +39,13 @@ union TeamSmem {
   WarpRing<false, SLOTS> warp[T / 32];
   struct { TreeWarp warp[T / 32]; TreeTable tab; } tree;
   struct { int start[SCAN_MAX + 1], warp[32]; } scan;
-  double slots[NH_SLOTS];
+  double sums[NH_SUMS];
   int queue[16 * T];   // FP64 force phase (k_force.cuh)
 };
 
 struct Team {
-  int rank, size, cluster;   // this block, blocks, 0: the whole grid
-  GroupCtl* ctl;
+  int rank, size, cluster;   // this block, blocks, 0: no cluster
+  TeamSync* sync;
   unsigned gen;              // grid: generation last seen released
   int par;                   // cluster: which vote slots are in use
   unsigned* slot;            // [2][TEAM_MAX_CLUSTER] in shared memory
@@ -74,19 +75,19 @@ struct Team {
                                      ((unsigned long long)((v & VOTE_BAD) >> 1) << 48);
       unsigned long long all;
       asm volatile("atom.add.acq_rel.gpu.global.u64 %0, [%1], %2;"
-                   : "=l"(all) : "l"(&ctl->team_arrive), "l"(add) : "memory");
+                   : "=l"(all) : "l"(&sync->arrive), "l"(add) : "memory");
       all += add;
       unsigned out;
       if ((unsigned)all == (unsigned)size) {
         out = (((all >> 32) & 0xffffu) ? VOTE_NEED : 0u) | ((all >> 48) ? VOTE_BAD : 0u);
-        ctl->team_arrive = 0ull;
+        sync->arrive = 0ull;
         const unsigned long long rel = ((unsigned long long)(gen + 1u) << 8) | out;
-        asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(&ctl->team_release), "l"(rel) : "memory");
+        asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(&sync->release), "l"(rel) : "memory");
       } else {
         out = VOTE_LOST;
         for (int k = 0; k < TEAM_SPIN; ++k) {
           unsigned long long rel;
-          asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(rel) : "l"(&ctl->team_release) : "memory");
+          asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(rel) : "l"(&sync->release) : "memory");
           if ((unsigned)(rel >> 8) == gen + 1u) {
             out = (unsigned)rel & 0xffu;
             break;
