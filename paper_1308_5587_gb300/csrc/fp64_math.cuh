@@ -33,15 +33,17 @@ struct FixDiff {
     m = (unsigned long long)L - m;
     sign ^= 0x80000000u;
   }
-  __device__ __forceinline__ double value(int fix_bits) const {
-    int sh;
-    if (hi() != 0u) {
-      sh = __clz(hi()) - 1;
-    } else {   // below 2^-29 of half the edge
-      if (m == 0ull) return 0.0;
-      sh = __clzll(m) - 1;
-    }
+  // as FP64; sets `close` where |d| is below 2^32 units (2^-29 of half the edge, or 0) and
+  // value_any is to be taken instead
+  __device__ __forceinline__ double value(int fix_bits, bool& close) const {
+    close |= hi() == 0u;
+    const int sh = (__clz(hi()) - 1) & 31;
     return fix_pack(m << sh, 1022 + 62 - fix_bits - sh, sign);
+  }
+  __device__ __forceinline__ double value_any(int fix_bits) const {
+    if (m == 0ull) return 0.0;
+    const int lead = __clzll(m);   // 1 at least
+    return fix_pack(m << (lead - 1), 1022 + 62 - fix_bits - (lead - 1), sign);
   }
 };
 __device__ __forceinline__ FixDiff fix_diff(long long a, long long b) {
@@ -56,12 +58,12 @@ struct FixR2 {
   __device__ __forceinline__ double value() const { return m ? fix_pack(m, e, 0u) : 0.0; }
 };
 
-// |d|^2 below 2^96 units: all 128 bits of it
-static __device__ __noinline__ FixR2 fix_r2_close(unsigned long long x, unsigned long long y,
-                                                  unsigned long long z, int fix_bits) {
+// |d|^2 of any size: all 128 bits of it
+static __device__ __noinline__ FixR2 fix_r2_any(unsigned long long x, unsigned long long y,
+                                                unsigned long long z, int fix_bits) {
   using u64 = unsigned long long;
   const unsigned __int128 r = (unsigned __int128)x * x + (unsigned __int128)y * y + (unsigned __int128)z * z;
-  u64 s = (u64)(r >> 64);   // below 2^32
+  u64 s = (u64)(r >> 64);   // below 2^61
   u64 t = (u64)r;
   int e = 1022 + 126 - 2 * fix_bits;
   if (s == 0ull) {
@@ -75,9 +77,10 @@ static __device__ __noinline__ FixR2 fix_r2_close(unsigned long long x, unsigned
   return FixR2{m, e - (lead - 1)};
 }
 
-// |d|^2 for components up to 2^61
+// |d|^2 for components up to 2^61; sets `close` where it is below 2^96 units (r below 2^-13
+// of half the longest edge) and fix_r2_any is to be taken instead
 __device__ __forceinline__ FixR2 fix_r2(const FixDiff& x, const FixDiff& y, const FixDiff& z,
-                                        int fix_bits) {
+                                        int fix_bits, bool& close) {
   using u64 = unsigned long long;
   const unsigned xl = (unsigned)x.m, yl = (unsigned)y.m, zl = (unsigned)z.m;
   const unsigned xh = x.hi(), yh = y.hi(), zh = z.hi();   // <= 2^29
@@ -89,9 +92,8 @@ __device__ __forceinline__ FixR2 fix_r2(const FixDiff& x, const FixDiff& y, cons
   const u64 a = (mid << 1) + low;
   const u64 s = high + (a >> 32);
   const unsigned t = (unsigned)a;
-  // r below 2^-13 of half the longest edge
-  if ((unsigned)(s >> 32) == 0u) return fix_r2_close(x.m, y.m, z.m, fix_bits);
-  const int sh = __clz((unsigned)(s >> 32)) - 1;   // 1 .. 30
+  close |= (unsigned)(s >> 32) == 0u;
+  const int sh = (__clz((unsigned)(s >> 32)) - 1) & 31;   // 1 .. 30
   return FixR2{s << sh | t >> (32 - sh), 1022 + 126 - 2 * fix_bits - sh};
 }
 
