@@ -1427,7 +1427,11 @@ int create_impl(const gbmd_desc* d, gbmd_system** out, bool device) {
   // steps 10% faster than with two lanes in 128-thread blocks), four lanes in
   // 128-thread blocks below (the 4,000-particle fluid 29% faster)
   const bool fp64 = d->precision == GBMD_FP64;
-  const int auto_tpp = fp64 ? (d->n >= 32768 ? 1 : 4) : (d->n >= (1 << 19) ? 1 : 2);
+  // FP64: four lanes while the team's warps take them in one turn (152 SMs of 16 warps,
+  // eight particles a warp: 19,456), us a step with 4 / 2 lanes: N = 4,000 22.0 / 30.6,
+  // 16,000 33.0 / 35.7, 20,000 53.1 / 41.0, 28,000 54.7 / 45.3; one from 32,768 on (64,000:
+  // 85.9, two lanes 91.0)
+  const int auto_tpp = fp64 ? (d->n >= 32768 ? 1 : d->n > 19456 ? 2 : 4) : (d->n >= (1 << 19) ? 1 : 2);
   s->own->tpp = d->threads_per_particle ? d->threads_per_particle : auto_tpp;
   s->own->fblock = fp64 && s->own->tpp == 1 ? 64 : 128;
   if (const char* ev = getenv("GBMD_NO_GRAPHS")) s->own->use_graphs = ev[0] != '1';

@@ -165,6 +165,31 @@ def test_batch_of_every_cluster_size_and_the_rest_equals_alone():
         s.close()
 
 
+@pytest.mark.parametrize("sizes", [
+    [2, 300, 1000, 2300, 2600, 3100, 3700, 4100, 4800, 5500, 6300, 7200, 8300, 9000],
+    [240 + k for k in range(160)]], ids=["shares_of_one_grid", "more_teams_than_SMs"])
+def test_batch_of_many_members_equals_alone(sizes):
+    ws = [few(n) if n == 2 else fluid(n)() for n in sizes]
+    b = gbmd.Batch("mixed")
+    b.set_tuning(2, 128)
+    ss = [gbmd.System.from_workload(w, precision="mixed") for w in ws]
+    for s in ss:
+        b.add(s)
+    b.step(STEPS)
+    got = [(s.state(), s.thermo()) for s in ss]
+    b.close()
+    for w, s, (st, th) in list(zip(ws, ss, got))[::max(1, len(ws) // 16)]:
+        a = gbmd.System.from_workload(w, precision="mixed")
+        a.set_tuning(2, 128)
+        a.step(STEPS)
+        for x, y in zip(a.state(), st):
+            assert np.array_equal(x, y)
+        assert a.thermo() == th
+        a.close()
+    for s in ss:
+        s.close()
+
+
 @pytest.mark.parametrize("n", [2, 31, 33, 4095, 131072, 131073])
 @pytest.mark.parametrize("prec", ["mixed", "fp64"])
 def test_thermo_sums_at_the_edges_of_its_tiles(prec, n):
