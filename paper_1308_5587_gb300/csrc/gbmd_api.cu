@@ -231,15 +231,22 @@ int tree_groups(const SysDev& d, int ty) {
 
 // Systems that the team kernel may step: the cell list on the global force path,
 // without ghosts (their rebuilds are the caller's).  Alone it pays while a step is short
-// beside the launches it saves: up to TEAM_ALONE_N particles (64,000, mixed: 27.7 us a
-// step against 28.2 by the step kernel and k_rebuild; 200,000: 73 against 66; FP64 at
-// 64,000: 223 against 223).  In a batch, where a shared launch makes every member wait
-// for any member's rebuild, up to what one cluster steps in about 50 us.
+// beside the launches it saves: up to one turn of its warps, in mixed precision with two
+// lanes a particle done by one (k_team.cuh), and with more lanes up to TEAM_ALONE_N.  With
+// readouts, us: N = 64,000 mixed, 50 steps, 1,789 by the step kernel and k_rebuild, 1,663
+// by the team; FP64, 20 steps, 2,291 and 2,211; FP64 NVT, 20 steps, 2,690 and 2,397.
+// (N = 200,000, several turns: 73 us a step by the team, 66 by the step kernel.)
+// In a batch, where a shared launch makes every member wait for any member's rebuild, up
+// to what one cluster steps in about 50 us.
 constexpr int TEAM_ALONE_N = 49152;
+constexpr int TEAM_TURN_N = 152 * TEAM_T;   // one turn of the team's warps, one lane a particle
 constexpr int TEAM_CLUSTER_N = 32768;
 constexpr int TEAM_STEPS = 64;   // steps of one launch
 bool team_member(const Group* g, const SysDev& d) {
-  return !d.tree && !d.staged && d.n_ghost == 0 && d.n <= (g->is_batch ? TEAM_CLUSTER_N : TEAM_ALONE_N);
+  if (d.tree || d.staged || d.n_ghost > 0) return false;
+  if (g->is_batch) return d.n <= TEAM_CLUSTER_N;
+  const int lanes = g->precision == GBMD_MIXED && g->tpp == 2 ? 1 : g->tpp;
+  return d.n <= std::max(TEAM_ALONE_N, TEAM_TURN_N / lanes);
 }
 
 // The force tiles of a system, `per` particles each.  The particles of a wide type of a
@@ -702,12 +709,24 @@ std::vector<int4> team_shares(const std::vector<int>& chunks, int sms) {
   return out;
 }
 int launch_team(Group* g, long long n) {
-  void* f = k_team_variant(g->eval, g->precision, g->tpp, g->multi);
+  void* f = k_team_variant(g->eval, g->precision, g->tpp, g->multi, false);
   TeamFit fit;
   RET(team_fit(f, TEAM_T, TEAM_SMEM, g->device, &fit));
-  if (fit.max_cluster < 1) return fail(GBMD_ERR_CUDA, "the team kernel does not fit the device");
   const int warps = TEAM_T / 32;
-  auto chunks_of = [&](int nn) { return (int)(((long long)nn * g->tpp + 31) / 32); };
+  // two lanes a particle as one where that leaves every warp of the chip a chunk: a
+  // system with more than one turn of them at two lanes, a batch with more than two
+  int lanes = g->tpp;
+  if (g->precision == GBMD_MIXED && g->tpp == 2) {
+    long long total = 0;
+    for (int nn : g->team_n) total += ((long long)nn * 2 + 31) / 32;
+    if (total > (long long)(g->is_batch ? 2 : 1) * fit.sms * warps) {
+      lanes = 1;
+      f = k_team_variant(g->eval, g->precision, g->tpp, g->multi, true);
+      RET(team_fit(f, TEAM_T, TEAM_SMEM, g->device, &fit));
+    }
+  }
+  if (fit.max_cluster < 1) return fail(GBMD_ERR_CUDA, "the team kernel does not fit the device");
+  auto chunks_of = [&](int nn) { return (int)(((long long)nn * lanes + 31) / 32); };
   TeamArgs a{};
   a.desc = g->d_desc;
   a.ctl = g->d_ctl;
@@ -736,7 +755,7 @@ int launch_team(Group* g, long long n) {
     if (g->share_dirty) {
       std::vector<int> chunks;
       for (int nn : g->team_n) chunks.push_back(chunks_of(nn));
-      g->share = team_shares(chunks, fit.sms);
+      g->share = team_shares(chunks, fit.sms);   // `lanes` changes with the layout only
       RET(grow(&g->d_share, &g->cap_share, g->share.size()));
       if (!g->d_sync) {   // a team a block at most
         RET(grow(&g->d_sync, &g->cap_sync, (size_t)fit.sms));

@@ -205,20 +205,20 @@ __global__ void __launch_bounds__(STAGED_BLOCK) k_force_staged(const SysDev* __r
 
 
 #define TEAM_DECL(e) \
-  void* k_team_##e##_mixed(int tpp, int mt); \
-  void* k_team_##e##_fp64(int tpp, int mt);
+  void* k_team_##e##_mixed(int tpp, int mt, bool two_in_one); \
+  void* k_team_##e##_fp64(int tpp, int mt, bool two_in_one);
 TEAM_DECL(lj)
 TEAM_DECL(mie)
 TEAM_DECL(yukawa)
 TEAM_DECL(gauss)
 #undef TEAM_DECL
-void* k_team_variant(int eval, int prec, int tpp, int mt) {
+void* k_team_variant(int eval, int prec, int tpp, int mt, bool two_in_one) {
   const bool d = prec == GBMD_FP64;
   switch (eval) {
-    case EVAL_MIE: return d ? k_team_mie_fp64(tpp, mt) : k_team_mie_mixed(tpp, mt);
-    case EVAL_YUKAWA: return d ? k_team_yukawa_fp64(tpp, mt) : k_team_yukawa_mixed(tpp, mt);
-    case EVAL_GAUSS: return d ? k_team_gauss_fp64(tpp, mt) : k_team_gauss_mixed(tpp, mt);
-    default: return d ? k_team_lj_fp64(tpp, mt) : k_team_lj_mixed(tpp, mt);
+    case EVAL_MIE: return d ? k_team_mie_fp64(tpp, mt, two_in_one) : k_team_mie_mixed(tpp, mt, two_in_one);
+    case EVAL_YUKAWA: return d ? k_team_yukawa_fp64(tpp, mt, two_in_one) : k_team_yukawa_mixed(tpp, mt, two_in_one);
+    case EVAL_GAUSS: return d ? k_team_gauss_fp64(tpp, mt, two_in_one) : k_team_gauss_mixed(tpp, mt, two_in_one);
+    default: return d ? k_team_lj_fp64(tpp, mt, two_in_one) : k_team_lj_mixed(tpp, mt, two_in_one);
   }
 }
 

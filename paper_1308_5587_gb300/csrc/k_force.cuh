@@ -208,7 +208,9 @@ __device__ __forceinline__ void pair2(const int4& qi, const int4& qa, const int4
 
 // The sums over the neighbour row of particle i, particle's lane h of TPP: slot groups
 // h, h + TPP, .. in order, U of them in flight (4 U gathers), pairs two at a time.  The
-// order of the sums does not depend on U.  COH: the positions and the list may have
+// order of the sums does not depend on U.  V = 2 (TPP = 1): one lane does the work of two
+// lanes a particle, even slot groups into fx[0], odd ones into fx[1], which the caller
+// adds up as two lanes would: the same sums.  COH: the positions and the list may have
 // been written by this kernel (plain loads), else they are read-only here.
 template <bool COH, typename T>
 __device__ __forceinline__ T load_ro(const T* p) {
@@ -227,10 +229,11 @@ __device__ __forceinline__ int4 load_list(const int4* p) {
         : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "l"(p));
   return v;
 }
-template <int TPP, int MT, int EVAL, bool EV, bool COH, int U>
+template <int TPP, int MT, int EVAL, bool EV, bool COH, int U, int V = 1>
 __device__ __forceinline__ void gather_mixed(const SysDev& s, const int4* qv, const int4& qi, int i,
-                                             int h, int n, const PairF* tabf, float2& fx,
-                                             float2& fy, float2& fz, float2& e, float2* w) {
+                                             int h, int n, const PairF* tabf, float2 (&fx)[V],
+                                             float2 (&fy)[V], float2 (&fz)[V], float2& e, float2* w) {
+  static_assert(V == 1 || (V == 2 && TPP == 1 && U == 2 && !EV), "virtual lanes");
   const int nt = s.ntypes;
   const int groups = (n + 3) >> 2;
   const int4* nl4 = reinterpret_cast<const int4*>(s.nl) + i;
@@ -255,8 +258,9 @@ __device__ __forceinline__ void gather_mixed(const SysDev& s, const int4* qv, co
     if (MT == 1) return tj ? r1 : r0;
     return tabf[qi.w * nt + tj];
   };
-  fx = fy = fz = e = make_float2(0.f, 0.f);
-  for (int c = 0; c < 6; ++c) w[c] = fx;
+  e = make_float2(0.f, 0.f);
+  for (int v = 0; v < V; ++v) fx[v] = fy[v] = fz[v] = e;
+  for (int c = 0; c < 6; ++c) w[c] = e;
   for (int gg = h; gg < groups; gg += U * TPP) {
     int4 q[U][4];
 #pragma unroll
@@ -279,8 +283,9 @@ __device__ __forceinline__ void gather_mixed(const SysDev& s, const int4* qv, co
       const bool o0 = k0 < n, o1 = k0 + 1 < n, o2 = k0 + 2 < n, o3 = k0 + 3 < n;
       const int4 q0 = q[u][0], q1 = q[u][1], q2 = q[u][2], q3 = q[u][3];
       const PairF P0 = par(q0.w), P1 = par(q1.w), P2 = par(q2.w), P3 = par(q3.w);
-      pair2<EVAL, EV>(qi, q0, q1, o0, o1, sc0, sc1, sc2, P0, P1, fx, fy, fz, e, w);
-      pair2<EVAL, EV>(qi, q2, q3, o2, o3, sc0, sc1, sc2, P2, P3, fx, fy, fz, e, w);
+      const int v = V == 1 ? 0 : u;
+      pair2<EVAL, EV>(qi, q0, q1, o0, o1, sc0, sc1, sc2, P0, P1, fx[v], fy[v], fz[v], e, w);
+      pair2<EVAL, EV>(qi, q2, q3, o2, o3, sc0, sc1, sc2, P2, P3, fx[v], fy[v], fz[v], e, w);
     }
   }
 }
@@ -466,12 +471,12 @@ __device__ __forceinline__ void force_body(const SysDev* __restrict__ sysv, cons
   if (PREC == GBMD_MIXED) {
     const int4* __restrict__ qv = q_at(s, step);
     const int4 qi = qv[i];
-    float2 fx, fy, fz, e, w[6];
+    float2 fx[1], fy[1], fz[1], e, w[6];
     gather_mixed<TPP, MT, EVAL, EV, false, 1>(s, qv, qi, i, h, n, tabf, fx, fy, fz, e, w);
     // the two halves of each packed accumulator, then the TPP lanes
-    const float Fx = group_sum<TPP>(fx.x + fx.y);
-    const float Fy = group_sum<TPP>(fy.x + fy.y);
-    const float Fz = group_sum<TPP>(fz.x + fz.y);
+    const float Fx = group_sum<TPP>(fx[0].x + fx[0].y);
+    const float Fy = group_sum<TPP>(fy[0].x + fy[0].y);
+    const float Fz = group_sum<TPP>(fz[0].x + fz[0].y);
     float E = 0.f, W[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     if (EV) {
       E = group_sum<TPP>(e.x + e.y);

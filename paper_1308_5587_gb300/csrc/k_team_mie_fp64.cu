@@ -3,6 +3,8 @@
 
 namespace gbmd {
 
-void* k_team_mie_fp64(int tpp, int mt) { return k_team_tpp<EVAL_MIE, GBMD_FP64>(tpp, mt); }
+void* k_team_mie_fp64(int tpp, int mt, bool two_in_one) {
+  return k_team_tpp<EVAL_MIE, GBMD_FP64>(tpp, mt, two_in_one);
+}
 
 }  // namespace gbmd

@@ -3,6 +3,8 @@
 
 namespace gbmd {
 
-void* k_team_mie_mixed(int tpp, int mt) { return k_team_tpp<EVAL_MIE, GBMD_MIXED>(tpp, mt); }
+void* k_team_mie_mixed(int tpp, int mt, bool two_in_one) {
+  return k_team_tpp<EVAL_MIE, GBMD_MIXED>(tpp, mt, two_in_one);
+}
 
 }  // namespace gbmd

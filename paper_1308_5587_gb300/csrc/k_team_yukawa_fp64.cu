@@ -3,6 +3,8 @@
 
 namespace gbmd {
 
-void* k_team_yukawa_fp64(int tpp, int mt) { return k_team_tpp<EVAL_YUKAWA, GBMD_FP64>(tpp, mt); }
+void* k_team_yukawa_fp64(int tpp, int mt, bool two_in_one) {
+  return k_team_tpp<EVAL_YUKAWA, GBMD_FP64>(tpp, mt, two_in_one);
+}
 
 }  // namespace gbmd

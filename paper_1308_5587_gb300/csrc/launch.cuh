@@ -132,7 +132,8 @@ struct TeamArgs {
   const int4* share;
   TeamSync* sync;
 };
-void* k_team_variant(int eval, int prec, int tpp, int mt);
+// two_in_one: mixed with two lanes a particle, one lane doing the work of both
+void* k_team_variant(int eval, int prec, int tpp, int mt, bool two_in_one);
 
 // arithmetic throughput probe (k_probe.cu): one timed launch over every SM
 cudaError_t probe_run(int kind, cudaStream_t st, int iters, double* ops, float* ms);

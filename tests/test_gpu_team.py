@@ -72,7 +72,13 @@ CASES = {
                          {"nvt": 1.2, "sort_period": 20}),
     "gauss_700_fp64": (fluid(700, pairs=wl.gauss_single()), "fp64", {}),
     "n49152_team": (fluid(49152), "mixed", {"sort_period": 30}),
-    "n49153_coop_rebuild": (fluid(49153), "mixed", {"sort_period": 30}),
+    "n49153_two_in_one": (fluid(49153), "mixed", {"sort_period": 30}),
+    "n77824_team_two_in_one": (fluid(77824), "mixed", {"sort_period": 30}),
+    "n40001_two_in_one_nvt": (fluid(40001), "mixed", {"nvt": 1.2}),
+    "ka_39001_two_in_one": (lambda: wl.lj_fluid(39001, 1.2, 1.0, seed=39, binary=True, r_buff=0.3),
+                            "mixed", {}),
+    "n77825_coop_rebuild": (fluid(77825), "mixed", {}),
+    "n60001_fp64_team": (fluid(60001), "fp64", {"sort_period": 30}),
     "clump_1728_buckets_run_over": (clump, "mixed", {"sort_period": 3}),
     "dilute_1500_no_buckets": (lambda: wl.lj_fluid(1500, 0.02, 1.2, seed=38), "mixed",
                                {"sort_period": 2}),
