@@ -449,9 +449,11 @@ std::vector<KernelCall> rebuild_calls(const Group* g) {
 }
 
 // forces at the current positions, outside the step (autotuning, readouts)
-KernelCall plain_force_call(const Group* g) {
+KernelCall plain_force_call(const Group* g, int readout = 0) {
+  StepArgs sa;
+  sa.readout = readout;
   return force_call(g->precision, g->multi, MODE_FORCE, g->tpp, g->fblock, g->d_desc, g->d_tf,
-                    g->ntf, g->d_ctl, StepArgs{}, g->eval);
+                    g->ntf, g->d_ctl, sa, g->eval);
 }
 
 // energy/virial launch of the global-list systems: the step's threads per particle
@@ -463,9 +465,9 @@ KernelCall ev_force_call(const Group* g, const SysDev* desc) {
 
 // readout force launches (ev = 0 forces, 1 also energy/virial): global-list systems,
 // then staged ones
-std::vector<KernelCall> force_calls(const Group* g, int ev) {
+std::vector<KernelCall> force_calls(const Group* g, int ev, int readout = 0) {
   std::vector<KernelCall> v;
-  if (g->ntf > 0) v.push_back(ev ? ev_force_call(g, g->d_desc) : plain_force_call(g));
+  if (g->ntf > 0) v.push_back(ev ? ev_force_call(g, g->d_desc) : plain_force_call(g, readout));
   if (g->ntb > 0)
     v.push_back(force_staged_call(g->multi, ev ? MODE_EV : MODE_FORCE, g->d_desc, g->d_tb, g->ntb,
                                   g->d_ctl, g->nte, g->window_cap, StepArgs{}));
@@ -1558,6 +1560,9 @@ void fill_thermo(gbmd_system* s, const Snapshot& snap, gbmd_thermo* out) {
 // So a readout costs one round trip to the device (two where its arrays are too big for
 // one copy through `bounce`), not one for each thing it must know.
 constexpr size_t BOUNCE_MAX = 256 * 1024;
+// forces and rows by one kernel / by two: N = 64,000 frame 19.4 / 21.5 us, N = 199,999 frame
+// 51.2 / 49.3, N = 10^6 forces 181 / 168 (and a launch)
+constexpr size_t FUSED_READ_N = 131072;
 
 int thermo_impl(gbmd_system* s, Snapshot* snap) {
   Group* g = s->own;
@@ -1581,13 +1586,19 @@ int export_impl(gbmd_system* s, double* pos, double* vel, int32_t* image, double
   if ((pp_u || pp_w) && !s->d_ppw) return fail(GBMD_ERR_STATE, "per-particle arrays not allocated");
   for (int turn = 0; turn < 2; ++turn) {
     RET(sync_layout(g));
+    // the global-list force kernel writes the rows of a readout itself; up to FUSED_READ_N,
+    // beyond which its stores to scattered tags cost more than k_export's launch
+    const int readout = !pp_u && !pp_w && (vel || force) && g->ntb == 0 && N <= FUSED_READ_N
+                            ? (force ? READ_FORCE : 0) | (vel ? READ_VEL : 0) | (pos ? READ_POS : 0) |
+                                  (image ? READ_IMAGE : 0)
+                            : 0;
     // forces and full-step velocities need F at the current positions: the step kernel
     // does not store its force, so evaluate it here (per-particle arrays: the energy pass)
     if (pp_u || pp_w)
       for (const KernelCall& c : force_calls(g, 1)) CK(launch(c, st));
     else if (vel || force)
-      for (const KernelCall& c : force_calls(g, 0)) CK(launch(c, st));
-    CK(launch(export_call(g->d_desc, g->d_tp, g->ntp, pos ? s->d_pos : nullptr,
+      for (const KernelCall& c : force_calls(g, 0, readout)) CK(launch(c, st));
+    if (!readout) CK(launch(export_call(g->d_desc, g->d_tp, g->ntp, pos ? s->d_pos : nullptr,
                           vel ? s->d_vel : nullptr, image ? s->d_img : nullptr,
                           force ? s->d_frc : nullptr, pp_u ? s->d_ppu : nullptr,
                           pp_w ? s->d_ppw : nullptr), st));

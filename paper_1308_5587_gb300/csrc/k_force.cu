@@ -239,7 +239,7 @@ KernelCall force_call(int prec, int multi, int mode, int tpp, int block, const S
   const size_t smem = prec == GBMD_FP64 ? (size_t)block * FP64_QUEUE * sizeof(int) : 0;
   KernelCall k = make_call(f, ntiles, block, smem);
   put(k, d); put(k, tiles_f); put(k, ctl); put(k, sa.nsys); put(k, sa.total_blocks);
-  put(k, sa.cond); put(k, sa.use_cond);
+  put(k, sa.cond); put(k, sa.use_cond); put(k, sa.readout);
   return k;
 }
 

@@ -11,6 +11,7 @@
 #include <cstring>
 
 #include "launch.cuh"
+#include "step_core.cuh"
 
 namespace gbmd {
 
@@ -19,22 +20,14 @@ namespace gbmd {
 // the kinetic term sum v^2 at full-step velocities, in a fixed order.
 // thermo[0] = pe, thermo[1] = sum v^2, thermo[2..7] = W.
 // ---------------------------------------------------------------------------
-// one thread: the system's flags and thermostat into its Snapshot
-__device__ __forceinline__ void take_snapshot(const SysDev& s) {
-  Snapshot* o = reinterpret_cast<Snapshot*>(s.thermo);
-  const volatile long long* f = reinterpret_cast<const volatile long long*>(s.flags);
-  long long* to = reinterpret_cast<long long*>(&o->flags);
-  for (int k = 0; k < (int)(sizeof(Flags) / 8); ++k) to[k] = f[k];
-  for (int k = 0; k < 3; ++k) o->nh[k] = s.nh[k];
-}
 __global__ void k_snapshot(const SysDev* __restrict__ d) { take_snapshot(*d); }
 
 // U, sum v.v and W (6) of one system from the per-tile partial sums that the
 // energy variant of the force kernel wrote just before, in a fixed order: each thread
 // sums tiles t, t + THERMO_T, ... (four tiles in flight), then the warps by shuffles,
 // then the warps' sums in order.  FP64 additions of one SM bound it (16 cycles a warp
-// each): 48 readouts in a batch with 64 steps 17,380 us with
-// one shuffle tree a sum, 17,097 so
+// each): 48 readouts in a batch with 64 steps 17,380 us with one shuffle tree a sum,
+// 17,097 so
 constexpr int THERMO_T = 512;
 __global__ void __launch_bounds__(THERMO_T) k_thermo(const SysDev* __restrict__ sysv,
                                                      const Tile* __restrict__ tiles) {
@@ -46,21 +39,8 @@ __global__ void __launch_bounds__(THERMO_T) k_thermo(const SysDev* __restrict__ 
 #pragma unroll 4
   for (int k = threadIdx.x; k < s.tile_count_f; k += THERMO_T)
     for (int c = 0; c < 8; ++c) acc[c] += p[8 * (size_t)k + c];
-  // the eight sums over the warp together: at distance 16 each half keeps four of them, at 8
-  // two, at 4 one: 9 additions a lane where one sum after another takes 40
-  const int lane = threadIdx.x & 31;
-#pragma unroll
-  for (int o = 16, keep = 4; o >= 4; o >>= 1, keep >>= 1) {
-    const bool up = lane & o;
-#pragma unroll
-    for (int c = 0; c < keep; ++c) {
-      const double got = __shfl_xor_sync(0xffffffffu, up ? acc[c] : acc[c + keep], o);
-      acc[c] = (up ? acc[c + keep] : acc[c]) + got;
-    }
-  }
-  acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 2);
-  acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 1);
-  if ((lane & 3) == 0) sh[threadIdx.x >> 5][lane >> 2] = acc[0];   // 4 (bit 4) + 2 (bit 3) + bit 2
+  const double sum = warp_sum8(acc);
+  if ((threadIdx.x & 3) == 0) sh[threadIdx.x >> 5][(threadIdx.x & 31) >> 2] = sum;
   __syncthreads();
   if (threadIdx.x < 8) {
     double r = 0;

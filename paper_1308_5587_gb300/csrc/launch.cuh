@@ -71,11 +71,13 @@ enum { MODE_FORCE = 0, MODE_EV = 1, MODE_STEP = 2, MODE_NVT_A = 3 };
 // that a readout's forces are the step's): not the register-capped step kernel of one
 // lane a particle
 __host__ __device__ constexpr bool has_wide(int prec, int tpp) { return prec == GBMD_FP64 || tpp > 1; }
+enum { READ_FORCE = 1, READ_VEL = 2, READ_POS = 4, READ_IMAGE = 8 };   // rows of a readout
 struct StepArgs {
   int nsys = 0;             // systems of the group (decisions of the last block)
   int total_blocks = 0;     // blocks of all the step's force launches
   cudaGraphConditionalHandle cond = 0;   // the rebuild conditional of the step graph
   int use_cond = 0;
+  int readout = 0;          // MODE_FORCE: the READ_ bits of what to write out
 };
 // eval: the PairEval of every system of the launch
 KernelCall force_call(int prec, int multi, int mode, int tpp, int block, const SysDev* d,

@@ -21,6 +21,60 @@
 
 namespace gbmd {
 
+// one thread: the system's flags and thermostat into its Snapshot
+__device__ __forceinline__ void take_snapshot(const SysDev& s) {
+  Snapshot* o = reinterpret_cast<Snapshot*>(s.thermo);
+  const volatile long long* f = reinterpret_cast<const volatile long long*>(s.flags);
+  long long* to = reinterpret_cast<long long*>(&o->flags);
+  for (int k = 0; k < (int)(sizeof(Flags) / 8); ++k) to[k] = f[k];
+  for (int k = 0; k < 3; ++k) o->nh[k] = s.nh[k];
+}
+
+// The row of particle i in a readout, at its tag, in the staging behind the Snapshot:
+// force f, full-step velocity, position and image, as the bits of `what` ask
+__device__ __forceinline__ void read_out(const SysDev& s, int i, const double (&f)[3], int vfull,
+                                         int what) {
+  const size_t n = (size_t)s.n, tg = (size_t)s.tag[i];
+  double* const out = s.thermo + SNAPSHOT_BYTES / 8 + 3 * tg;
+  int* const image = reinterpret_cast<int*>(s.thermo + SNAPSHOT_BYTES / 8 + 9 * n) + 3 * tg;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    if (what & READ_FORCE) out[a] = f[a];
+    if (what & READ_VEL) {
+      double v = s.v[a * n + i];
+      if (!vfull) {
+        v = fma(s.h, f[a], v);
+        if (s.nvt) v *= s.nh[2];   // NVT: the closing thermostat scaling
+      }
+      out[3 * n + a] = v;
+    }
+    if (what & READ_POS) out[6 * n + a] = s.x[a * n + i] * (s.L[a] / 4294967296.0);
+    if (what & READ_IMAGE) image[a] = s.img[a * n + i];
+  }
+}
+
+// Eight values of every lane summed over the warp together: at distance 16 each half of
+// the warp keeps four of them, at 8 two, at 4 one -- 9 FP64 additions where one shuffle
+// tree after another takes 40.  Returns the sum of value lane / 4 to each four lanes.
+__device__ __forceinline__ double warp_sum8(const double (&in)[8]) {
+  const int lane = threadIdx.x & 31;
+  double acc[8];
+#pragma unroll
+  for (int c = 0; c < 8; ++c) acc[c] = in[c];
+#pragma unroll
+  for (int o = 16, keep = 4; o >= 4; o >>= 1, keep >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int c = 0; c < keep; ++c) {
+      const double got = __shfl_xor_sync(0xffffffffu, up ? acc[c] : acc[c + keep], o);
+      acc[c] = (up ? acc[c + keep] : acc[c]) + got;
+    }
+  }
+  acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 2);
+  acc[0] += __shfl_xor_sync(0xffffffffu, acc[0], 1);
+  return acc[0];
+}
+
 // float -> double, exactly, on the integer pipe.  Zero and subnormal inputs (a
 // force below 1.2e-38) give zero; inf / NaN set `bad`.
 __device__ __forceinline__ double widen_f32(float f, bool& bad) {

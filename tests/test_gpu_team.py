@@ -196,6 +196,31 @@ def test_batch_of_many_members_equals_alone(sizes):
         s.close()
 
 
+@pytest.mark.parametrize("name", ["n33", "n500_fp64_nvt", "n4097_grid_nvt", "tree_3000",
+                                  "n33001_fp64_one_lane"])
+def test_readouts_of_parts_equal_the_whole(name):
+    """Each array of a readout alone (positions without the force kernel) and in pairs, small
+    (one copy) and large, against the whole state."""
+    import ctypes
+    s = create(name)
+    s.step(7)
+    n = s.info()["n"]
+    pos, vel, image, step = s.state()
+    whole = {"pos": pos, "vel": vel, "image": image}
+    F = s.forces()
+    for parts in (["pos"], ["vel"], ["image"], ["pos", "image"], ["vel", "image"], ["pos", "vel"]):
+        got = {k: np.full_like(whole[k], -7) for k in parts}
+        at = ctypes.c_int64()
+        args = [got[k].ctypes.data_as(ctypes.c_void_p) if k in got else None
+                for k in ("pos", "vel", "image")]
+        assert gbmd.load().gbmd_get_state(s.handle, *args, ctypes.byref(at)) == 0
+        assert at.value == step and len(pos) == n
+        for k in parts:
+            assert np.array_equal(got[k], whole[k]), (parts, k)
+        assert np.array_equal(s.forces(), F)
+    s.close()
+
+
 @pytest.mark.parametrize("n", [2, 31, 33, 4095, 131072, 131073])
 @pytest.mark.parametrize("prec", ["mixed", "fp64"])
 def test_thermo_sums_at_the_edges_of_its_tiles(prec, n):
