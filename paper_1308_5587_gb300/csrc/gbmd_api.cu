@@ -269,6 +269,35 @@ void force_tiles(const SysDev& d, int sys, int prec, int tpp, int per, std::vect
   }
 }
 
+std::vector<int4> team_shares(const std::vector<int>& work, int sms);
+int team_cluster(int chunks, int per_block, int most);
+
+// Whether a batch's members of n[] particles go by the team: not where the shared launches
+// keep the chip busy anyway, and not as shares of the grid with too much on one block
+// (every member has at least one).  us a step by the shared graph / the team, replicas of
+// 500 to 20,000: 12 (32,000 particles) 90 / 32, 48 (315,000) 213 / 112, 96 (572,000) 293 /
+// 245, and with the fullest share 2.3 and 3.3 times the mean 128 (736,000) 351 / 424,
+// 152 (914,000) 364 / 797; more members than SMs, by clusters, 200 (1,241,000) 451 / 450,
+// 256 (1,543,000) 526 / 562.
+constexpr long long TEAM_BATCH_SUM = 655360;
+constexpr double TEAM_UNEVEN = 1.8;
+bool batch_by_team(const Group* g, const std::vector<int>& n) {
+  constexpr int SMS = TEAM_TURN_N / TEAM_T, WARPS = TEAM_T / 32, AT_ONCE = 8;   // clusters of 16
+  long long sum = 0;
+  int blocks = 0, largest = 0;
+  for (int k : n) {
+    const int c = team_cluster((int)(((long long)k * g->tpp + 31) / 32), WARPS, TEAM_MAX_CLUSTER);
+    sum += k;
+    blocks += c;
+    largest += c == TEAM_MAX_CLUSTER;
+  }
+  if (sum > TEAM_BATCH_SUM) return false;
+  if ((blocks <= SMS && largest <= AT_ONCE) || (int)n.size() > SMS) return true;
+  double most = 0;
+  for (const int4& s : team_shares(n, SMS)) most = std::max(most, (double)n[s.x] / s.z);
+  return most <= TEAM_T || most <= TEAM_UNEVEN * sum / SMS;   // one turn of a block's warps, or even
+}
+
 // Rebuild descriptor copies and tile tables for the group's current members.
 int sync_layout(Group* g) {
   if (!g->layout_dirty) return GBMD_OK;
@@ -286,6 +315,14 @@ int sync_layout(Group* g) {
       }
     }
   std::stable_sort(g->team.begin(), g->team.end(), [&](int a, int b) { return m[a]->h.n > m[b]->h.n; });
+  if (g->is_batch) {
+    std::vector<int> n;
+    for (int k : g->team) n.push_back(m[k]->h.n);
+    if (!batch_by_team(g, n)) {
+      g->team.clear();
+      g->team_max_n = 0;
+    }
+  }
   g->team_n.clear();
   for (int k : g->team) g->team_n.push_back(m[k]->h.n);
   g->share_dirty = true;
@@ -690,11 +727,11 @@ int team_cluster(int chunks, int per_block, int most) {
 }
 // shares of `sms` blocks for the team's members: one each, then the next always to the
 // member with the most work a block
-std::vector<int4> team_shares(const std::vector<int>& chunks, int sms) {
-  const int teams = (int)chunks.size();
+std::vector<int4> team_shares(const std::vector<int>& work, int sms) {
+  const int teams = (int)work.size();
   std::vector<int> blocks(teams, 1);
   auto less = [&](int a, int b) {   // work a block; the earlier of equals first
-    const long long x = (long long)chunks[a] * blocks[b], y = (long long)chunks[b] * blocks[a];
+    const long long x = (long long)work[a] * blocks[b], y = (long long)work[b] * blocks[a];
     return x != y ? x < y : a > b;
   };
   std::vector<int> heap(teams);
