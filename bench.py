@@ -484,7 +484,9 @@ def fp64_roofline(n, nbar, force_ms, peaks, r_cut, r_list):
     measured by the probe), r^-6 (2), the force factor (3) and the three
     accumulations (3); per particle the integration's kicks, drifts, rounding and
     FP64 shadow (13).  The share of listed pairs inside r_cut is the uniform-fluid
-    estimate (r_cut / r_list)^3."""
+    estimate (r_cut / r_list)^3.  The kernel does displacement, r^2, reciprocal and powers
+    in integer arithmetic rounded to FP64 once; they count here as the FP64 operations
+    they stand for."""
     rcp = peaks["drcp_in_dfma_slots"]
     f_cut = (r_cut / r_list) ** 3
     per_pair = f_cut * (14 + rcp)
