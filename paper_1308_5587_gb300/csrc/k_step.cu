@@ -303,7 +303,19 @@ static KernelCall mk(void* f, int grid, int block, size_t smem = 0) {
 cudaError_t launch(const KernelCall& k, cudaStream_t st) {
   void* a[10];
   args_of(k, a);
-  return cudaLaunchKernel(k.func, k.grid, k.block, a, k.smem, st);
+  if (!k.cooperative) return cudaLaunchKernel(k.func, k.grid, k.block, a, k.smem, st);
+  // its blocks wait for each other: all of them resident, whatever else is running
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = k.grid;
+  cfg.blockDim = k.block;
+  cfg.dynamicSmemBytes = k.smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeCooperative;
+  at.val.cooperative = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelExC(&cfg, k.func, a);
 }
 
 KernelCall thermo_call(const SysDev* d, const Tile* tiles_s, int nsys, GroupCtl*) {
