@@ -82,8 +82,10 @@ __global__ void __launch_bounds__(STAGED_BLOCK) k_force_staged(const SysDev* __r
   const int b = t.first;
   const int4 info = s.blk_info[b];          // (first member, particles, window total, 0)
   // an error (e.g. a window too large) leaves nothing valid, and a window is never
-  // indexed past its capacity; step mode also skips a system at its step limit
-  const bool run = fw.error == 0 && info.z <= s.window_cap && (!STEP || sl.y < 0 || sl.x < sl.y);
+  // indexed past its capacity; step mode also skips a system at its step limit.  Decided
+  // for the block: another block may set the error while this one's warps read it
+  const bool run = __syncthreads_and(fw.error == 0 && info.z <= s.window_cap &&
+                                     (!STEP || sl.y < 0 || sl.x < sl.y));
   bool need = false, bad = false;
   if (run) {
   const int4* __restrict__ qv = q_at(s, step);

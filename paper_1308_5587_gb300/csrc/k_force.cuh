@@ -452,7 +452,10 @@ __device__ __forceinline__ void force_body(const SysDev* __restrict__ sysv, cons
   if (MODE == MODE_FORCE && readout && threadIdx.x == 0 && blockIdx.x == 0) take_snapshot(s);
   const FlagWords fw = load_flag_words(s.flags);
   const longlong2 sl = load_flag_pair(&s.flags->step);   // (step, step_limit)
-  const bool active = !(STEP || NVTA) || (fw.error == 0 && (sl.y < 0 || sl.x < sl.y));   // uniform
+  // Another block of this launch may set the error in the meantime (step_tail), so the
+  // warps of a block may decide differently; a warp decides as one
+  const bool active =
+      !(STEP || NVTA) || __all_sync(0xffffffffu, fw.error == 0 && (sl.y < 0 || sl.x < sl.y));
   const long long step = sl.x;
   bool need = false, bad = false;
   double uu = 0.0;   // NVT: v.v after the closing half
@@ -474,6 +477,8 @@ __device__ __forceinline__ void force_body(const SysDev* __restrict__ sysv, cons
   const int g = threadIdx.x / TPP, h = threadIdx.x % TPP;
   const bool valid = g < t.count;
   const int i = t.first + (valid ? g : 0);
+  constexpr bool FULL_WARPS = STEP && PREC == GBMD_MIXED && TPP > 1;
+  __shared__ float4 fsh[FULL_WARPS ? 512 / TPP : 1];
   if (active) {
   const int n = valid ? s.nn[i] : 0;
   if (STEP && valid && h == 0) prefetch_particle(s, i);   // in flight during the gathers
@@ -491,21 +496,8 @@ __device__ __forceinline__ void force_body(const SysDev* __restrict__ sysv, cons
       E = group_sum<TPP>(e.x + e.y);
       for (int c = 0; c < 6; ++c) W[c] = group_sum<TPP>(w[c].x + w[c].y);
     }
-    if (STEP && TPP > 1) {
-      // the step needs no stored force.  The integration's FP64 instructions hold their
-      // pipe 16 cycles a warp however few lanes are active: the block's particles go to
-      // its first threads, in full warps (with readouts: N = 199,999, 30 steps 2,781 ->
-      // 2,692 us; WCA 1:10, N = 100,100, 40 steps 1,901 -> 1,793)
-      __shared__ float4 fsh[STEP ? 512 / TPP : 1];
+    if (FULL_WARPS) {   // the step needs no stored force
       if (h == 0) fsh[g] = make_float4(Fx, Fy, Fz, __int_as_float(qi.w));
-      __syncthreads();
-      if ((int)threadIdx.x < t.count) {
-        const int p = t.first + (int)threadIdx.x;
-        const float4 F = fsh[threadIdx.x];
-        const double f[3] = {widen_f32(F.x, bad), widen_f32(F.y, bad), widen_f32(F.z, bad)};
-        integrate_one<PREC>(s, p, __float_as_int(F.w), f, fw.v_full, load_particle(s, p),
-                            q_at(s, step + 1), nullptr, need, bad);
-      }
     } else if (STEP) {   // each lane integrates its particle
       if (valid && h == 0) {
         const double f[3] = {widen_f32(Fx, bad), widen_f32(Fy, bad), widen_f32(Fz, bad)};
@@ -576,6 +568,20 @@ __device__ __forceinline__ void force_body(const SysDev* __restrict__ sysv, cons
     }
   }
   }   // active
+  // The integration's FP64 instructions hold their pipe 16 cycles a warp however few lanes
+  // are active: the block's particles go to its first threads, in full warps (with
+  // readouts: N = 199,999, 30 steps 2,781 -> 2,692 us; WCA 1:10, N = 100,100, 40 steps
+  // 1,901 -> 1,793).  Every warp comes to this barrier, and unless all of them were active
+  // the block leaves its particles as they are.
+  if constexpr (FULL_WARPS) {
+    if (__syncthreads_and(active) && (int)threadIdx.x < t.count) {
+      const int p = t.first + (int)threadIdx.x;
+      const float4 F = fsh[threadIdx.x];
+      const double f[3] = {widen_f32(F.x, bad), widen_f32(F.y, bad), widen_f32(F.z, bad)};
+      integrate_one<GBMD_MIXED>(s, p, __float_as_int(F.w), f, fw.v_full, load_particle(s, p),
+                                q_at(s, step + 1), nullptr, need, bad);
+    }
+  }
   if (STEP) step_tail(s, sysv, ctl, nsys, total_blocks, cond, use_cond, need, bad);
   if (NVTA) {
     if (bad) atomicCAS(&s.flags->error, 0, (int)DEV_NONFINITE);

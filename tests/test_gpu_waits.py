@@ -1,5 +1,6 @@
 """Kernels whose blocks wait for each other: systems on different streams and threads at the
-same time."""
+same time; and launches of many waves in which an early block ends the run, so that warps
+of later blocks find the system frozen."""
 import threading
 
 import numpy as np
@@ -48,3 +49,37 @@ def test_systems_on_streams_of_their_own_equal_one_after_another(n):
         for a, b in zip(g, e):
             for x, y in zip(a, b):
                 assert np.array_equal(x, y)
+
+
+def overlapping_at_the_corner(w):
+    """Two particles of one type at one place, at the start of the sort order: blocks of the
+    first wave find the non-finite force."""
+    a = int(np.argmin((w.pos + 0.5 * w.box).sum(1)))
+    d = w.pos - w.pos[a]
+    d -= w.box * np.rint(d / w.box)
+    r2 = np.where(w.types == w.types[a], (d * d).sum(1), np.inf)
+    r2[a] = np.inf
+    pos = w.pos.copy()
+    pos[int(np.argmin(r2))] = pos[a]
+    return pos
+
+
+@pytest.mark.parametrize("name,kw", [
+    ("lj", {"threads_per_particle": 2}), ("lj", {"threads_per_particle": 4}),
+    ("lj", {"threads_per_particle": 1}), ("lj", {"precision": "fp64"}),
+    ("lj", {"integrator": "nvt", "kT": 1.2, "tau": 0.5}), ("lj", {"force_path": "staged"}),
+    ("colloid", {"nlist": "tree"})])
+def test_a_launch_of_many_waves_ends_when_an_early_block_finds_a_non_finite_force(name, kw):
+    """Step kernels (no team at these sizes), hundreds to thousands of blocks."""
+    w = wl.lj_fluid(120_000, 0.84, 1.2, seed=710) if name == "lj" else \
+        wl.colloid_mixture(100_000, ratio=10.0, seed=711)
+    s = gbmd.System.from_workload(w, **kw)
+    s.step(2)
+    s.sync()
+    s.set_state(overlapping_at_the_corner(w), w.vel)
+    for _ in range(2):
+        s.step(3)
+        with pytest.raises(gbmd.GbmdError) as e:
+            s.sync()
+        assert e.value.status == "NONFINITE"
+    s.close()
