@@ -266,7 +266,10 @@ __device__ __forceinline__ int nlist_cell(const SysDev& s, int r, WarpRing<STAGE
         cnt += 4;
       }
       const int left = c & 3;
-      const int j0 = at[0], j1 = at[32], j2 = at[64];   // in the buffer, perhaps unused
+      int j0 = 0, j1 = 0, j2 = 0;   // a full buffer ends behind its last slot: read what is left
+      if (left > 0) j0 = at[0];
+      if (left > 1) j1 = at[32];
+      if (left > 2) j2 = at[64];
       if (last) {
         if (left && cnt < cap)
           *row = make_int4(j0, left > 1 ? j1 : j0, left > 2 ? j2 : j0, j0);
