@@ -59,7 +59,8 @@ typedef enum gbmd_status {
     GBMD_ERR_NLIST_OVERFLOW = -4,   /* neighbour list overflow that could not be recovered */
     GBMD_ERR_NONFINITE = -5,        /* a coordinate became NaN/Inf, or moved > L/2 in a step */
     GBMD_ERR_CUDA = -6,             /* a CUDA runtime call failed */
-    GBMD_ERR_TIMEOUT = -7,          /* a bounded wait ran out */
+    GBMD_ERR_TIMEOUT = -7,          /* a bounded wait ran out: the system cannot be stepped or
+                                       given a new state any more, only destroyed */
     GBMD_ERR_STATE = -8,            /* call not valid in the current state (e.g. in a batch) */
     GBMD_ERR_NO_DEVICE = -9         /* no usable CUDA device */
 } gbmd_status;
@@ -233,7 +234,7 @@ typedef struct gbmd_batch gbmd_batch;
 
 /* Create a system from HOST arrays: uploads, wraps, builds the cell and
  * neighbour lists and computes the initial forces.  *out receives the handle.
- * Errors: BAD_ARG, BOX_TOO_SMALL, OOM, CUDA, NO_DEVICE. */
+ * Errors: BAD_ARG, BOX_TOO_SMALL, OOM, CUDA, NO_DEVICE, TIMEOUT. */
 int gbmd_create(const gbmd_desc *d, gbmd_system **out);
 
 /* As gbmd_create, but pos, vel, type and image are DEVICE pointers (same

@@ -146,6 +146,7 @@ struct Group {
   size_t cap_share = 0, cap_sync = 0;
   std::vector<int> team_n;             // their particles
   int team_max_n = 0;
+  int polls = TEAM_POLLS;
   cudaStream_t side[TEAM_SIDES] = {};
   cudaEvent_t side_ev[TEAM_SIDES + 1] = {};
   Group* rest = nullptr;
@@ -302,6 +303,9 @@ bool batch_by_team(const Group* g, const std::vector<int>& n) {
 int sync_layout(Group* g) {
   if (!g->layout_dirty) return GBMD_OK;
   std::vector<gbmd_system*> m = live(g);
+  g->polls = TEAM_POLLS;
+  // a test lets the waits run out
+  if (const char* ev = getenv("GBMD_TEAM_POLLS")) g->polls = std::max(0, atoi(ev));
   g->team.clear();
   g->team_max_n = 0;
   std::vector<gbmd_system*> others;
@@ -421,6 +425,10 @@ int sync_layout(Group* g) {
     CK(cudaMalloc(&g->d_ctl, sizeof(GroupCtl)));
     CK(cudaMemsetAsync(g->d_ctl, 0, sizeof(GroupCtl), g->stream));
   }
+  // a wait that was given up leaves arrivals behind.  Its system stays stopped, so nothing
+  // meets them before the group's members change, which comes through here
+  CK(cudaMemsetAsync(&g->d_ctl->team, 0, sizeof(TeamSync), g->stream));
+  if (g->d_sync) CK(cudaMemsetAsync(g->d_sync, 0, g->cap_sync * sizeof(TeamSync), g->stream));
   auto up = [&](void* dst, const std::vector<Tile>& v) -> cudaError_t {
     if (v.empty()) return cudaSuccess;
     return cudaMemcpyAsync(dst, v.data(), v.size() * sizeof(Tile), cudaMemcpyHostToDevice, g->stream);
@@ -594,7 +602,7 @@ int coop_rebuild(const Group* g, KernelCall* out) {
   TeamFit fit;
   RET(team_fit(rebuild_func(g->multi > 0), REBUILD_T, REBUILD_SMEM, g->device, &fit));
   if (fit.blocks_per_sm < 1) return GBMD_OK;
-  *out = rebuild_call(g->d_desc, fit.sms, g->d_ctl, g->multi > 0);
+  *out = rebuild_call(g->d_desc, fit.sms, g->d_ctl, g->multi > 0, g->polls);
   return GBMD_OK;
 }
 
@@ -769,6 +777,7 @@ int launch_team(Group* g, long long n) {
   TeamArgs a{};
   a.desc = g->d_desc;
   a.ctl = g->d_ctl;
+  a.polls = g->polls;
   cudaLaunchConfig_t cfg{};
   cfg.blockDim = dim3(TEAM_T);
   cfg.dynamicSmemBytes = TEAM_SMEM;
@@ -949,14 +958,26 @@ int grow_nlist(gbmd_system* s, int need) {
   return refresh_desc(s);
 }
 
+// the errors that nothing recovers from.  After DEV_TEAM the bins' counts and, in a
+// re-sort, the particles' order may be half written, so that not even a new state (which
+// keeps the types) can be taken
+int stopped(const Flags& f) {
+  if (f.error == DEV_NONFINITE)
+    return fail(GBMD_ERR_NONFINITE, "non-finite coordinate or a particle moved more than L/2 in one step (step %lld)", f.step);
+  if (f.error == DEV_TEAM)
+    return fail(GBMD_ERR_TIMEOUT, "a wait between thread blocks ran out (step %lld)", f.step);
+  if (f.error == DEV_TREE)
+    return fail(GBMD_ERR_TIMEOUT, "a tree traversal passed its node bound (step %lld)", f.step);
+  return GBMD_OK;
+}
+
 // Wait for the system's work; recover from overflow; run what remains of its steps.
 int sync_system(gbmd_system* s) {
   cudaStream_t st = cur_stream(s);
   for (int round = 0; round < 64; ++round) {
     Flags f;
     RET(read_flags(s, &f, st));   // waits for the stream
-    if (f.error == DEV_NONFINITE)
-      return fail(GBMD_ERR_NONFINITE, "non-finite coordinate or a particle moved more than L/2 in one step (step %lld)", f.step);
+    RET(stopped(f));
     if (f.error == DEV_WINDOW) {   // a staged window outgrew shared memory
       s->h.staged = 0;
       RET(refresh_desc(s));
@@ -976,17 +997,6 @@ int sync_system(gbmd_system* s) {
       RET(rebuild_and_force(s, 0));   // finishes the interrupted step
       continue;
     }
-    if (f.error == DEV_TEAM) {   // arrivals may be left over: the next launch starts clean
-      for (Group* g : {s->own, s->batch})
-        if (g && g->d_ctl)
-          CK(cudaMemsetAsync(&g->d_ctl->team.arrive, 0, sizeof(g->d_ctl->team.arrive), g->stream));
-      if (s->batch && s->batch->d_sync)
-        CK(cudaMemsetAsync(s->batch->d_sync, 0, s->batch->cap_sync * sizeof(TeamSync), s->batch->stream));
-      CK(cudaStreamSynchronize(st));
-      return fail(GBMD_ERR_TIMEOUT, "a wait between thread blocks ran out (step %lld)", f.step);
-    }
-    if (f.error == DEV_TREE)
-      return fail(GBMD_ERR_TIMEOUT, "a tree traversal passed its node bound (step %lld)", f.step);
     if (f.error) return fail(GBMD_ERR_CUDA, "unknown device error %d", f.error);
     long long want = s->target_step;
     if (s->step_limit >= 0) want = std::min(want, s->step_limit);
@@ -1532,6 +1542,7 @@ int load_state(gbmd_system* s, const double* pos, const double* vel, const int32
   Flags after = snap.flags;
   if (after.error == DEV_BADTYPE) return fail(GBMD_ERR_BAD_ARG, "type id out of range in the device type array");
   s->target_step = step;
+  RET(stopped(after));
   if (after.error == DEV_WINDOW) {
     s->h.staged = 0;
     RET(refresh_desc(s));
@@ -1540,6 +1551,7 @@ int load_state(gbmd_system* s, const double* pos, const double* vel, const int32
     RET(write_flags(s, &after, st));
     RET(rebuild_and_force(s, 0));
     RET(read_flags(s, &after, st));
+    RET(stopped(after));
   }
   if (after.error == DEV_OVERFLOW) {
     RET(grow_nlist(s, after.overflow_need));
@@ -1549,6 +1561,7 @@ int load_state(gbmd_system* s, const double* pos, const double* vel, const int32
     RET(write_flags(s, &after, st));
     RET(rebuild_and_force(s, 0));
     RET(read_flags(s, &after, st));
+    RET(stopped(after));
     if (after.error) return fail(GBMD_ERR_NLIST_OVERFLOW, "neighbour list overflow at creation");
   }
   return GBMD_OK;
@@ -1734,6 +1747,7 @@ int regrid(gbmd_system* s, double scale) {
   }
   Flags f;
   RET(read_flags(s, &f, st));
+  RET(stopped(f));
   if (f.error) return fail(GBMD_ERR_STATE, "device error %d after a new cell grid", f.error);
   f.do_rebuild = 0;
   f.do_sort = 0;
@@ -1770,6 +1784,7 @@ int time_rebuild(Group* g, float* ms) {
   for (auto* s : m) {   // the lists stand for the current positions
     Flags f;
     RET(read_flags(s, &f, g->stream));
+    RET(stopped(f));
     if (f.error) return fail(GBMD_ERR_STATE, "device error %d while timing a rebuild", f.error);
     f.do_rebuild = 0;
     RET(write_flags(s, &f, g->stream));

@@ -19,7 +19,6 @@
 
 namespace gbmd {
 
-constexpr int TEAM_SPIN = 1 << 22;   // polls of ~0.5 us: two seconds
 enum : unsigned { VOTE_NEED = 1u, VOTE_BAD = 2u, VOTE_LOST = 4u };
 
 // The team's cell sort takes buckets: the histogram's atomic places each particle in its
@@ -50,6 +49,7 @@ struct Team {
   int par;                   // cluster: which vote slots are in use
   unsigned* slot;            // [2][TEAM_MAX_CLUSTER] in shared memory
   unsigned* word;            // one word in shared memory
+  int polls;                 // grid: of a wait, at most
 
   // Every thread of every block of the team: all of them have arrived, what they wrote
   // is visible, and the votes are ORed (VOTE_LOST: a wait ran out; the team stops).
@@ -85,7 +85,7 @@ struct Team {
         asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(&sync->release), "l"(rel) : "memory");
       } else {
         out = VOTE_LOST;
-        for (int k = 0; k < TEAM_SPIN; ++k) {
+        for (int k = 0; k < polls; ++k) {
           unsigned long long rel;
           asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(rel) : "l"(&sync->release) : "memory");
           if ((unsigned)(rel >> 8) == gen + 1u) {
