@@ -342,10 +342,13 @@ int64_t gbmd_footprint_bytes(const gbmd_desc *d);
 int gbmd_set_step_limit(gbmd_system *s, int64_t step);
 
 /* Autotuner (Section 5: kernel parameters are tuned on the device at run time).
- * Chooses, by timing the candidates on this system's current state: the cell
- * width (a list rebuild at cells of 1, 1.1, 1.2 and 1.35 times r_list,max; kept
- * at 1 on the staged force path), then the force kernel's threads per particle
- * (1, 2, 4) and block size (128, 256, 512).  With a non-NULL cache_path the
+ * Chooses, by timing the candidates from this system's current state: the cell
+ * width (cells of 1, 1.1, 1.2 and 1.35 times r_list,max; kept at 1 on the staged
+ * force path), then the force kernel's threads per particle (1, 2, 4) and block
+ * size (128, 256, 512; FP64 also 64).  A system small enough that resident blocks
+ * may run its steps is timed over real steps: its memory is copied aside and put
+ * back, so that it is where it was (without room for the copy, and for the others,
+ * the rebuild and the force kernel are timed).  With a non-NULL cache_path the
  * choice is read from / appended to that text file (one line per shape: key,
  * threads per particle, block, cell scale), keyed by device, precision, type
  * mode, size and density class. */

@@ -75,7 +75,7 @@ struct gbmd_system {
   SysDev h{};                 // master descriptor (device pointers)
   Flags* d_flags = nullptr;
   cudaStream_t stream = nullptr;     // the caller's stream
-  std::vector<void*> allocs;
+  std::map<void*, size_t> allocs;   // device memory and its bytes
   size_t footprint = 0;
   Group* own = nullptr;       // the system alone
   Group* batch = nullptr;
@@ -937,21 +937,25 @@ int dalloc(gbmd_system* s, void** p, size_t bytes) {
   bytes = std::max<size_t>(bytes, 16);
   cudaError_t e = cudaMalloc(p, bytes);
   if (e != cudaSuccess) return fail(GBMD_ERR_OOM, "cudaMalloc(%zu) failed: %s", bytes, cudaGetErrorString(e));
-  s->allocs.push_back(*p);
+  s->allocs[*p] = bytes;
   s->footprint += bytes;
   return GBMD_OK;
+}
+
+void dfree(gbmd_system* s, void* p) {
+  auto it = s->allocs.find(p);
+  if (it != s->allocs.end()) {
+    s->footprint -= it->second;
+    s->allocs.erase(it);
+  }
+  cudaFree(p);
 }
 
 // Grow the neighbour list to hold `need` neighbours per particle.
 int grow_nlist(gbmd_system* s, int need) {
   const int cap = (int)round_up((size_t)need + need / 4 + 8, 8);
   CK(cudaStreamSynchronize(cur_stream(s)));
-  auto it = std::find(s->allocs.begin(), s->allocs.end(), (void*)s->h.nl);
-  if (it != s->allocs.end()) {
-    s->allocs.erase(it);
-    s->footprint -= (size_t)s->h.nl_stride * s->h.cap * sizeof(int);
-  }
-  CK(cudaFree(s->h.nl));
+  dfree(s, s->h.nl);
   s->h.nl = nullptr;
   RET(dalloc(s, (void**)&s->h.nl, (size_t)s->h.nl_stride * cap * sizeof(int)));
   s->h.cap = cap;
@@ -1236,27 +1240,16 @@ bool staged_ok(const SysDev& h, const int nc[3]) {
          WIN_CELLS * per_cell * 1.35 + 96 <= STAGED_WINDOW_CAP;
 }
 
-void dfree(gbmd_system* s, void* p, size_t bytes) {
-  if (!p) return;
-  auto it = std::find(s->allocs.begin(), s->allocs.end(), p);
-  if (it != s->allocs.end()) {
-    s->allocs.erase(it);
-    s->footprint -= std::max<size_t>(bytes, 16);
-  }
-  cudaFree(p);
-}
-
 // The cell grid: nc cells per axis, the arrays sized by the cell count and the
 // Morton rank of every cell.  Replaces an existing grid (its arrays are freed).
 int setup_cells(gbmd_system* s, const int nc[3], cudaStream_t st) {
   SysDev& h = s->h;
   CK(cudaStreamSynchronize(st));
   if (h.cell_cnt) {
-    const size_t oc = (size_t)h.ncells, ob = (size_t)h.nblocks, obins = (size_t)h.nbins;
-    dfree(s, h.cell_cnt, (obins + 1) * 4); dfree(s, h.cell_start, (obins + 1) * 4);
-    dfree(s, h.cell_cursor, (obins + 1) * 4);
-    dfree(s, const_cast<int*>(h.rank2lin), oc * 4); dfree(s, const_cast<int*>(h.lin2rank), oc * 4);
-    dfree(s, h.blk_win, ob * WIN_CELLS * sizeof(int2)); dfree(s, h.blk_info, ob * sizeof(int4));
+    for (void* p : {(void*)h.cell_cnt, (void*)h.cell_start, (void*)h.cell_cursor,
+                    (void*)const_cast<int*>(h.rank2lin), (void*)const_cast<int*>(h.lin2rank),
+                    (void*)h.blk_win, (void*)h.blk_info})
+      dfree(s, p);
     h.cell_cnt = h.cell_start = h.cell_cursor = nullptr;
     h.rank2lin = h.lin2rank = nullptr;
     h.blk_win = nullptr;
@@ -1754,7 +1747,72 @@ int regrid(gbmd_system* s, double scale) {
   return write_flags(s, &f, st);
 }
 
-// Mean time of one full list rebuild (no re-sort) of every member of the group.
+// Mean time of a step, rebuilds included, as gbmd_step / gbmd_batch_step would run it: the
+// members' memory is copied aside, steps run, and all of it is put back.  *ms < 0: no room
+// for the copy.
+int time_steps(Group* g, float* ms) {
+  *ms = -1.f;
+  RET(sync_layout(g));
+  std::vector<gbmd_system*> m = live(g);
+  size_t bytes = 0;
+  auto step256 = [](size_t b) { return (b + 255) / 256 * 256; };
+  for (auto* s : m)
+    for (const auto& a : s->allocs) bytes += step256(a.second);
+  char* aside = nullptr;
+  if (cudaMalloc(&aside, bytes) != cudaSuccess) {
+    cudaGetLastError();
+    return GBMD_OK;
+  }
+  auto copy = [&](bool back) -> int {
+    char* at = aside;
+    for (auto* s : m)
+      for (const auto& a : s->allocs) {
+        CK(cudaMemcpyAsync(back ? a.first : at, back ? at : a.first, a.second, cudaMemcpyDeviceToDevice, g->stream));
+        at += step256(a.second);
+      }
+    return GBMD_OK;
+  };
+  auto run = [&]() -> int {
+    cudaEvent_t a, b;
+    CK(cudaEventCreate(&a));
+    CK(cudaEventCreate(&b));
+    for (auto* s : m) {   // also where a limit holds the system
+      Flags f;
+      RET(read_flags(s, &f, g->stream));
+      f.step_limit = -1;
+      RET(write_flags(s, &f, g->stream));
+    }
+    constexpr int WARM = 16, STEPS = 64;
+    RET(enqueue_steps(g, WARM));
+    CK(cudaEventRecord(a, g->stream));
+    RET(enqueue_steps(g, STEPS));
+    CK(cudaEventRecord(b, g->stream));
+    CK(cudaEventSynchronize(b));
+    float t = 0;
+    CK(cudaEventElapsedTime(&t, a, b));
+    cudaEventDestroy(a);
+    cudaEventDestroy(b);
+    *ms = t / STEPS;
+    for (auto* s : m) {   // a system that stopped (a list that overflowed) was not timed
+      Flags f;
+      RET(read_flags(s, &f, g->stream));
+      if (f.error) *ms = 1e30f;
+    }
+    return GBMD_OK;
+  };
+  int rc = copy(false);
+  if (rc == GBMD_OK) {
+    rc = run();
+    const int rb = copy(true);
+    if (rc == GBMD_OK) rc = rb;
+  }
+  cudaStreamSynchronize(g->stream);
+  cudaFree(aside);
+  return rc;
+}
+
+// Mean time of one full list rebuild (no re-sort) of every member of the group, by the
+// kernels that the step graph takes.
 int time_rebuild(Group* g, float* ms) {
   RET(sync_layout(g));
   std::vector<gbmd_system*> m = live(g);
@@ -1765,7 +1823,11 @@ int time_rebuild(Group* g, float* ms) {
     f.do_sort = 0;
     RET(write_flags(s, &f, g->stream));
   }
-  const std::vector<KernelCall> calls = rebuild_calls(g);
+  std::vector<KernelCall> calls = rebuild_calls(g);
+  KernelCall coop;
+  coop.func = nullptr;
+  if (g->use_graphs) RET(coop_rebuild(g, &coop));
+  if (coop.func) calls = {coop};
   cudaEvent_t a, b;
   CK(cudaEventCreate(&a));
   CK(cudaEventCreate(&b));
@@ -1849,6 +1911,24 @@ int autotune_group(Group* g, const char* cache) {
       return set_tuning(g, bt, bb);
     }
   }
+  // Where the team would step some member at one of the lane counts, what counts is the
+  // step itself: the lanes that suit the step kernel need not suit the team, and may be too
+  // many for it (team_member).  us a step by default / chosen by the step kernel's time /
+  // by the step's: mixed N = 20,000 14.8 / 18.6 / 14.9, FP64 40,000 65.4 / 77.7 / 65.5,
+  // FP64 64,000 82.6 / 92.1 / 82.6, 16 replicas of 2,000 30.8 / 20.3 / 20.0.  Otherwise the
+  // step kernel and the rebuild are timed.
+  const int tpp0 = g->tpp, block0 = g->fblock;
+  bool by_steps = false;
+  for (int tpp : {1, 2, 4}) {
+    RET(set_tuning(g, tpp, block0));
+    by_steps |= !g->team.empty();
+  }
+  RET(set_tuning(g, tpp0, block0));
+  if (by_steps) {
+    float ms;
+    RET(time_steps(g, &ms));
+    by_steps = ms >= 0.f;
+  }
   // cell width: the list rebuild at each candidate width (the global force path does
   // not depend on it); a wider cell only wins if it is clearly faster
   double best_s = 1.0;
@@ -1866,8 +1946,10 @@ int autotune_group(Group* g, const char* cache) {
         seen.push_back(grid);
         for (auto* s : live(g)) RET(regrid(s, sc));
         float ms;
-        RET(time_rebuild(g, &ms));
-        if (getenv("GBMD_VERBOSE")) fprintf(stderr, "gbmd autotune %s cell_scale=%.2f rebuild %.4f ms\n", key.c_str(), sc, ms);
+        if (by_steps) RET(time_steps(g, &ms));
+        else RET(time_rebuild(g, &ms));
+        if (by_steps && ms < 0.f) continue;
+        if (getenv("GBMD_VERBOSE")) fprintf(stderr, "gbmd autotune %s cell_scale=%.2f %s %.4f ms\n", key.c_str(), sc, by_steps ? "step" : "rebuild", ms);
         if (ms < 0.97f * best_r) { best_r = ms; best_s = sc; }
       }
       for (auto* s : live(g)) RET(regrid(s, best_s));
@@ -1877,15 +1959,34 @@ int autotune_group(Group* g, const char* cache) {
   float best = 1e30f;
   // FP64 also tries 64-thread blocks (its best step shape from 32k particles on)
   const bool fp64 = g->precision == GBMD_FP64;
+  auto tried = [&](int tpp, int block, const char* what, float ms) {
+    if (getenv("GBMD_VERBOSE")) fprintf(stderr, "gbmd autotune %s tpp=%d block=%d %s %.4f ms\n", key.c_str(), tpp, block, what, ms);
+  };
+  bool readouts_only = false;   // the best lanes' block size serves readouts alone
   for (int tpp : {1, 2, 4})
     for (int block : {64, 128, 256, 512}) {
       if (block == 64 && !fp64) continue;
       RET(set_tuning(g, tpp, block));
       float ms;
-      RET(time_force(g, &ms));
-      if (getenv("GBMD_VERBOSE")) fprintf(stderr, "gbmd autotune %s tpp=%d block=%d %.4f ms\n", key.c_str(), tpp, block, ms);
-      if (ms < best) { best = ms; best_t = tpp; best_b = block; }
+      if (by_steps) RET(time_steps(g, &ms));
+      else RET(time_force(g, &ms));
+      if (ms < 0.f) continue;
+      tried(tpp, block, by_steps ? "step" : "force", ms);
+      const bool whole = by_steps && g->team.size() == live(g).size();   // team.size() > 0
+      if (ms < best) { best = ms; best_t = tpp; best_b = block; readouts_only = whole; }
+      if (whole) break;   // the team's blocks are its own: every block size is the same
     }
+  if (readouts_only) {
+    best = 1e30f;
+    for (int block : {64, 128, 256, 512}) {
+      if (block == 64 && !fp64) continue;
+      RET(set_tuning(g, best_t, block));
+      float ms;
+      RET(time_force(g, &ms));
+      tried(best_t, block, "force", ms);
+      if (ms < best) { best = ms; best_b = block; }
+    }
+  }
   RET(set_tuning(g, best_t, best_b));
   if (cache) {
     std::ofstream o(cache, std::ios::app);
@@ -1951,7 +2052,7 @@ int gbmd_destroy(gbmd_system* s) {
     s->batch = nullptr;
   }
   if (s->own) cudaStreamSynchronize(s->own->stream);
-  for (void* p : s->allocs) cudaFree(p);
+  for (const auto& p : s->allocs) cudaFree(p.first);
   if (s->own) {
     free_group(s->own);
   }
