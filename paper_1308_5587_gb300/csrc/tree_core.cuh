@@ -114,7 +114,8 @@ GBMD_HD int tree_leaves(int n) {
 // Visit every leaf of the tree (boxes[1 .. 2P - 1], leaves at P .. 2P - 1) whose box
 // lies within sqrt(r2) of the point: visit(leaf index b) for leaf node P + b.  At
 // most max_nodes nodes are examined; returns the number examined, or -1 when that
-// limit cut the traversal short.
+// limit cut the traversal short.  The plain form, for one point and one thread, that the
+// host checks the boxes with; the kernels query for a group by one warp (tree_rows.cuh).
 template <class Visit>
 GBMD_HD int tree_query(const TreeBox* boxes, int P, uint32_t ux, uint32_t uy, uint32_t uz,
                        float fs0, float fs1, float fs2, float r2, int max_nodes,
