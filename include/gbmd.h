@@ -375,7 +375,10 @@ int gbmd_set_tuning(gbmd_system *s, int32_t threads_per_particle, int32_t block)
  * records of two CUDA events (cudaEvent_t, created by the caller with timing
  * enabled), so the caller can time that kernel inside real steps; may be called
  * between steps with new events (the step graph is updated, not rebuilt).
- * NULL, NULL removes the records.  Multi-step calls are unaffected. */
+ * NULL, NULL removes the records.  Calls of more steps are unaffected.  A system
+ * small enough that resident blocks run its steps (force and integration in one
+ * kernel, which no record can divide) takes the step kernel of the larger systems
+ * for these single steps: the same results, other times. */
 int gbmd_set_force_events(gbmd_system *s, void *ev_begin, void *ev_end);
 
 /* ---- many systems stepped together ------------------------------------------ */

@@ -863,12 +863,13 @@ int launch_team(Group* g, long long n) {
   return GBMD_OK;
 }
 
-// enqueue n steps of the group: by the team kernel, and (members it does not take; event
-// records around the force kernel; graphs switched off) graphs or direct launches
+// enqueue n steps of the group: by the team kernel, and (members it does not take; a single
+// step with event records around its force kernel; graphs switched off) graphs or direct
+// launches
 int enqueue_steps(Group* g, long long n) {
   if (n <= 0 || live(g).empty()) return GBMD_OK;
   RET(sync_layout(g));
-  if (!g->team.empty() && !(g->ev_begin && g->ev_end)) {
+  if (!g->team.empty() && !(n == 1 && g->ev_begin && g->ev_end)) {
     RET(launch_team(g, n));
     return g->rest ? enqueue_steps(g->rest, n) : GBMD_OK;
   }
