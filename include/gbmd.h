@@ -268,13 +268,13 @@ int gbmd_get_thermo(gbmd_system *s, gbmd_thermo *out);
  * is an error.  The paper has no counterpart; it is part of this library's API
  * only.  It runs the same energy/virial kernels as gbmd_get_thermo, but their
  * per-tile partial sums and the system descriptor they read live in static
- * device arrays of this library (2 MiB + one descriptor, held on every device
+ * device arrays of this library (8 MiB + one descriptor, held on every device
  * that loads the library until the process exits) instead of in buffers the
  * library allocates.  Limits and behaviour:
- *   - systems with more than GBMD_NOALLOC_MAX_TILES energy tiles are rejected
- *     with GBMD_ERR_BAD_ARG: one tile is 128 particles on the global force path
- *     (so at most 4,194,304 particles) and one 2x2x2 block of cells on the
- *     staged path;
+ *   - systems with more than 128 GBMD_NOALLOC_MAX_TILES = 4,194,304 particles on
+ *     the global force path, or more than GBMD_NOALLOC_MAX_TILES energy tiles
+ *     (2x2x2 blocks of cells) on the staged path, are rejected with
+ *     GBMD_ERR_BAD_ARG;
  *   - the first call on a device looks up the static arrays' device addresses
  *     (cudaGetSymbolAddress), once; make that first call before any stream
  *     capture begins;

@@ -2504,10 +2504,15 @@ int gbmd_batch_destroy(gbmd_batch* bh) {
 // ============================================================================
 namespace {
 
+// The limit is in tiles of EV_TILE_P particles.  A tree list's wide types (force_tiles) take
+// more: each holds at most n / 32 particles, and a wide tile as few as EV_TILE_P / 32 of
+// them (one lane a particle), so up to as many tiles again as the whole system for each
+// type but the one that is not wide, and a partial one a type
 constexpr int kNoallocMaxTiles = GBMD_NOALLOC_MAX_TILES;
+constexpr int kNoallocTiles = MAXT * (kNoallocMaxTiles + 2);
 constexpr int kNoallocMaxDevices = 64;
 
-static __device__ __align__(256) double g_noalloc_partials[8 * kNoallocMaxTiles];   // 2 MiB
+static __device__ __align__(256) double g_noalloc_partials[8 * kNoallocTiles];   // 8 MiB
 static __device__ __align__(256) SysDev g_noalloc_desc;
 
 struct NoallocAddrs {
@@ -2556,9 +2561,10 @@ extern "C" int gbmd_get_thermo_noalloc(gbmd_system* s, gbmd_thermo* out) {
   if (s->step_limit >= 0) want = std::min(want, s->step_limit);
   if (f.step < want) return fail(GBMD_ERR_STATE, "steps still owed after a recovery: call gbmd_sync first");
   if (g->layout_dirty) return fail(GBMD_ERR_STATE, "layout changed: call gbmd_sync or gbmd_get_thermo first");
-  if (g->nte + g->ntb > kNoallocMaxTiles)
+  const int tiles = g->ntb > 0 ? g->ntb : (s->h.n + EV_TILE_P - 1) / EV_TILE_P;
+  if (tiles > kNoallocMaxTiles || g->nte + g->ntb > kNoallocTiles)
     return fail(GBMD_ERR_BAD_ARG, "%d energy tiles exceed the allocation-free limit of %d",
-                g->nte + g->ntb, kNoallocMaxTiles);
+                tiles, kNoallocMaxTiles);
   // the system's descriptor, pointed at the static partials (own group: tiles from 0)
   SysDev d = s->h;
   d.tile_first_f = 0;

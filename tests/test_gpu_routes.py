@@ -1,4 +1,5 @@
 """Which kernels run a call: seen by the launches that the library counts."""
+import numpy as np
 import pytest
 
 from paper_1308_5587_gb300 import gbmd, workloads as wl
@@ -40,3 +41,24 @@ def test_event_records_leave_calls_of_many_steps_as_they_are(prec):
     s.set_force_events(None, None)
     assert launches(1) == 1
     s.close()
+
+
+def test_noalloc_thermo_of_a_tree_list_whose_wide_types_take_many_tiles():
+    """2,197,000 particles, fewer than the 4,194,304 of the header, whose 66,575 far-reaching
+    ones take four to an energy tile: 33,288 tiles."""
+    m = 130
+    g = np.arange(m) - 0.5 * (m - 1)
+    rng = np.random.default_rng(760)
+    pos = np.stack(np.meshgrid(g, g, g, indexing="ij"), -1).reshape(-1, 3)
+    pos += rng.uniform(-0.05, 0.05, pos.shape)
+    types = np.zeros(len(pos), np.int32)
+    types[rng.permutation(len(pos))[:len(pos) // 33]] = 1
+    rcut = np.array([[0.9, 2.4], [2.4, 2.4]])   # one type without neighbours, one with ~90
+    pairs = wl.PairTable(np.full((2, 2), 0.1), np.full((2, 2), 0.9), rcut)
+    w = wl.Workload(pos, np.zeros_like(pos), types, np.full(3, float(m)), pairs, r_buff=0.4)
+    s = gbmd.System.from_workload(w, precision="fp64", nlist="tree", threads_per_particle=1)
+    t = gbmd.gbmd_get_thermo_noalloc(s.handle)
+    ref = gbmd.gbmd_get_thermo(s.handle)
+    assert t["pe"] == ref["pe"] < 0.0 and t["virial"] == ref["virial"]
+    s.close()
+
