@@ -2467,12 +2467,14 @@ int gbmd_batch_info(gbmd_batch* bh, int32_t* members, int64_t* particles, int64_
     *particles = np;
   }
   if (launches) {
-    GroupCtl c{};
-    if (b->d_ctl) {
-      CK(cudaMemcpyAsync(&c, b->d_ctl, sizeof(c), cudaMemcpyDeviceToHost, b->stream));
+    *launches = 0;
+    for (const Group* g : {b, b->rest}) {   // the members outside the team count apart
+      if (!g || !g->d_ctl) continue;
+      GroupCtl c{};
+      CK(cudaMemcpyAsync(&c, g->d_ctl, sizeof(c), cudaMemcpyDeviceToHost, b->stream));
       CK(cudaStreamSynchronize(b->stream));
+      *launches += (int64_t)c.launches;
     }
-    *launches = (int64_t)c.launches;
   }
   return GBMD_OK;
 }

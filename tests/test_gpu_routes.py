@@ -62,3 +62,21 @@ def test_noalloc_thermo_of_a_tree_list_whose_wide_types_take_many_tiles():
     assert t["pe"] == ref["pe"] < 0.0 and t["virial"] == ref["virial"]
     s.close()
 
+
+def test_a_batch_counts_the_launches_of_every_member():
+    """A member that the team takes and one too large for it: 16 steps are one launch of
+    the first and at least 16 of the second."""
+    b = gbmd.Batch("mixed")
+    ss = [gbmd.System.from_workload(wl.lj_fluid(n, 0.84, 1.2, seed=770)) for n in (2000, 60000)]
+    for s in ss:
+        b.add(s)
+    b.step(16)
+    b.sync()
+    first = b.info()["kernel_launches"]
+    assert first >= 16
+    b.step(16)
+    b.sync()
+    assert b.info()["kernel_launches"] - first >= 16
+    b.close()
+    for s in ss:
+        s.close()
