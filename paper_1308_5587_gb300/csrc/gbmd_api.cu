@@ -371,7 +371,9 @@ int sync_layout(Group* g) {
       for (int b = 0; b < d.nblocks; b += 8) tbk.push_back({(int)k, b, std::min(8, d.nblocks - b), 0});
       g->window_cap = std::max(g->window_cap, d.window_cap);
     } else {
+      d.nh_blocks = -(int)tf.size();
       force_tiles(d, (int)k, g->precision, g->tpp, per_f, &tf);
+      d.nh_blocks += (int)tf.size();
       d.nh_first = nh_chunks;
       d.nh_count = (int)(((long long)n * g->tpp + 31) / 32);
       nh_chunks += d.nh_count;

@@ -171,14 +171,15 @@ struct SysDev {
   int *rmember;            // particle index -> member rank
   int sort_period;
   double dt, h;            // h = dt / (2 m)
-  // NVT (Nose-Hoover, MTK form): nh = {xi, eta, exp(-xi dt/2), 0} on the device;
+  // NVT (Nose-Hoover, MTK form): nh = {xi, eta, exp(-xi dt/2), arrivals} on the device, the
+  // arrivals of the force half's nh_blocks blocks as an unsigned (0 between launches);
   // nh_part: the group's partial sums of v.v, one per chunk of 32 / TPP particles, this
   // system's from nh_first on
   int nvt;
   double kT, tau, gdof;    // gdof = 3N - 3
   double* nh;
   double* nh_part;
-  int nh_first, nh_count;
+  int nh_first, nh_count, nh_blocks;
   double dtq[3];           // dt * 2^32 / L: the drift in box-fraction units
   double mass;
   int eval;                // PairEval of the system's potential
@@ -220,7 +221,6 @@ struct TeamSync {
 // group-level control block (one per single system or batch)
 struct GroupCtl {
   unsigned int blocks_done;  // last-block counter of the step kernel
-  unsigned int blocks_done_a;   // last-block counter of the NVT force half
   int any_rebuild;
   unsigned long long launches;
   TeamSync team;             // of a team that is a whole grid

@@ -586,8 +586,7 @@ __device__ __forceinline__ void force_body(const SysDev* __restrict__ sysv, cons
   if (NVTA) {
     if (bad) atomicCAS(&s.flags->error, 0, (int)DEV_NONFINITE);
     const int p0 = (int)(threadIdx.x & ~31u) / TPP;   // this warp's first particle of the tile
-    nvt_half_tail(s, sysv, ctl, nsys, total_blocks, uu,
-                  p0 < t.count ? (t.first + p0) / (32 / TPP) : -1);
+    nvt_half_tail(s, uu, p0 < t.count ? (t.first + p0) / (32 / TPP) : -1);
   }
 }
 

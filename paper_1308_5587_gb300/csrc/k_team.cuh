@@ -160,7 +160,7 @@ __global__ void __launch_bounds__(TEAM_T, 1) k_team(TeamArgs a) {
       const unsigned v = tm.vote(bad ? VOTE_BAD : 0u);
       if (v & VOTE_LOST) { error = DEV_TEAM; break; }
       if (v & VOTE_BAD) { error = DEV_NONFINITE; break; }
-      const double sum = nh_total(s.nh_part + s.nh_first, s.nh_count, sm.sums);
+      const double sum = nh_total<1>(s.nh_part + s.nh_first, s.nh_count, sm.sums);
       if (threadIdx.x == 0) nvt_sc = nh_update(s, sum, vfull, xi, eta);
       __syncthreads();
       sc = nvt_sc;

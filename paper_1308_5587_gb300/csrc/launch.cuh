@@ -63,8 +63,8 @@ KernelCall tree_nlist_call(const SysDev* d, const Tile* tiles_g, int ntiles, Gro
 // update of every particle into the next shadow buffer, and the end-of-step
 // decisions by the last of sa.total_blocks blocks over the step's force launches.
 // MODE_NVT_A: the first half of an NVT step -- forces, the closing half kick and
-// thermostat scaling of the previous step, v.v partial sums; the last block updates
-// the thermostat.  nvt_b_call: the second half (opening scaling and kick, drift,
+// thermostat scaling of the previous step, v.v partial sums; a system's last block
+// updates its thermostat.  nvt_b_call: the second half (opening scaling and kick, drift,
 // shadow, rebuild check, end-of-step decisions).
 enum { MODE_FORCE = 0, MODE_EV = 1, MODE_STEP = 2, MODE_NVT_A = 3 };
 // which step configurations take wide tiles, a warp a particle (all modes of one do, so

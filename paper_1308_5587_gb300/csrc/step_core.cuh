@@ -206,27 +206,40 @@ __device__ __forceinline__ double nh_warp_sum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
   return v;   // lane 0
 }
-// every thread of the block (whole warps) calls it; the sum is returned to all.  `sums`
-// (shared) may be written again after the block's next barrier.
+// Every thread of the block (whole warps) calls it; the sum is returned to all.  `sums`
+// (shared) may be written again after the block's next barrier.  SIDE: slots that a thread
+// sums side by side, four loads in flight for each (from L2: other blocks wrote them).  The
+// team's 512 threads take one each; the tail of the step kernel's force half, often 128
+// threads, four: one after another they were a chain of 20 such rounds at N = 160,000 (NVT,
+// mixed: 90.8 us a step so, 86.4 side by side).
+template <int SIDE>
 __device__ __forceinline__ double nh_total(const double* part, int count, double* sums) {
-  const int lane = threadIdx.x & 31;
-  for (int v = threadIdx.x; v < NH_SLOTS; v += blockDim.x) {
-    double a = 0.0;
-    int k = v;
-    for (; k + 3 * NH_SLOTS < count; k += 4 * NH_SLOTS) {   // four loads in flight (from L2:
-      double p[4];                                          // other blocks wrote them)
+  constexpr int DEEP = 4;
+  const int lane = threadIdx.x & 31, nt = (int)blockDim.x;
+  for (int v0 = threadIdx.x; v0 < NH_SLOTS; v0 += SIDE * nt) {   // the same for a warp's lanes
+    double a[SIDE];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) p[u] = __ldcg(part + k + u * NH_SLOTS);
+    for (int q = 0; q < SIDE; ++q) a[q] = 0.0;
+    for (int k = v0; k < count; k += DEEP * NH_SLOTS) {
+      double p[SIDE][DEEP];
 #pragma unroll
-      for (int u = 0; u < 4; ++u) a += p[u];
+      for (int q = 0; q < SIDE; ++q)
+#pragma unroll
+        for (int u = 0; u < DEEP; ++u) {
+          const int at = k + q * nt + u * NH_SLOTS;
+          p[q][u] = v0 + q * nt < NH_SLOTS && at < count ? __ldcg(part + at) : 0.0;
+        }
+#pragma unroll
+      for (int q = 0; q < SIDE; ++q)
+#pragma unroll
+        for (int u = 0; u < DEEP; ++u) a[q] += p[q][u];
     }
-    double p[3];
 #pragma unroll
-    for (int u = 0; u < 3; ++u) p[u] = k + u * NH_SLOTS < count ? __ldcg(part + k + u * NH_SLOTS) : 0.0;
-#pragma unroll
-    for (int u = 0; u < 3; ++u) a += p[u];
-    a = nh_warp_sum(a);
-    if (lane == 0) sums[v >> 5] = a;
+    for (int q = 0; q < SIDE; ++q) {
+      const int v = v0 + q * nt;
+      const double w = nh_warp_sum(a[q]);
+      if (lane == 0 && v < NH_SLOTS) sums[v >> 5] = w;
+    }
   }
   __syncthreads();
   double r = sums[lane & (NH_SUMS - 1)];
@@ -254,40 +267,37 @@ __device__ __forceinline__ double nh_update(const SysDev& s, double sum, int vfu
 }
 
 // End of the NVT force half, every block: publish the warps' v.v sums (chunk `chunk` of
-// the system for this warp, -1: none) and count the arrival; the last block updates
-// every NVT system's thermostat.
-__device__ __forceinline__ void nvt_half_tail(const SysDev& s, const SysDev* __restrict__ sysv,
-                                              GroupCtl* ctl, int nsys, int total_blocks,
-                                              double uu, int chunk) {
+// the system for this warp, -1: none) and count the arrival; the last block of the system's
+// own (nh_blocks of them) updates its thermostat.  (By the launch's last block for one
+// system after another, us a step: 200 replicas of 500 1,118, so 231; 128 of 500 to 20,000
+// 992 and 374; FP64 1,619 and 982.)
+__device__ __forceinline__ void nvt_half_tail(const SysDev& s, double uu, int chunk) {
   const double part = nh_warp_sum(uu);
   if ((threadIdx.x & 31) == 0 && chunk >= 0) s.nh_part[s.nh_first + chunk] = part;
   __shared__ int last;
   __shared__ double sums[NH_SUMS];
+  unsigned* const arrive = reinterpret_cast<unsigned*>(s.nh + 3);
   __threadfence();
   __syncthreads();
   if (threadIdx.x == 0) {
     __threadfence();
-    last = (atomicAdd(&ctl->blocks_done_a, 1u) == (unsigned)total_blocks - 1u);
+    last = (atomicAdd(arrive, 1u) == (unsigned)s.nh_blocks - 1u);
   }
   __syncthreads();
   if (!last) return;
   __threadfence();
-  for (int k = 0; k < nsys; ++k) {   // uniform over the block
-    const SysDev& sk = sysv[k];
-    if (!sk.nvt) continue;
-    const FlagWords w = load_flag_words(sk.flags);
-    const longlong2 sl = load_flag_pair(&sk.flags->step);
-    if (!(w.error == 0 && (sl.y < 0 || sl.x < sl.y))) continue;
-    __syncthreads();   // the previous system's sums have been read
-    const double sum = nh_total(sk.nh_part + sk.nh_first, sk.nh_count, sums);
-    if (threadIdx.x == 0) {
-      double xi = sk.nh[0], eta = sk.nh[1];
-      sk.nh[2] = nh_update(sk, sum, w.v_full, xi, eta);
-      sk.nh[0] = xi;
-      sk.nh[1] = eta;
-    }
+  if (threadIdx.x == 0) *arrive = 0u;
+  // every block of the system has arrived: nothing writes its flags any more
+  const FlagWords w = load_flag_words(s.flags);
+  const longlong2 sl = load_flag_pair(&s.flags->step);
+  if (!(w.error == 0 && (sl.y < 0 || sl.x < sl.y))) return;
+  const double sum = nh_total<4>(s.nh_part + s.nh_first, s.nh_count, sums);
+  if (threadIdx.x == 0) {
+    double xi = s.nh[0], eta = s.nh[1];
+    s.nh[2] = nh_update(s, sum, w.v_full, xi, eta);
+    s.nh[0] = xi;
+    s.nh[1] = eta;
   }
-  if (threadIdx.x == 0) ctl->blocks_done_a = 0;
 }
 
 // End of the step, every block of the step's force launches: publish this block's
