@@ -214,26 +214,41 @@ __device__ __forceinline__ double nh_warp_sum(double v) {
 // mixed: 90.8 us a step so, 86.4 side by side).
 template <int SIDE>
 __device__ __forceinline__ double nh_total(const double* part, int count, double* sums) {
-  constexpr int DEEP = 4;
   const int lane = threadIdx.x & 31, nt = (int)blockDim.x;
+  // full rounds while the farthest slot of a thread has one (a block of more than a quarter
+  // of the slots' threads has fewer slots side by side: the others read nothing); then a
+  // slot has TAIL terms left at most
+  constexpr int TAIL = SIDE == 1 ? 3 : 4;
+  const int far = SIDE == 1 ? 0 : min((SIDE - 1) * nt, NH_SLOTS - 1);
   for (int v0 = threadIdx.x; v0 < NH_SLOTS; v0 += SIDE * nt) {   // the same for a warp's lanes
     double a[SIDE];
 #pragma unroll
     for (int q = 0; q < SIDE; ++q) a[q] = 0.0;
-    for (int k = v0; k < count; k += DEEP * NH_SLOTS) {
-      double p[SIDE][DEEP];
+    int k = v0;
+    for (; k + far + 3 * NH_SLOTS < count; k += 4 * NH_SLOTS) {
+      double p[SIDE][4];
 #pragma unroll
       for (int q = 0; q < SIDE; ++q)
 #pragma unroll
-        for (int u = 0; u < DEEP; ++u) {
-          const int at = k + q * nt + u * NH_SLOTS;
-          p[q][u] = v0 + q * nt < NH_SLOTS && at < count ? __ldcg(part + at) : 0.0;
-        }
+        for (int u = 0; u < 4; ++u)
+          p[q][u] = SIDE == 1 || v0 + q * nt < NH_SLOTS ? __ldcg(part + k + q * nt + u * NH_SLOTS) : 0.0;
 #pragma unroll
       for (int q = 0; q < SIDE; ++q)
 #pragma unroll
-        for (int u = 0; u < DEEP; ++u) a[q] += p[q][u];
+        for (int u = 0; u < 4; ++u) a[q] += p[q][u];
     }
+    double p[SIDE][TAIL];
+#pragma unroll
+    for (int q = 0; q < SIDE; ++q)
+#pragma unroll
+      for (int u = 0; u < TAIL; ++u) {
+        const int at = k + q * nt + u * NH_SLOTS;
+        p[q][u] = (SIDE == 1 || v0 + q * nt < NH_SLOTS) && at < count ? __ldcg(part + at) : 0.0;
+      }
+#pragma unroll
+    for (int q = 0; q < SIDE; ++q)
+#pragma unroll
+      for (int u = 0; u < TAIL; ++u) a[q] += p[q][u];
 #pragma unroll
     for (int q = 0; q < SIDE; ++q) {
       const int v = v0 + q * nt;
