@@ -383,9 +383,11 @@ int gbmd_set_force_events(gbmd_system *s, void *ev_begin, void *ev_end);
 
 /* ---- many systems stepped together ------------------------------------------ */
 
-/* A batch steps all its systems with one launch per kernel per step (all systems
- * share every launch) inside captured CUDA graphs.  Every member must have the
- * batch's precision and device.  stream: cudaStream_t or NULL; device: ordinal
+/* A batch steps its systems with shared launches: small members on the cell list by
+ * resident blocks, many steps a launch and each member at its own pace, where that
+ * is the faster way; the others, or all of them, with one launch per kernel per step
+ * inside captured CUDA graphs.  The results are the same.  Every member must have
+ * the batch's precision and device.  stream: cudaStream_t or NULL; device: ordinal
  * or -1 for the calling thread's current device. */
 int gbmd_batch_create(int32_t precision, void *stream, int32_t device, gbmd_batch **out);
 

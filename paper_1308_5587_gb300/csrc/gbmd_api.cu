@@ -95,6 +95,23 @@ struct gbmd_system {
 
 constexpr int TEAM_SIDES = 4;   // cluster sizes 16, 8, 4, 2, 1: the first on the group's stream
 
+// what a resident kernel may use of the device: SMs, its blocks on one, and how many of its
+// clusters of 2^k blocks run at once (fewer than the SMs would hold: a cluster stays in one
+// part of the chip, 18 or 20 SMs; of 1, 2, .. 16 blocks, one an SM: 152, 76, 36, 15, 7)
+struct TeamFit { int sms = 0, blocks_per_sm = 0, max_cluster = 0, clusters[TEAM_SIDES + 1] = {}; };
+
+// how a group's team members are stepped: the kernel, its lanes a particle, and its launches,
+// members [first, last) of the team each by clusters of that many blocks (0: by the whole
+// grid, as shares of it or a system alone)
+struct TeamClass { int first, last, cluster; };
+struct TeamPlan {
+  void* func = nullptr;
+  int lanes = 1;
+  TeamFit fit;
+  bool shares = false;
+  std::vector<TeamClass> cls;
+};
+
 struct Group {
   int device = 0;
   std::vector<gbmd_system*> members;   // may contain nullptr (free slots of a batch)
@@ -134,18 +151,17 @@ struct Group {
   bool graphs_dirty = true;
   bool use_graphs = true;
   // the members that the team kernel steps (positions among the live members, the
-  // largest first); the others, if any, are stepped by the graph of `rest`
+  // largest first) and how; the others, if any, are stepped by the graph of `rest`
   std::vector<int> team;
+  std::vector<int> team_n;             // their particles
+  TeamPlan plan;
   int* d_team = nullptr;
   size_t cap_team = 0;
   // a batch's teams as shares of one grid: per block (member, rank, blocks, team)
   std::vector<int4> share;
-  bool share_dirty = true;
   int4* d_share = nullptr;
   TeamSync* d_sync = nullptr;
   size_t cap_share = 0, cap_sync = 0;
-  std::vector<int> team_n;             // their particles
-  int team_max_n = 0;
   int polls = TEAM_POLLS;
   cudaStream_t side[TEAM_SIDES] = {};
   cudaEvent_t side_ev[TEAM_SIDES + 1] = {};
@@ -238,16 +254,15 @@ int tree_groups(const SysDev& d, int ty) {
 // by the team; FP64, 20 steps, 2,291 and 2,211; FP64 NVT, 20 steps, 2,690 and 2,397.
 // (N = 200,000, several turns: 73 us a step by the team, 66 by the step kernel.)
 // In a batch, where a shared launch makes every member wait for any member's rebuild, up
-// to what one cluster steps in about 50 us.
+// to TEAM_MEMBER_N (measured to 30,000), as far as that pays (plan_team).
 constexpr int TEAM_ALONE_N = 49152;
-constexpr int TEAM_TURN_N = 152 * TEAM_T;   // one turn of the team's warps, one lane a particle
-constexpr int TEAM_CLUSTER_N = 32768;
+constexpr int TEAM_MEMBER_N = 32768;
 constexpr int TEAM_STEPS = 64;   // steps of one launch
-bool team_member(const Group* g, const SysDev& d) {
+bool team_member(const Group* g, const SysDev& d, int sms) {
   if (d.tree || d.staged || d.n_ghost > 0) return false;
-  if (g->is_batch) return d.n <= TEAM_CLUSTER_N;
+  if (g->is_batch) return d.n <= TEAM_MEMBER_N;
   const int lanes = g->precision == GBMD_MIXED && g->tpp == 2 ? 1 : g->tpp;
-  return d.n <= std::max(TEAM_ALONE_N, TEAM_TURN_N / lanes);
+  return d.n <= std::max(TEAM_ALONE_N, sms * TEAM_T / lanes);
 }
 
 // The force tiles of a system, `per` particles each.  The particles of a wide type of a
@@ -270,66 +285,197 @@ void force_tiles(const SysDev& d, int sys, int prec, int tpp, int per, std::vect
   }
 }
 
-std::vector<int4> team_shares(const std::vector<int>& work, int sms);
-int team_cluster(int chunks, int per_block, int most);
-
-// Whether a batch's members of n[] particles go by the team: not where the shared launches
-// keep the chip busy anyway, and not as shares of the grid with too much on one block
-// (every member has at least one).  us a step by the shared graph / the team, replicas of
-// 500 to 20,000: 12 (32,000 particles) 90 / 32, 48 (315,000) 213 / 112, 96 (572,000) 293 /
-// 245, and with the fullest share 2.3 and 3.3 times the mean 128 (736,000) 351 / 424,
-// 152 (914,000) 364 / 797; more members than SMs, by clusters, 200 (1,241,000) 451 / 450,
-// 256 (1,543,000) 526 / 562.
-constexpr long long TEAM_BATCH_SUM = 655360;
-constexpr double TEAM_UNEVEN = 1.8;
-bool batch_by_team(const Group* g, const std::vector<int>& n) {
-  constexpr int SMS = TEAM_TURN_N / TEAM_T, WARPS = TEAM_T / 32, AT_ONCE = 8;   // clusters of 16
-  long long sum = 0;
-  int blocks = 0, largest = 0;
-  for (int k : n) {
-    const int c = team_cluster((int)(((long long)k * g->tpp + 31) / 32), WARPS, TEAM_MAX_CLUSTER);
-    sum += k;
-    blocks += c;
-    largest += c == TEAM_MAX_CLUSTER;
+// TeamFit of a resident kernel, asked once per kernel and device
+int team_fit(void* f, int threads, size_t smem, int dev, TeamFit* out) {
+  static std::mutex mu;
+  static std::map<std::pair<int, void*>, TeamFit> known;
+  std::lock_guard<std::mutex> lock(mu);
+  auto it = known.find({dev, f});
+  if (it != known.end()) {
+    *out = it->second;
+    return GBMD_OK;
   }
-  if (sum > TEAM_BATCH_SUM) return false;
-  if ((blocks <= SMS && largest <= AT_ONCE) || (int)n.size() > SMS) return true;
-  double most = 0;
-  for (const int4& s : team_shares(n, SMS)) most = std::max(most, (double)n[s.x] / s.z);
-  return most <= TEAM_T || most <= TEAM_UNEVEN * sum / SMS;   // one turn of a block's warps, or even
+  TeamFit t;
+  CK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+  CK(cudaDeviceGetAttribute(&t.sms, cudaDevAttrMultiProcessorCount, dev));
+  CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&t.blocks_per_sm, f, threads, smem));
+  CK(cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+  for (int k = 0; k <= TEAM_SIDES; ++k) {
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(1u << k);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim = {1u << k, 1, 1};
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(&t.clusters[k], f, &cfg) != cudaSuccess) {
+      cudaGetLastError();
+      t.clusters[k] = 0;
+    }
+    if (t.clusters[k] > 0) t.max_cluster = 1 << k;
+  }
+  known[{dev, f}] = t;
+  *out = t;
+  return GBMD_OK;
 }
 
-// Rebuild descriptor copies and tile tables for the group's current members.
-int sync_layout(Group* g) {
-  if (!g->layout_dirty) return GBMD_OK;
-  std::vector<gbmd_system*> m = live(g);
-  g->polls = TEAM_POLLS;
-  // a test lets the waits run out
-  if (const char* ev = getenv("GBMD_TEAM_POLLS")) g->polls = std::max(0, atoi(ev));
-  g->team.clear();
-  g->team_max_n = 0;
-  std::vector<gbmd_system*> others;
-  if (g->use_graphs && !g->is_rest)
-    for (size_t k = 0; k < m.size(); ++k) {
-      if (team_member(g, m[k]->h)) {
-        g->team.push_back((int)k);
-        g->team_max_n = std::max(g->team_max_n, m[k]->h.n);
-      } else {
-        others.push_back(m[k]);
-      }
-    }
-  std::stable_sort(g->team.begin(), g->team.end(), [&](int a, int b) { return m[a]->h.n > m[b]->h.n; });
-  if (g->is_batch) {
-    std::vector<int> n;
-    for (int k : g->team) n.push_back(m[k]->h.n);
-    if (!batch_by_team(g, n)) {
-      g->team.clear();
-      g->team_max_n = 0;
+// A system alone takes one cluster up to TEAM_CLUSTER_CHUNKS warps' work a step (FP64,
+// bound by the SMs' FP64 pipes: one block's warps), and every SM beyond that (N = 2,000,
+// mixed: 8.1 us a step either way; N = 4,000: 12 on a cluster of 16, 9 on the grid).
+constexpr int TEAM_CLUSTER_CHUNKS = 128;
+int team_cluster(int chunks, int per_block, int most) {
+  int c = 1;
+  while (c < most && (long long)c * per_block < chunks) c *= 2;
+  return c;
+}
+// shares of `sms` blocks for the team's members: one each, then the next always to the
+// member with the most work a block
+std::vector<int4> team_shares(const std::vector<int>& work, int sms) {
+  const int teams = (int)work.size();
+  std::vector<int> blocks(teams, 1);
+  auto less = [&](int a, int b) {   // work a block; the earlier of equals first
+    const long long x = (long long)work[a] * blocks[b], y = (long long)work[b] * blocks[a];
+    return x != y ? x < y : a > b;
+  };
+  std::vector<int> heap(teams);
+  for (int t = 0; t < teams; ++t) heap[t] = t;
+  std::make_heap(heap.begin(), heap.end(), less);
+  for (int k = teams; k < sms; ++k) {
+    std::pop_heap(heap.begin(), heap.end(), less);
+    ++blocks[heap.back()];
+    std::push_heap(heap.begin(), heap.end(), less);
+  }
+  std::vector<int4> out;
+  for (int t = 0; t < teams; ++t)
+    for (int r = 0; r < blocks[t]; ++r) out.push_back(make_int4(t, r, blocks[t], t));
+  return out;
+}
+
+// How the group's team members (g->team, g->team_n) are stepped; without a plan that pays
+// the list is emptied.
+//
+// A batch's members divide one grid: each gets a share of the SMs by its particles, and no SM
+// waits for a cluster to fit or stands beside a power of two.  Its barriers go through
+// memory (2 us a step) where a cluster's take 0.5: clusters of 16, 8, .. 1 blocks by a
+// member's own size, one launch a size, side by side on streams of their own, the largest
+// first, serve batches whose clusters all run at once with up to half a turn of its warps on
+// a block, mixed also up to two turns where no member has more than CLUSTER_SMALL_N particles,
+// FP64 (bound by the SMs' FP64 pipes) up to a quarter.  us a step by clusters / shares, mixed:
+// 4 of 500 9.7 / 11.4, 32 of 500 11.1 / 12.3, 64 of 500 21.2 / 22.1; 8 of 2,000 16.5 / 12.5, 4
+// of 4,000 16.9 / 12.8, 2 of 8,000 27.8 / 13.2, 2 of 20,000 59 / 23; FP64: 4 of 500 29.4 /
+// 30.9, 16 of 500 35.5 / 31.0, 4 of 4,000 55 / 36, 2 of 20,000 213 / 80.  More members than
+// SMs take clusters as they become free.
+//
+// Against the shared graph, whose kernels spread every member over the chip: the fullest block
+// of the team has more than the mean to do, and the step waits for it (TEAM_US a particle);
+// in the graph every step waits for any member's rebuild, and for the graph itself where no
+// other members need it (GRAPH_US, GRAPH_US_MEMBER).  us a step by the graph / the team,
+// mixed: 96 of 4,000 174 / 154, 100 of 8,000 266 / 332, 32 of 20,000 230 / 219, 48 of 20,000
+// 308 / 302, 40 of 30,000 363 / 427, 150 of 1,000 139 / 46, 96 of 500 to 20,000 287 / 243,
+// 200 of 500 193 / 44, 200 of 500 to 20,000 445 / 475; FP64: 96 of 4,000 524 / 650, 16 of
+// 20,000 434 / 384, 32 of 20,000 797 / 831, 48 of 500 to 20,000 489 / 419; with others: eight
+// of 4,000 and two of 64,000 88 / 70, four of 20,000 and four of 40,000 99 / 108.
+constexpr int CLUSTER_SMALL_N = 1024;
+constexpr double TEAM_US_MIXED = 0.041, TEAM_US_FP64 = 0.16;
+constexpr double GRAPH_US = 22.0, GRAPH_US_MEMBER = 1.5, TEAM_BASE_US = 10.0;
+constexpr int GRAPH_MEMBERS = 64;   // from here on some member rebuilds at every step
+constexpr double TEAM_WAVES = 1.35; // clusters one after another: the last ones' SMs stand idle
+// A member's share where the chip has less than a turn of its warps to do, mixed: by its
+// chunks and this many more, since a small member's rebuild is a chain that more blocks
+// shorten (12 of 500 to 3,000: 31 us a step without, 16 with).  FP64 forces, bound by their pipe,
+// want blocks by the pairs alone (24 of 500 to 3,000: 62 without, 78 with).
+constexpr int SHARE_EXTRA = 64;
+int plan_team(Group* g, bool others) {
+  TeamPlan& p = g->plan;
+  p = TeamPlan();
+  g->share.clear();
+  if (g->team.empty()) return GBMD_OK;
+  constexpr int warps = TEAM_T / 32;
+  const int teams = (int)g->team_n.size();
+  p.lanes = g->tpp;
+  p.func = k_team_variant(g->eval, g->precision, g->tpp, g->multi, false);
+  RET(team_fit(p.func, TEAM_T, TEAM_SMEM, g->device, &p.fit));
+  // two lanes a particle as one where that leaves every warp of the chip a chunk: a
+  // system with more than one turn of them at two lanes, a batch with more than two
+  if (g->precision == GBMD_MIXED && g->tpp == 2) {
+    long long total = 0;
+    for (int nn : g->team_n) total += ((long long)nn * 2 + 31) / 32;
+    if (total > (long long)(g->is_batch ? 2 : 1) * p.fit.sms * warps) {
+      p.lanes = 1;
+      p.func = k_team_variant(g->eval, g->precision, g->tpp, g->multi, true);
+      RET(team_fit(p.func, TEAM_T, TEAM_SMEM, g->device, &p.fit));
     }
   }
+  const TeamFit& fit = p.fit;
+  auto drop = [&]() -> int {
+    g->team.clear();
+    g->team_n.clear();
+    g->share.clear();
+    p = TeamPlan();
+    return GBMD_OK;
+  };
+  if (fit.max_cluster < 1 || fit.blocks_per_sm < 1) return drop();
+  auto chunks_of = [&](int nn) { return (int)(((long long)nn * p.lanes + 31) / 32); };
+  if (!g->is_batch && chunks_of(g->team_n[0]) > (g->precision == GBMD_FP64 ? warps : TEAM_CLUSTER_CHUNKS)) {
+    p.cls.push_back({0, 1, 0});
+    return GBMD_OK;
+  }
+  int per_block = 2;
+  auto cluster_of = [&](int nn) { return team_cluster(chunks_of(nn), per_block, fit.max_cluster); };
+  auto at_once = [&]() {
+    double chip = 0;
+    for (int nn : g->team_n) chip += 1.0 / fit.clusters[31 - __builtin_clz((unsigned)cluster_of(nn))];
+    return chip <= 1.0 + 1e-9;
+  };
+  while (per_block < 4 * warps && !at_once()) per_block *= 2;
+  const bool fits = at_once();
+  double fullest = 0, sum = 0;   // particles of a block
+  for (int nn : g->team_n) {
+    fullest = std::max(fullest, (double)nn / cluster_of(nn));
+    sum += nn;
+  }
+  const bool fp64 = g->precision == GBMD_FP64;
+  const double turns = fp64 ? 0.25 : g->team_n[0] <= CLUSTER_SMALL_N ? 2.0 : 0.5;
+  p.shares = g->is_batch && teams <= fit.sms && !(fits && fullest * p.lanes <= turns * TEAM_T);
+  if (p.shares) {
+    const int extra = !fp64 && sum * p.lanes < (double)fit.sms * TEAM_T ? SHARE_EXTRA : 0;
+    std::vector<int> work;
+    for (int nn : g->team_n) work.push_back(chunks_of(nn) + extra);
+    g->share = team_shares(work, fit.sms);
+    fullest = 0;
+    for (const int4& q : g->share) fullest = std::max(fullest, (double)g->team_n[q.x] / q.z);
+    p.cls.push_back({0, teams, 0});
+  } else {
+    if (!fits) fullest = std::max(fullest, TEAM_WAVES * sum / fit.sms);
+    for (int k = 0; k < teams; ++k) {
+      const int c = cluster_of(g->team_n[k]);
+      if (p.cls.empty() || p.cls.back().cluster != c) p.cls.push_back({k, k, c});
+      p.cls.back().last = k + 1;
+    }
+  }
+  if (!g->is_batch) return GBMD_OK;
+  const double more = (fullest - sum / fit.sms) * (fp64 ? TEAM_US_FP64 : TEAM_US_MIXED);
+  const double less = (others ? 0.0 : GRAPH_US) + GRAPH_US_MEMBER * std::min(teams, GRAPH_MEMBERS) - TEAM_BASE_US;
+  return more <= less ? GBMD_OK : drop();
+}
+
+// Which members the team kernel steps, and the group of the others
+int split_members(Group* g, const std::vector<gbmd_system*>& m) {
+  g->team.clear();
   g->team_n.clear();
+  std::vector<gbmd_system*> others;
+  int sms = 0;
+  CK(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, g->device));
+  if (g->use_graphs && !g->is_rest)
+    for (size_t k = 0; k < m.size(); ++k) {
+      if (team_member(g, m[k]->h, sms)) g->team.push_back((int)k);
+      else others.push_back(m[k]);
+    }
+  std::stable_sort(g->team.begin(), g->team.end(), [&](int a, int b) { return m[a]->h.n > m[b]->h.n; });
   for (int k : g->team) g->team_n.push_back(m[k]->h.n);
-  g->share_dirty = true;
+  RET(plan_team(g, !others.empty()));
   if (!g->team.empty() && !others.empty()) {
     if (!g->rest) {
       g->rest = new Group();
@@ -348,6 +494,16 @@ int sync_layout(Group* g) {
     g->rest->members.clear();
     g->rest->layout_dirty = true;
   }
+  return GBMD_OK;
+}
+
+// Rebuild descriptor copies and tile tables for the group's current members.
+int sync_layout(Group* g) {
+  if (!g->layout_dirty) return GBMD_OK;
+  std::vector<gbmd_system*> m = live(g);
+  g->polls = TEAM_POLLS;
+  // a test lets the waits run out
+  if (const char* ev = getenv("GBMD_TEAM_POLLS")) g->polls = std::max(0, atoi(ev));
   std::vector<SysDev> desc;
   std::vector<Tile> tp, tf, tc, ts, tb, tbk, te, tt, tg, tn;
   const int per_f = g->fblock / g->tpp;
@@ -403,6 +559,7 @@ int sync_layout(Group* g) {
       if (d.nc[0] < 3 || d.nc[1] < 3 || d.nc[2] < 3) g->rel = false;
     }
   }
+  RET(split_members(g, m));
   for (auto& d : desc)
     if (d.staged) d.tile_first_f += (int)te.size();   // staged partial sums follow the global ones
   RET(grow(&g->d_partials, &g->cap_part, 8 * std::max<size_t>(te.size() + tb.size(), 1)));
@@ -423,6 +580,8 @@ int sync_layout(Group* g) {
   RET(grow(&g->d_tg, &g->cap_tg, tg.size()));
   RET(grow(&g->d_tn, &g->cap_tn, tn.size()));
   RET(grow(&g->d_team, &g->cap_team, g->team.size()));
+  RET(grow(&g->d_share, &g->cap_share, g->share.size()));
+  if (!g->share.empty()) RET(grow(&g->d_sync, &g->cap_sync, (size_t)g->plan.fit.sms));   // a team a block at most
   if (!g->d_ctl) {
     CK(cudaMalloc(&g->d_ctl, sizeof(GroupCtl)));
     CK(cudaMemsetAsync(g->d_ctl, 0, sizeof(GroupCtl), g->stream));
@@ -446,6 +605,8 @@ int sync_layout(Group* g) {
   CK(up(g->d_tt, tt));
   CK(up(g->d_tg, tg));
   CK(up(g->d_tn, tn));
+  if (!g->share.empty())
+    CK(cudaMemcpyAsync(g->d_share, g->share.data(), g->share.size() * sizeof(int4), cudaMemcpyHostToDevice, g->stream));
   if (!g->team.empty())
     CK(cudaMemcpyAsync(g->d_team, g->team.data(), g->team.size() * sizeof(int), cudaMemcpyHostToDevice, g->stream));
   CK(cudaStreamSynchronize(g->stream));   // host vectors die here
@@ -550,45 +711,6 @@ std::vector<KernelCall> step_calls(const Group* g, cudaGraphConditionalHandle co
     v.push_back(force_staged_call(g->multi, MODE_STEP, g->d_desc, g->d_tb, g->ntb, g->d_ctl, g->nte,
                                   g->window_cap, sa));
   return v;
-}
-
-// what a team kernel may use of the device, asked once per kernel and device
-struct TeamFit { int sms = 0, blocks_per_sm = 0, max_cluster = 0, clusters = 0; };   // clusters: of the largest at once
-int team_fit(void* f, int threads, size_t smem, int dev, TeamFit* out) {
-  static std::mutex mu;
-  static std::map<std::pair<int, void*>, TeamFit> known;
-  std::lock_guard<std::mutex> lock(mu);
-  auto it = known.find({dev, f});
-  if (it != known.end()) {
-    *out = it->second;
-    return GBMD_OK;
-  }
-  TeamFit t;
-  CK(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-  CK(cudaDeviceGetAttribute(&t.sms, cudaDevAttrMultiProcessorCount, dev));
-  CK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&t.blocks_per_sm, f, threads, smem));
-  CK(cudaFuncSetAttribute(f, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
-  for (int c = TEAM_MAX_CLUSTER; c >= 1 && !t.max_cluster; c /= 2) {
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(c);
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = smem;
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim = {(unsigned)c, 1, 1};
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
-    int num = 0;
-    if (cudaOccupancyMaxActiveClusters(&num, f, &cfg) == cudaSuccess && num > 0) {
-      t.max_cluster = c;
-      t.clusters = num;
-    } else {
-      cudaGetLastError();
-    }
-  }
-  known[{dev, f}] = t;
-  *out = t;
-  return GBMD_OK;
 }
 
 // The rebuild of a step of one system alone as one cooperative kernel after the step
@@ -714,72 +836,17 @@ int team_stream(Group* g, size_t q) {
   return GBMD_OK;
 }
 
-// n steps of the group's team members, one launch per TEAM_STEPS steps.  A system
-// alone takes one cluster up to TEAM_CLUSTER_CHUNKS warps' work a step (FP64, bound by
-// the SMs' FP64 pipes: one block's warps), and every SM beyond that (N = 2,000, mixed: 8.1
-// us a step either way; N = 4,000: 12 on a cluster of 16, 9 on the grid).  A batch's
-// members take clusters of 16, 8, .. 1 blocks by their own size, one launch a size, side
-// by side on streams of their own, the largest first.  A step is shortest with few warps
-// on an SM, the SMs' throughput best with many: a block gets two warps' work while all
-// clusters then fit the SMs at once, else up to four turns of its warps.
-//
-// A batch that would fill the SMs for more than one turn of their warps, or has more
-// teams for the largest clusters than run at once (one of 16 blocks to each part of the
-// chip with 18 or 20 SMs), divides one grid instead: each member gets a share of the SMs
-// by its particles, and no SM waits for a cluster to fit or stands beside a power of two.
-// Its barriers go through memory (2 us instead of 0.5).  48 replicas (N = 500 to 20,000),
-// 64 steps and their readouts: 20.4 ms by clusters, 17.4 by shares.
-constexpr int TEAM_CLUSTER_CHUNKS = 128;
-int team_cluster(int chunks, int per_block, int most) {
-  int c = 1;
-  while (c < most && (long long)c * per_block < chunks) c *= 2;
-  return c;
-}
-// shares of `sms` blocks for the team's members: one each, then the next always to the
-// member with the most work a block
-std::vector<int4> team_shares(const std::vector<int>& work, int sms) {
-  const int teams = (int)work.size();
-  std::vector<int> blocks(teams, 1);
-  auto less = [&](int a, int b) {   // work a block; the earlier of equals first
-    const long long x = (long long)work[a] * blocks[b], y = (long long)work[b] * blocks[a];
-    return x != y ? x < y : a > b;
-  };
-  std::vector<int> heap(teams);
-  for (int t = 0; t < teams; ++t) heap[t] = t;
-  std::make_heap(heap.begin(), heap.end(), less);
-  for (int k = teams; k < sms; ++k) {
-    std::pop_heap(heap.begin(), heap.end(), less);
-    ++blocks[heap.back()];
-    std::push_heap(heap.begin(), heap.end(), less);
-  }
-  std::vector<int4> out;
-  for (int t = 0; t < teams; ++t)
-    for (int r = 0; r < blocks[t]; ++r) out.push_back(make_int4(t, r, blocks[t], t));
-  return out;
-}
+// n steps of the group's team members by its plan, one launch per TEAM_STEPS steps
 int launch_team(Group* g, long long n) {
-  void* f = k_team_variant(g->eval, g->precision, g->tpp, g->multi, false);
-  TeamFit fit;
-  RET(team_fit(f, TEAM_T, TEAM_SMEM, g->device, &fit));
-  const int warps = TEAM_T / 32;
-  // two lanes a particle as one where that leaves every warp of the chip a chunk: a
-  // system with more than one turn of them at two lanes, a batch with more than two
-  int lanes = g->tpp;
-  if (g->precision == GBMD_MIXED && g->tpp == 2) {
-    long long total = 0;
-    for (int nn : g->team_n) total += ((long long)nn * 2 + 31) / 32;
-    if (total > (long long)(g->is_batch ? 2 : 1) * fit.sms * warps) {
-      lanes = 1;
-      f = k_team_variant(g->eval, g->precision, g->tpp, g->multi, true);
-      RET(team_fit(f, TEAM_T, TEAM_SMEM, g->device, &fit));
-    }
-  }
-  if (fit.max_cluster < 1) return fail(GBMD_ERR_CUDA, "the team kernel does not fit the device");
-  auto chunks_of = [&](int nn) { return (int)(((long long)nn * lanes + 31) / 32); };
+  const TeamPlan& p = g->plan;
   TeamArgs a{};
   a.desc = g->d_desc;
   a.ctl = g->d_ctl;
   a.polls = g->polls;
+  if (p.shares) {
+    a.share = g->d_share;
+    a.sync = g->d_sync;
+  }
   cudaLaunchConfig_t cfg{};
   cfg.blockDim = dim3(TEAM_T);
   cfg.dynamicSmemBytes = TEAM_SMEM;
@@ -787,54 +854,11 @@ int launch_team(Group* g, long long n) {
   cfg.attrs = &at;
   cfg.numAttrs = 1;
   void* args[1] = {&a};
-  // the classes: [first, last) of the list, blocks per team
-  struct Class { int first, last, cluster; };
-  std::vector<Class> cls;
-  const int most = g->precision == GBMD_FP64 ? warps : TEAM_CLUSTER_CHUNKS;
-  const int teams = (int)g->team.size();
-  int full = 0, largest = 0;   // blocks for one turn of their warps; teams of the largest size
-  for (int nn : g->team_n) {
-    const int c = team_cluster(chunks_of(nn), warps, fit.max_cluster);
-    full += c;
-    largest += c == fit.max_cluster;
-  }
-  if (!g->is_batch && chunks_of(g->team_max_n) > most) {
-    cls.push_back({0, 1, 0});
-  } else if (teams > 1 && teams <= fit.sms && fit.blocks_per_sm > 0 &&
-             (full > fit.sms || largest > fit.clusters)) {
-    if (g->share_dirty) {
-      std::vector<int> chunks;
-      for (int nn : g->team_n) chunks.push_back(chunks_of(nn));
-      g->share = team_shares(chunks, fit.sms);   // `lanes` changes with the layout only
-      RET(grow(&g->d_share, &g->cap_share, g->share.size()));
-      if (!g->d_sync) {   // a team a block at most
-        RET(grow(&g->d_sync, &g->cap_sync, (size_t)fit.sms));
-        CK(cudaMemsetAsync(g->d_sync, 0, g->cap_sync * sizeof(TeamSync), g->stream));
-      }
-      CK(cudaMemcpyAsync(g->d_share, g->share.data(), g->share.size() * sizeof(int4),
-                         cudaMemcpyHostToDevice, g->stream));
-      g->share_dirty = false;
-    }
-    a.share = g->d_share;
-    a.sync = g->d_sync;
-    cls.push_back({0, teams, 0});
-  } else {
-    int per_block = 2;
-    for (; per_block < 4 * warps; per_block *= 2) {
-      long long blocks = 0;
-      for (int nn : g->team_n) blocks += team_cluster(chunks_of(nn), per_block, fit.max_cluster);
-      if (blocks <= fit.sms) break;
-    }
-    for (int k = 0; k < (int)g->team.size(); ++k) {
-      const int c = team_cluster(chunks_of(g->team_n[k]), per_block, fit.max_cluster);
-      if (cls.empty() || cls.back().cluster != c) cls.push_back({k, k, c});
-      cls.back().last = k + 1;
-    }
-  }
+  const std::vector<TeamClass>& cls = p.cls;
   for (long long k = 0; k < n; k += TEAM_STEPS) {
     a.nsteps = (int)std::min<long long>(TEAM_STEPS, n - k);
     for (size_t q = 0; q < cls.size(); ++q) {
-      const Class& c = cls[q];
+      const TeamClass& c = cls[q];
       a.list = g->d_team + c.first;
       a.cluster = c.cluster;
       cfg.stream = g->stream;
@@ -851,11 +875,11 @@ int launch_team(Group* g, long long n) {
         at.id = cudaLaunchAttributeClusterDimension;
         at.val.clusterDim = {(unsigned)c.cluster, 1, 1};
       } else {
-        cfg.gridDim = dim3(a.share ? (int)g->share.size() : fit.blocks_per_sm * fit.sms);
+        cfg.gridDim = dim3(a.share ? (int)g->share.size() : p.fit.blocks_per_sm * p.fit.sms);
         at.id = cudaLaunchAttributeCooperative;
         at.val.cooperative = 1;
       }
-      CK(cudaLaunchKernelExC(&cfg, f, args));
+      CK(cudaLaunchKernelExC(&cfg, p.func, args));
     }
   }
   for (size_t q = 1; q < cls.size(); ++q) {
