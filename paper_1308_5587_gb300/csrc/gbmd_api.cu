@@ -100,6 +100,13 @@ constexpr int TEAM_SIDES = 4;   // cluster sizes 16, 8, 4, 2, 1: the first on th
 // part of the chip, 18 or 20 SMs; of 1, 2, .. 16 blocks, one an SM: 152, 76, 36, 15, 7)
 struct TeamFit { int sms = 0, blocks_per_sm = 0, max_cluster = 0, clusters[TEAM_SIDES + 1] = {}; };
 
+struct StepGraphs {
+  cudaGraphExec_t many = nullptr, one = nullptr;
+  cudaGraph_t graph_one = nullptr;                 // kept alive for node updates
+  cudaGraphNode_t ev_begin = nullptr, ev_end = nullptr;
+  bool built = false;
+};
+
 // how a group's team members are stepped: the kernel, its lanes a particle, and its launches,
 // members [first, last) of the team each by clusters of that many blocks (0: by the whole
 // grid, as shares of it or a system alone)
@@ -142,13 +149,11 @@ struct Group {
   size_t cap_nhpart = 0;
   double* d_partials = nullptr;
   GroupCtl* d_ctl = nullptr;
-  cudaGraphExec_t exec_many = nullptr, exec_one = nullptr;
-  // optional event records around the force kernel of the single-step graph
+  // the step graphs; [1]: beside work on other streams (no launch that needs the whole chip)
+  StepGraphs graphs[2];
+  // optional event records around the force kernel of the single-step graphs
   cudaEvent_t ev_begin = nullptr, ev_end = nullptr;
-  cudaGraph_t graph_one = nullptr;                 // kept alive for node updates
-  cudaGraphNode_t node_ev_begin = nullptr, node_ev_end = nullptr;
   bool layout_dirty = true;
-  bool graphs_dirty = true;
   bool use_graphs = true;
   // the members that the team kernel steps (positions among the live members, the
   // largest first) and how; the others, if any, are stepped by the graph of `rest`
@@ -215,13 +220,43 @@ void free_group(Group* g) {
 }
 
 void destroy_graphs(Group* g) {
-  if (g->exec_many) cudaGraphExecDestroy(g->exec_many);
-  if (g->exec_one) cudaGraphExecDestroy(g->exec_one);
-  if (g->graph_one) cudaGraphDestroy(g->graph_one);
-  g->exec_many = g->exec_one = nullptr;
-  g->graph_one = nullptr;
-  g->node_ev_begin = g->node_ev_end = nullptr;
-  g->graphs_dirty = true;
+  for (StepGraphs& q : g->graphs) {
+    if (q.many) cudaGraphExecDestroy(q.many);
+    if (q.one) cudaGraphExecDestroy(q.one);
+    if (q.graph_one) cudaGraphDestroy(q.graph_one);
+    q = StepGraphs();
+  }
+}
+
+// The streams with steps enqueued that the host has not waited for since.  A cooperative launch
+// of the whole grid waits until every SM is free for it, and what other streams launch waits
+// for it in turn, so systems on streams of their own would go one after another: while some
+// other stream of the device has work, neither the team's grid nor the cooperative
+// rebuild is used.  us for a step of all, side by side, with them / so: 4 of 4,000 44.6 /
+// 28.3, 8 of 20,000 119 / 74, 8 of 150,000 515 / 367, FP64 8 of 20,000 340 / 197.  (Clusters
+// take part of the chip and stay: 8 of 1,000 13 us, 52 by the graph.)  Kept on the host, so
+// that nothing is asked of the device while some thread captures; a stream that was waited
+// for by other means counts until the library's next wait for it.
+std::mutex pending_mu;
+std::vector<std::pair<int, cudaStream_t>> pending;
+
+// nothing is pending on the device's other streams
+bool alone(int dev, cudaStream_t st) {
+  std::lock_guard<std::mutex> lock(pending_mu);
+  for (const auto& p : pending)
+    if (p.first == dev && p.second != st) return false;
+  return true;
+}
+void enqueued(int dev, cudaStream_t st) {
+  std::lock_guard<std::mutex> lock(pending_mu);
+  const std::pair<int, cudaStream_t> me(dev, st);
+  if (std::find(pending.begin(), pending.end(), me) == pending.end()) pending.push_back(me);
+}
+cudaError_t wait_for(int dev, cudaStream_t st) {
+  const cudaError_t e = cudaStreamSynchronize(st);
+  std::lock_guard<std::mutex> lock(pending_mu);
+  pending.erase(std::remove(pending.begin(), pending.end(), std::make_pair(dev, st)), pending.end());
+  return e;
 }
 
 // Which list builder serves the rebuild's own launch (the rows are the same): four warps
@@ -719,10 +754,10 @@ std::vector<KernelCall> step_calls(const Group* g, cudaGraphConditionalHandle co
 // resident warps do (KA 10^6: 312 us a step with the conditional node, 357 with this;
 // N = 200,000: 70 and 66).
 constexpr int COOP_MAX_N = 400000;
-int coop_rebuild(const Group* g, KernelCall* out) {
+int coop_rebuild(const Group* g, bool alone, KernelCall* out) {
   out->func = nullptr;
   std::vector<gbmd_system*> m = live(g);
-  if (m.size() != 1 || m[0]->h.staged || m[0]->h.n > COOP_MAX_N) return GBMD_OK;
+  if (!alone || m.size() != 1 || m[0]->h.staged || m[0]->h.n > COOP_MAX_N) return GBMD_OK;
   TeamFit fit;
   RET(team_fit(rebuild_func(g->multi > 0), REBUILD_T, REBUILD_SMEM, g->device, &fit));
   if (fit.blocks_per_sm < 1) return GBMD_OK;
@@ -750,13 +785,13 @@ int add_kernel(cudaGraph_t graph, const cudaGraphNode_t* dep, const KernelCall& 
   return GBMD_OK;
 }
 
-int build_graph(Group* g, int nsteps, cudaGraphExec_t* exec) {
+int build_graph(Group* g, int nsteps, bool alone, StepGraphs* q, cudaGraphExec_t* exec) {
   cudaGraph_t graph;
   CK(cudaGraphCreate(&graph, 0));
   const bool events = nsteps == 1 && g->ev_begin && g->ev_end;
   cudaGraphNode_t prev = nullptr;
   KernelCall coop;
-  int rc = coop_rebuild(g, &coop);
+  int rc = coop_rebuild(g, alone, &coop);
   for (int st = 0; st < nsteps && rc == GBMD_OK; ++st) {
     cudaGraphConditionalHandle h = 0;
     cudaError_t e = coop.func ? cudaSuccess
@@ -765,10 +800,10 @@ int build_graph(Group* g, int nsteps, cudaGraphExec_t* exec) {
     // force + integrate (event nodes around them when asked), then IF(rebuild){lists}
     cudaGraphNode_t before = prev;
     if (events) {
-      e = cudaGraphAddEventRecordNode(&g->node_ev_begin, graph, before ? &before : nullptr, before ? 1 : 0,
+      e = cudaGraphAddEventRecordNode(&q->ev_begin, graph, before ? &before : nullptr, before ? 1 : 0,
                                       g->ev_begin);
       if (e != cudaSuccess) { rc = fail(GBMD_ERR_CUDA, "event node: %s", cudaGetErrorString(e)); break; }
-      before = g->node_ev_begin;
+      before = q->ev_begin;
     }
     for (const KernelCall& k : step_calls(g, h, coop.func ? 0 : 1)) {
       cudaGraphNode_t n5;
@@ -778,9 +813,9 @@ int build_graph(Group* g, int nsteps, cudaGraphExec_t* exec) {
     }
     if (rc) break;
     if (events) {
-      e = cudaGraphAddEventRecordNode(&g->node_ev_end, graph, &before, 1, g->ev_end);
+      e = cudaGraphAddEventRecordNode(&q->ev_end, graph, &before, 1, g->ev_end);
       if (e != cudaSuccess) { rc = fail(GBMD_ERR_CUDA, "event node: %s", cudaGetErrorString(e)); break; }
-      before = g->node_ev_end;
+      before = q->ev_end;
     }
     if (coop.func) {
       cudaGraphNode_t nr;
@@ -812,17 +847,21 @@ int build_graph(Group* g, int nsteps, cudaGraphExec_t* exec) {
     cudaError_t e = cudaGraphInstantiate(exec, graph, 0);
     if (e != cudaSuccess) rc = fail(GBMD_ERR_CUDA, "graph instantiate: %s", cudaGetErrorString(e));
   }
-  if (events && rc == GBMD_OK) g->graph_one = graph;   // node handles stay valid
+  if (events && rc == GBMD_OK) q->graph_one = graph;   // node handles stay valid
   else cudaGraphDestroy(graph);
   return rc;
 }
 
-int ensure_graphs(Group* g) {
+int ensure_graphs(Group* g, bool alone, StepGraphs** out) {
   RET(sync_layout(g));
-  if (!g->graphs_dirty) return GBMD_OK;
-  RET(build_graph(g, STEPS_PER_GRAPH, &g->exec_many));
-  RET(build_graph(g, 1, &g->exec_one));
-  g->graphs_dirty = false;
+  KernelCall coop;
+  RET(coop_rebuild(g, true, &coop));
+  StepGraphs& q = g->graphs[alone || !coop.func ? 0 : 1];   // the same without that kernel
+  *out = &q;
+  if (q.built) return GBMD_OK;
+  RET(build_graph(g, STEPS_PER_GRAPH, alone, &q, &q.many));
+  RET(build_graph(g, 1, alone, &q, &q.one));
+  q.built = true;
   return GBMD_OK;
 }
 
@@ -890,19 +929,21 @@ int launch_team(Group* g, long long n) {
 }
 
 // enqueue n steps of the group: by the team kernel, and (members it does not take; a single
-// step with event records around its force kernel; graphs switched off) graphs or direct
-// launches
-int enqueue_steps(Group* g, long long n) {
+// step with event records around its force kernel; a grid beside other streams' work; graphs
+// switched off) graphs or direct launches
+int enqueue_steps(Group* g, long long n, bool alone) {
   if (n <= 0 || live(g).empty()) return GBMD_OK;
   RET(sync_layout(g));
-  if (!g->team.empty() && !(n == 1 && g->ev_begin && g->ev_end)) {
+  const bool whole_grid = !g->plan.cls.empty() && g->plan.cls[0].cluster == 0;
+  if (!g->team.empty() && !(n == 1 && g->ev_begin && g->ev_end) && (alone || !whole_grid)) {
     RET(launch_team(g, n));
-    return g->rest ? enqueue_steps(g->rest, n) : GBMD_OK;
+    return g->rest ? enqueue_steps(g->rest, n, alone) : GBMD_OK;
   }
   if (g->use_graphs) {
-    RET(ensure_graphs(g));
-    for (long long k = 0; k < n / STEPS_PER_GRAPH; ++k) CK(cudaGraphLaunch(g->exec_many, g->stream));
-    for (long long k = 0; k < n % STEPS_PER_GRAPH; ++k) CK(cudaGraphLaunch(g->exec_one, g->stream));
+    StepGraphs* q;
+    RET(ensure_graphs(g, alone, &q));
+    for (long long k = 0; k < n / STEPS_PER_GRAPH; ++k) CK(cudaGraphLaunch(q->many, g->stream));
+    for (long long k = 0; k < n % STEPS_PER_GRAPH; ++k) CK(cudaGraphLaunch(q->one, g->stream));
     return GBMD_OK;
   }
   for (long long k = 0; k < n; ++k) {
@@ -919,9 +960,16 @@ int enqueue_steps(Group* g, long long n) {
   return GBMD_OK;
 }
 
+// the same as a caller's steps
+int take_steps(Group* g, long long n) {
+  const bool al = alone(g->device, g->stream);
+  enqueued(g->device, g->stream);
+  return enqueue_steps(g, n, al);
+}
+
 int read_flags(gbmd_system* s, Flags* f, cudaStream_t st) {
   CK(cudaMemcpyAsync(f, s->d_flags, sizeof(Flags), cudaMemcpyDeviceToHost, st));
-  CK(cudaStreamSynchronize(st));
+  CK(wait_for(s->device, st));
   return GBMD_OK;
 }
 
@@ -934,7 +982,7 @@ int write_flags(gbmd_system* s, const Flags* f, cudaStream_t st) {
 // the Snapshot that the last readout kernel left
 int read_snapshot(gbmd_system* s, Snapshot* o, cudaStream_t st) {
   CK(cudaMemcpyAsync(o, s->h.thermo, sizeof(Snapshot), cudaMemcpyDeviceToHost, st));
-  CK(cudaStreamSynchronize(st));
+  CK(wait_for(s->device, st));
   return GBMD_OK;
 }
 
@@ -953,7 +1001,7 @@ int rebuild_and_force(gbmd_system* s, int ev) {
   RET(sync_layout(g));
   KernelCall coop;
   coop.func = nullptr;
-  if (g->use_graphs) RET(coop_rebuild(g, &coop));
+  if (g->use_graphs) RET(coop_rebuild(g, alone(g->device, g->stream), &coop));
   if (coop.func) CK(launch(coop, g->stream));
   else for (const KernelCall& c : rebuild_calls(g)) CK(launch(c, g->stream));
   for (const KernelCall& c : force_calls(g, ev)) CK(launch(c, g->stream));
@@ -981,7 +1029,7 @@ void dfree(gbmd_system* s, void* p) {
 // Grow the neighbour list to hold `need` neighbours per particle.
 int grow_nlist(gbmd_system* s, int need) {
   const int cap = (int)round_up((size_t)need + need / 4 + 8, 8);
-  CK(cudaStreamSynchronize(cur_stream(s)));
+  CK(wait_for(s->device, cur_stream(s)));
   dfree(s, s->h.nl);
   s->h.nl = nullptr;
   RET(dalloc(s, (void**)&s->h.nl, (size_t)s->h.nl_stride * cap * sizeof(int)));
@@ -1032,7 +1080,7 @@ int sync_system(gbmd_system* s) {
     long long want = s->target_step;
     if (s->step_limit >= 0) want = std::min(want, s->step_limit);
     if (f.step < want) {
-      RET(enqueue_steps(s->own, want - f.step));
+      RET(take_steps(s->own, want - f.step));
       continue;
     }
     return GBMD_OK;
@@ -1679,7 +1727,7 @@ int export_impl(gbmd_system* s, double* pos, double* vel, int32_t* image, double
     if (one) {
       s->bounce.resize(bytes);
       CK(cudaMemcpyAsync(s->bounce.data(), s->h.thermo, bytes, cudaMemcpyDeviceToHost, st));
-      CK(cudaStreamSynchronize(st));
+      CK(wait_for(s->device, st));
       memcpy(&snap, s->bounce.data(), sizeof(snap));
     } else {
       RET(read_snapshot(s, &snap, st));
@@ -1810,9 +1858,9 @@ int time_steps(Group* g, float* ms) {
       RET(write_flags(s, &f, g->stream));
     }
     constexpr int WARM = 16, STEPS = 64;
-    RET(enqueue_steps(g, WARM));
+    RET(enqueue_steps(g, WARM, true));
     CK(cudaEventRecord(a, g->stream));
-    RET(enqueue_steps(g, STEPS));
+    RET(enqueue_steps(g, STEPS, true));
     CK(cudaEventRecord(b, g->stream));
     CK(cudaEventSynchronize(b));
     float t = 0;
@@ -1853,7 +1901,7 @@ int time_rebuild(Group* g, float* ms) {
   std::vector<KernelCall> calls = rebuild_calls(g);
   KernelCall coop;
   coop.func = nullptr;
-  if (g->use_graphs) RET(coop_rebuild(g, &coop));
+  if (g->use_graphs) RET(coop_rebuild(g, true, &coop));
   if (coop.func) calls = {coop};
   cudaEvent_t a, b;
   CK(cudaEventCreate(&a));
@@ -2078,7 +2126,7 @@ int gbmd_destroy(gbmd_system* s) {
     b->layout_dirty = true;
     s->batch = nullptr;
   }
-  if (s->own) cudaStreamSynchronize(s->own->stream);
+  if (s->own) wait_for(s->device, s->own->stream);
   for (const auto& p : s->allocs) cudaFree(p.first);
   if (s->own) {
     free_group(s->own);
@@ -2093,7 +2141,7 @@ int gbmd_step(gbmd_system* s, int64_t nsteps) {
   RET(use_device(s->device));
   if (s->batch) return fail(GBMD_ERR_STATE, "system belongs to a batch; use gbmd_batch_step");
   s->target_step += nsteps;
-  return enqueue_steps(s->own, nsteps);
+  return take_steps(s->own, nsteps);
 }
 
 int gbmd_sync(gbmd_system* s) {
@@ -2328,9 +2376,12 @@ int gbmd_set_force_events(gbmd_system* s, void* ev_begin, void* ev_end) {
   const bool had = g->ev_begin != nullptr;
   g->ev_begin = b;
   g->ev_end = e;
-  if (had && b && g->exec_one && g->node_ev_begin && !g->graphs_dirty) {
-    CK(cudaGraphExecEventRecordNodeSetEvent(g->exec_one, g->node_ev_begin, b));
-    CK(cudaGraphExecEventRecordNodeSetEvent(g->exec_one, g->node_ev_end, e));
+  if (had && b) {   // the built graphs get the new events
+    for (StepGraphs& q : g->graphs) {
+      if (!q.built || !q.ev_begin) continue;
+      CK(cudaGraphExecEventRecordNodeSetEvent(q.one, q.ev_begin, b));
+      CK(cudaGraphExecEventRecordNodeSetEvent(q.one, q.ev_end, e));
+    }
     return GBMD_OK;
   }
   destroy_graphs(g);   // rebuilt with (or without) the records at the next step
@@ -2397,7 +2448,7 @@ int gbmd_batch_add(gbmd_batch* bh, gbmd_system* s, int32_t* slot) {
   }
   if (s->device != b->device) return fail(GBMD_ERR_BAD_ARG, "system and batch are on different devices");
   RET(sync_system(s));
-  CK(cudaStreamSynchronize(b->stream));
+  CK(wait_for(b->device, b->stream));
   int k = -1;
   for (size_t i = 0; i < b->members.size(); ++i)
     if (!b->members[i]) { k = (int)i; break; }
@@ -2422,7 +2473,7 @@ int gbmd_batch_remove(gbmd_batch* bh, int32_t slot) {
   RET(use_device(reinterpret_cast<Group*>(bh)->device));
   gbmd_system* s = b->members[slot];
   RET(sync_system(s));
-  CK(cudaStreamSynchronize(b->stream));
+  CK(wait_for(b->device, b->stream));
   b->members[slot] = nullptr;
   s->batch = nullptr;
   s->batch_slot = -1;
@@ -2437,7 +2488,7 @@ int gbmd_batch_step(gbmd_batch* bh, int64_t nsteps) {
   if (!b || nsteps < 0) return fail(GBMD_ERR_BAD_ARG, "bad argument");
   RET(use_device(reinterpret_cast<Group*>(bh)->device));
   for (auto* s : live(b)) s->target_step += nsteps;
-  return enqueue_steps(b, nsteps);
+  return take_steps(b, nsteps);
 }
 
 int gbmd_batch_sync(gbmd_batch* bh) {
@@ -2445,7 +2496,7 @@ int gbmd_batch_sync(gbmd_batch* bh) {
   Group* b = reinterpret_cast<Group*>(bh);
   if (!b) return fail(GBMD_ERR_BAD_ARG, "NULL batch");
   RET(use_device(reinterpret_cast<Group*>(bh)->device));
-  CK(cudaStreamSynchronize(b->stream));
+  CK(wait_for(b->device, b->stream));
   int first = GBMD_OK;
   std::string msg;
   for (auto* s : live(b)) {
@@ -2498,7 +2549,7 @@ int gbmd_batch_info(gbmd_batch* bh, int32_t* members, int64_t* particles, int64_
       if (!g || !g->d_ctl) continue;
       GroupCtl c{};
       CK(cudaMemcpyAsync(&c, g->d_ctl, sizeof(c), cudaMemcpyDeviceToHost, b->stream));
-      CK(cudaStreamSynchronize(b->stream));
+      CK(wait_for(b->device, b->stream));
       *launches += (int64_t)c.launches;
     }
   }
@@ -2509,7 +2560,7 @@ int gbmd_batch_destroy(gbmd_batch* bh) {
   Group* b = reinterpret_cast<Group*>(bh);
   if (!b) return fail(GBMD_ERR_BAD_ARG, "NULL batch");
   use_device(b->device);
-  cudaStreamSynchronize(b->stream);
+  wait_for(b->device, b->stream);
   for (auto* s : live(b)) {
     s->batch = nullptr;
     s->batch_slot = -1;

@@ -80,3 +80,39 @@ def test_a_batch_counts_the_launches_of_every_member():
     b.close()
     for s in ss:
         s.close()
+
+
+@pytest.mark.parametrize("n,resident", [(20000, True), (100_000, False)])
+def test_a_system_beside_work_on_another_stream_takes_no_launch_of_the_whole_chip(n, resident):
+    """While another stream's steps have not been waited for, a system's steps are single
+    launches, which the others' can run beside; the results are the same."""
+    import torch
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    w = wl.lj_fluid(n, 0.84, 1.2, seed=771)
+    a, b = (gbmd.System.from_workload(w, stream=x.cuda_stream) for x in streams)
+    a.sync()
+    b.sync()
+
+    def launches(s):
+        return s.info()["kernel_launches"]   # waits for the system's stream alone
+
+    start = launches(a)
+    assert launches(b) == start
+    a.step(64)                    # alone
+    b.step(64)                    # beside a
+    alone, beside = launches(a) - start, launches(b) - start
+    if resident:
+        assert alone == 1 and beside >= 64
+    else:                         # the rebuild by one kernel, and by seven
+        assert beside > alone >= 64
+    for x, y in zip(a.state(), b.state()):
+        assert np.array_equal(x, y)
+    start = launches(b)
+    b.step(64)                    # nothing pending elsewhere any more
+    if resident:
+        assert launches(b) - start == 1
+    a.step(64)
+    for x, y in zip((*a.state(), a.forces()), (*b.state(), b.forces())):
+        assert np.array_equal(x, y)
+    a.close()
+    b.close()
