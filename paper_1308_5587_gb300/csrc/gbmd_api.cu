@@ -133,7 +133,7 @@ struct Group {
   Tile *d_tp = nullptr, *d_tf = nullptr, *d_tc = nullptr, *d_ts = nullptr;
   Tile *d_tb = nullptr, *d_tbk = nullptr;   // staged force blocks; their window kernel
   Tile* d_te = nullptr;   // energy/virial launches: ev_tile(n) particles per tile, whatever
-                          // the tuning, so the FP64 sums do not depend on it
+                          // the force block, so the FP64 sums depend on the lanes alone
   int ev_tile = EV_TILE_P;   // the largest of them
   Tile *d_tt = nullptr, *d_tg = nullptr;   // tree-list systems: tiles over their trees'
                                            // leaves, and over the groups that query them

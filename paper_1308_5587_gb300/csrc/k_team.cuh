@@ -6,8 +6,8 @@
 // kernels.  Evaluating that node costs ~13 us a step (64k particles, mixed: 18.8 us for
 // steps without the nodes, 32.6 us with them), a launch ~2 us, and a rebuild seven
 // launches; in a batch, where some member rebuilds at nearly every step, every member
-// waits for the whole chain.  A team needs one barrier a step and five a rebuild, and
-// each system goes at its own pace.
+// waits for the whole chain.  A team needs one barrier a step (NVT: two) and three a rebuild
+// (a re-sort two more, a bucket that ran over two more), and each system goes at its own pace.
 //
 // Blocks keep contiguous ranges of chunks (32 / TPP particles, one warp), so a block's
 // gathers reuse its L1.  The sums over a particle's neighbours, the list rows and the

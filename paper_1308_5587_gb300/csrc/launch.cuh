@@ -8,7 +8,8 @@ namespace gbmd {
 
 constexpr int TILE_P = 256;     // particles per block of the streaming kernels
 // particles per FP64 energy/virial partial sum (a block of the energy launches), by the
-// system's size alone, so the sums depend on no tuning.  Up to EV_SMALL_N particles a
+// system's size, so the sums depend on the lanes per particle (a warp's 32 / TPP particles
+// are summed first; wide tiles hold TPP / 32 as many) but not on the force block.  Up to EV_SMALL_N particles a
 // block of 128 leaves SMs idle or unevenly loaded (FP64, N = 4,000: 32 blocks of 512
 // threads, 120 us; the whole readout 177 us with them, 68 with tiles of 32)
 constexpr int EV_TILE_P = 128, EV_TILE_SMALL = 32, EV_SMALL_N = 131072;
@@ -44,8 +45,8 @@ KernelCall copyback_call(const SysDev* d, const Tile* tiles_p, int ntiles, Group
 KernelCall blocks_call(const SysDev* d, const Tile* tiles_b, int ntiles, GroupCtl* ctl);
 KernelCall nlist_call(const SysDev* d, const Tile* tiles_c, int ntiles, GroupCtl* ctl, bool rel,
                       bool multi, bool staged);
-// all of the above for the single system d[0], by the grid of a cooperative launch (no
-// staged window, no tree); returns at once when the step asked for no rebuild
+// all of the above for the single system d[0], tree lists included, by the grid of a
+// cooperative launch (no staged window); returns at once when the step asked for no rebuild
 void* rebuild_func(bool multi);
 KernelCall rebuild_call(const SysDev* d, int blocks, GroupCtl* ctl, bool multi, int polls);
 // the same rows built by four warps per cell (tiles over (cell, part) items)
@@ -115,7 +116,8 @@ KernelCall nlist_export_call(const SysDev* d, const Tile* tiles_p, int ntiles, i
 cudaError_t launch(const KernelCall& k, cudaStream_t st);
 
 // the team kernel (k_team.cuh): many steps of one or more systems in one launch
-// one block an SM, 128 registers a thread: no spills, and the warps a small system fills;
+// one block an SM, 128 registers a thread, and the warps a small system fills (spilled, by
+// -Xptxas -v: 40 to 110 bytes in the mixed LJ instances, 200 to 220 in the FP64 ones);
 // the rest of the SM's 256 KB stays L1 for the force phase's gathers
 constexpr int TEAM_T = 512;
 constexpr size_t TEAM_SMEM = 112 * 1024;
