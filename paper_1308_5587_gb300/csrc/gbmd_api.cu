@@ -167,7 +167,6 @@ struct Group {
   int4* d_share = nullptr;
   TeamSync* d_sync = nullptr;
   size_t cap_share = 0, cap_sync = 0;
-  int polls = TEAM_POLLS;
   cudaStream_t side[TEAM_SIDES] = {};
   cudaEvent_t side_ev[TEAM_SIDES + 1] = {};
   Group* rest = nullptr;
@@ -536,9 +535,6 @@ int split_members(Group* g, const std::vector<gbmd_system*>& m) {
 int sync_layout(Group* g) {
   if (!g->layout_dirty) return GBMD_OK;
   std::vector<gbmd_system*> m = live(g);
-  g->polls = TEAM_POLLS;
-  // a test lets the waits run out
-  if (const char* ev = getenv("GBMD_TEAM_POLLS")) g->polls = std::max(0, atoi(ev));
   std::vector<SysDev> desc;
   std::vector<Tile> tp, tf, tc, ts, tb, tbk, te, tt, tg, tn;
   const int per_f = g->fblock / g->tpp;
@@ -622,9 +618,14 @@ int sync_layout(Group* g) {
     CK(cudaMemsetAsync(g->d_ctl, 0, sizeof(GroupCtl), g->stream));
   }
   // a wait that was given up leaves arrivals behind.  Its system stays stopped, so nothing
-  // meets them before the group's members change, which comes through here
-  CK(cudaMemsetAsync(&g->d_ctl->team, 0, sizeof(TeamSync), g->stream));
-  if (g->d_sync) CK(cudaMemsetAsync(g->d_sync, 0, g->cap_sync * sizeof(TeamSync), g->stream));
+  // meets them before the group's members change, which comes through here.  (GBMD_TEAM_POLLS=0:
+  // a test lets every wait run out at once)
+  const char* polls = getenv("GBMD_TEAM_POLLS");
+  const TeamSync clean{polls && polls[0] == '0' ? TEAM_CLOSED : 0ull, 0ull};
+  const std::vector<TeamSync> sync(std::max<size_t>(g->d_sync ? g->cap_sync : 0, 1), clean);
+  CK(cudaMemcpyAsync(&g->d_ctl->team, sync.data(), sizeof(TeamSync), cudaMemcpyHostToDevice, g->stream));
+  if (g->d_sync)
+    CK(cudaMemcpyAsync(g->d_sync, sync.data(), g->cap_sync * sizeof(TeamSync), cudaMemcpyHostToDevice, g->stream));
   auto up = [&](void* dst, const std::vector<Tile>& v) -> cudaError_t {
     if (v.empty()) return cudaSuccess;
     return cudaMemcpyAsync(dst, v.data(), v.size() * sizeof(Tile), cudaMemcpyHostToDevice, g->stream);
@@ -761,7 +762,7 @@ int coop_rebuild(const Group* g, bool alone, KernelCall* out) {
   TeamFit fit;
   RET(team_fit(rebuild_func(g->multi > 0), REBUILD_T, REBUILD_SMEM, g->device, &fit));
   if (fit.blocks_per_sm < 1) return GBMD_OK;
-  *out = rebuild_call(g->d_desc, fit.sms, g->d_ctl, g->multi > 0, g->polls);
+  *out = rebuild_call(g->d_desc, fit.sms, g->d_ctl, g->multi > 0);
   return GBMD_OK;
 }
 
@@ -881,7 +882,6 @@ int launch_team(Group* g, long long n) {
   TeamArgs a{};
   a.desc = g->d_desc;
   a.ctl = g->d_ctl;
-  a.polls = g->polls;
   if (p.shares) {
     a.share = g->d_share;
     a.sync = g->d_sync;

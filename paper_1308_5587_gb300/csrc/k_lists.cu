@@ -305,7 +305,7 @@ __global__ void __launch_bounds__(NS_T, 6) k_nlist_split(const SysDev* __restric
 // step with the node and seven kernels in its body, 28.2 us with this kernel).
 template <bool MULTI>
 __global__ void __launch_bounds__(REBUILD_T, 1) k_rebuild(const SysDev* __restrict__ sysv,
-                                                            GroupCtl* ctl, int polls) {
+                                                            GroupCtl* ctl) {
   constexpr int T = REBUILD_T;
   using Smem = TeamSmem<T, NL_SLOTS>;
   static_assert(sizeof(Smem) <= REBUILD_SMEM, "shared memory");
@@ -326,7 +326,6 @@ __global__ void __launch_bounds__(REBUILD_T, 1) k_rebuild(const SysDev* __restri
   tm.par = 0;
   tm.slot = nullptr;
   tm.word = &word;
-  tm.polls = polls;
   split_table(s, tab);
   __syncthreads();
   const unsigned r = team_rebuild<T, MULTI>(s, tm, sm, tab, step_of(s.flags), fw.do_sort != 0);
@@ -361,10 +360,10 @@ SIMPLE_CALL(blocks_call, k_blocks, 256)
 #undef SIMPLE_CALL
 
 void* rebuild_func(bool multi) { return multi ? (void*)k_rebuild<true> : (void*)k_rebuild<false>; }
-KernelCall rebuild_call(const SysDev* d, int blocks, GroupCtl* ctl, bool multi, int polls) {
+KernelCall rebuild_call(const SysDev* d, int blocks, GroupCtl* ctl, bool multi) {
   KernelCall k = make_call(rebuild_func(multi), blocks, REBUILD_T, REBUILD_SMEM);
   k.cooperative = true;
-  put(k, d); put(k, ctl); put(k, polls);
+  put(k, d); put(k, ctl);
   return k;
 }
 

@@ -56,7 +56,6 @@ __global__ void __launch_bounds__(TEAM_T, 1) k_team(TeamArgs a) {
   tm.par = 0;
   tm.slot = slot;
   tm.word = &word;
-  tm.polls = a.polls;
   const SysDev& s = a.desc[a.list[member]];
   // The flags change only after the team's first barrier, so every block reads the same.
   const FlagWords fw = load_flag_words(s.flags);

@@ -48,7 +48,7 @@ KernelCall nlist_call(const SysDev* d, const Tile* tiles_c, int ntiles, GroupCtl
 // all of the above for the single system d[0], tree lists included, by the grid of a
 // cooperative launch (no staged window); returns at once when the step asked for no rebuild
 void* rebuild_func(bool multi);
-KernelCall rebuild_call(const SysDev* d, int blocks, GroupCtl* ctl, bool multi, int polls);
+KernelCall rebuild_call(const SysDev* d, int blocks, GroupCtl* ctl, bool multi);
 // the same rows built by four warps per cell (tiles over (cell, part) items)
 KernelCall nlist_split_call(const SysDev* d, const Tile* tiles_n, int ntiles, GroupCtl* ctl, bool multi);
 // tree neighbour list (k_tree.cu): the boxes of every type's tree (one thread per
@@ -125,9 +125,6 @@ constexpr size_t TEAM_SMEM = 112 * 1024;
 constexpr int REBUILD_T = 768;
 constexpr size_t REBUILD_SMEM = 220 * 1024;
 constexpr int TEAM_MAX_CLUSTER = 16;
-// polls of a wait between blocks through memory, ~0.5 us each: two seconds; then the wait
-// is given up, the kernel returns and the system stops with DEV_TEAM
-constexpr int TEAM_POLLS = 1 << 22;
 struct TeamArgs {
   const SysDev* desc;
   const int* list;   // the systems of the launch (positions in desc), the largest first
@@ -138,7 +135,6 @@ struct TeamArgs {
   // blocks, its barrier in sync)
   const int4* share;
   TeamSync* sync;
-  int polls;         // of a wait in memory, at most
 };
 // two_in_one: mixed with two lanes a particle, one lane doing the work of both
 void* k_team_variant(int eval, int prec, int tpp, int mt, bool two_in_one);

@@ -20,6 +20,9 @@
 namespace gbmd {
 
 enum : unsigned { VOTE_NEED = 1u, VOTE_BAD = 2u, VOTE_LOST = 4u };
+// polls of a wait between blocks through memory, ~0.5 us each: two seconds; then the wait
+// is given up, the kernel returns and the system stops with DEV_TEAM
+constexpr int TEAM_POLLS = 1 << 22;
 
 // The team's cell sort takes buckets: the histogram's atomic places each particle in its
 // bin's bucket, every block scans the counts for itself, and each bin is sorted out of
@@ -49,7 +52,6 @@ struct Team {
   int par;                   // cluster: which vote slots are in use
   unsigned* slot;            // [2][TEAM_MAX_CLUSTER] in shared memory
   unsigned* word;            // one word in shared memory
-  int polls;                 // grid: of a wait, at most
 
   // Every thread of every block of the team: all of them have arrived, what they wrote
   // is visible, and the votes are ORed (VOTE_LOST: a wait ran out; the team stops).
@@ -79,13 +81,13 @@ struct Team {
       all += add;
       unsigned out;
       if ((unsigned)all == (unsigned)size) {
-        out = (((all >> 32) & 0xffffu) ? VOTE_NEED : 0u) | ((all >> 48) ? VOTE_BAD : 0u);
-        sync->arrive = 0ull;
+        out = (((all >> 32) & 0xffffu) ? VOTE_NEED : 0u) | (((all & ~TEAM_CLOSED) >> 48) ? VOTE_BAD : 0u);
+        sync->arrive = all & TEAM_CLOSED;
         const unsigned long long rel = ((unsigned long long)(gen + 1u) << 8) | out;
         asm volatile("st.release.gpu.global.u64 [%0], %1;" ::"l"(&sync->release), "l"(rel) : "memory");
       } else {
         out = VOTE_LOST;
-        for (int k = 0; k < polls; ++k) {
+        for (int k = all & TEAM_CLOSED ? TEAM_POLLS : 0; k < TEAM_POLLS; ++k) {
           unsigned long long rel;
           asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(rel) : "l"(&sync->release) : "memory");
           if ((unsigned)(rel >> 8) == gen + 1u) {
