@@ -751,14 +751,17 @@ std::vector<KernelCall> step_calls(const Group* g, cudaGraphConditionalHandle co
 
 // The rebuild of a step of one system alone as one cooperative kernel after the step
 // kernel (no conditional node); null func: the group does not take it.  Up to COOP_MAX_N
-// particles: the separate kernels of a big rebuild balance better over the SMs than
-// resident warps do (KA 10^6: 312 us a step with the conditional node, 357 with this;
-// N = 200,000: 70 and 66).
-constexpr int COOP_MAX_N = 400000;
+// particles, with several types on the cell list COOP_MAX_TYPES_N: the separate kernels of a
+// big rebuild balance better over the SMs than resident warps do.  us a step with the
+// conditional node / with this: one type, N = 250,000 83.7 / 78.1, 400,000 118.3 / 114.8,
+// 700,000 163.8 / 164.6, 10^6 245 / 254; KA 90,000 55.9 / 52.7, 250,000 109.7 / 109.1, 400,000
+// 163 / 171, 10^6 314 / 351; WCA 1:10 on the tree 250,000 59 / 51.
+constexpr int COOP_MAX_N = 400000, COOP_MAX_TYPES_N = 262144;
 int coop_rebuild(const Group* g, bool alone, KernelCall* out) {
   out->func = nullptr;
   std::vector<gbmd_system*> m = live(g);
-  if (!alone || m.size() != 1 || m[0]->h.staged || m[0]->h.n > COOP_MAX_N) return GBMD_OK;
+  if (!alone || m.size() != 1 || m[0]->h.staged) return GBMD_OK;
+  if (m[0]->h.n > (g->multi && !m[0]->h.tree ? COOP_MAX_TYPES_N : COOP_MAX_N)) return GBMD_OK;
   TeamFit fit;
   RET(team_fit(rebuild_func(g->multi > 0), REBUILD_T, REBUILD_SMEM, g->device, &fit));
   if (fit.blocks_per_sm < 1) return GBMD_OK;
