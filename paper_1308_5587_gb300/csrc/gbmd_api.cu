@@ -696,7 +696,7 @@ std::vector<KernelCall> rebuild_calls(const Group* g) {
 KernelCall plain_force_call(const Group* g, int readout = 0) {
   StepArgs sa;
   sa.readout = readout;
-  return force_call(g->precision, g->multi, MODE_FORCE, g->tpp, g->fblock, g->d_desc, g->d_tf,
+  return force_call(g->precision, g->multi, readout ? MODE_READ : MODE_FORCE, g->tpp, g->fblock, g->d_desc, g->d_tf,
                     g->ntf, g->d_ctl, sa, g->eval);
 }
 

@@ -431,10 +431,11 @@ __device__ __forceinline__ void gather_fp64(const SysDev& s, const longlong4_32a
   }
 }
 
-// MODE_FORCE: forces at the current positions, and with `readout` the rows of a readout
-// in tag order and the Snapshot (one system; single steps of N = 500 with their forces
-// 63 -> 59 us, 48 replicas' frames and log lines with 64 steps 17,097 -> 16,766, with the
-// reduction by warps); MODE_EV: also the
+// MODE_FORCE: forces at the current positions; MODE_READ: also the rows of a readout, as
+// `readout` asks, in tag order and the Snapshot (one system; single steps of N = 500 with
+// their forces 63 -> 59 us, 48 replicas' frames and log lines with 64 steps 17,097 ->
+// 16,766, with the reduction by warps.  A kernel of its own: with the rows under a condition
+// in the plain one, that took 181 us at KA 10^6 instead of 163); MODE_EV: also the
 // energy / virial / v.v partial sums; MODE_STEP: the step kernel -- forces, then each
 // particle's velocity Verlet update into the next shadow buffer (step_core.cuh), then
 // the end-of-step decisions by the last of `total_blocks` blocks.  A system that is
@@ -449,7 +450,7 @@ __device__ __forceinline__ void force_body(const SysDev* __restrict__ sysv, cons
   const SysDev& s = sysv[t.sys];
   if (threadIdx.x == 0 && t.first == 0) atomicAdd(&s.flags->launches, 1ull);
   if (threadIdx.x == 0 && blockIdx.x == 0) atomicAdd(&ctl->launches, 1ull);
-  if (MODE == MODE_FORCE && readout && threadIdx.x == 0 && blockIdx.x == 0) take_snapshot(s);
+  if (MODE == MODE_READ && threadIdx.x == 0 && blockIdx.x == 0) take_snapshot(s);
   const FlagWords fw = load_flag_words(s.flags);
   const longlong2 sl = load_flag_pair(&s.flags->step);   // (step, step_limit)
   // Another block of this launch may set the error in the meantime (step_tail), so the
@@ -512,7 +513,7 @@ __device__ __forceinline__ void force_body(const SysDev* __restrict__ sysv, cons
       }
     } else if (valid && h == 0) {
       s.f32[i] = make_float4(Fx, Fy, Fz, EV ? E : 0.f);
-      if (MODE == MODE_FORCE && readout) read_out(s, i, {Fx, Fy, Fz}, fw.v_full, readout);
+      if (MODE == MODE_READ) read_out(s, i, {Fx, Fy, Fz}, fw.v_full, readout);
     }
     if (EV) {
       double vals[NPART] = {valid ? (double)E : 0.0};
@@ -554,7 +555,7 @@ __device__ __forceinline__ void force_body(const SysDev* __restrict__ sysv, cons
       }
     } else if (valid && h == 0) {
       s.f64[i] = make_double4_32a(fx, fy, fz, EV ? e : 0.0);
-      if (MODE == MODE_FORCE && readout) read_out(s, i, {fx, fy, fz}, fw.v_full, readout);
+      if (MODE == MODE_READ) read_out(s, i, {fx, fy, fz}, fw.v_full, readout);
     }
     if (EV) {
       double vals[NPART] = {valid ? e : 0.0};
@@ -637,6 +638,7 @@ void* k_force_mode(int mode) {
       if constexpr (PREC == GBMD_MIXED && TPP == 1) return (void*)k_force_step1<MT, EVAL>;
       else return (void*)k_force<PREC, TPP, MT, MODE_STEP, EVAL>;
     case MODE_NVT_A: return (void*)k_force<PREC, TPP, MT, MODE_NVT_A, EVAL>;
+    case MODE_READ: return (void*)k_force<PREC, TPP, MT, MODE_READ, EVAL>;
     default: return (void*)k_force<PREC, TPP, MT, MODE_FORCE, EVAL>;
   }
 }

@@ -58,16 +58,16 @@ constexpr int TREE_WARPS = 8;   // groups a block
 constexpr int TREE_G = 8;       // particles of a group: TREE_G x 4 lanes
 KernelCall tree_build_call(const SysDev* d, const Tile* tiles_l, int ntiles, GroupCtl* ctl);
 KernelCall tree_nlist_call(const SysDev* d, const Tile* tiles_g, int ntiles, GroupCtl* ctl);
-// pair force kernels.  MODE_FORCE: forces at the current positions (readouts);
-// MODE_EV: also energy / virial / v.v partial sums (+ per-particle arrays when the
-// descriptor has them); MODE_STEP: the step kernel -- forces, the velocity Verlet
+// pair force kernels.  MODE_FORCE: forces at the current positions; MODE_READ: also a
+// readout's rows (sa.readout); MODE_EV: also energy / virial / v.v partial sums (+
+// per-particle arrays when the descriptor has them); MODE_STEP: the step kernel -- forces, the velocity Verlet
 // update of every particle into the next shadow buffer, and the end-of-step
 // decisions by the last of sa.total_blocks blocks over the step's force launches.
 // MODE_NVT_A: the first half of an NVT step -- forces, the closing half kick and
 // thermostat scaling of the previous step, v.v partial sums; a system's last block
 // updates its thermostat.  nvt_b_call: the second half (opening scaling and kick, drift,
 // shadow, rebuild check, end-of-step decisions).
-enum { MODE_FORCE = 0, MODE_EV = 1, MODE_STEP = 2, MODE_NVT_A = 3 };
+enum { MODE_FORCE = 0, MODE_EV = 1, MODE_STEP = 2, MODE_NVT_A = 3, MODE_READ = 4 };
 // which step configurations take wide tiles, a warp a particle (all modes of one do, so
 // that a readout's forces are the step's): not the register-capped step kernel of one
 // lane a particle
@@ -78,7 +78,7 @@ struct StepArgs {
   int total_blocks = 0;     // blocks of all the step's force launches
   cudaGraphConditionalHandle cond = 0;   // the rebuild conditional of the step graph
   int use_cond = 0;
-  int readout = 0;          // MODE_FORCE: the READ_ bits of what to write out
+  int readout = 0;          // MODE_READ: the READ_ bits of what to write out
 };
 // eval: the PairEval of every system of the launch
 KernelCall force_call(int prec, int multi, int mode, int tpp, int block, const SysDev* d,
