@@ -435,7 +435,7 @@ __device__ __forceinline__ void gather_fp64(const SysDev& s, const longlong4_32a
 // `readout` asks, in tag order and the Snapshot (one system; single steps of N = 500 with
 // their forces 63 -> 59 us, 48 replicas' frames and log lines with 64 steps 17,097 ->
 // 16,766, with the reduction by warps.  A kernel of its own: with the rows under a condition
-// in the plain one, that took 181 us at KA 10^6 instead of 163); MODE_EV: also the
+// in the plain one, that took 181 us at KA 10^6 instead of 156); MODE_EV: also the
 // energy / virial / v.v partial sums; MODE_STEP: the step kernel -- forces, then each
 // particle's velocity Verlet update into the next shadow buffer (step_core.cuh), then
 // the end-of-step decisions by the last of `total_blocks` blocks.  A system that is
