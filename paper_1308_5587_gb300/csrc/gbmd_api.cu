@@ -963,8 +963,9 @@ int enqueue_steps(Group* g, long long n, bool alone) {
   return GBMD_OK;
 }
 
-// the same as a caller's steps
+// the same for a caller, whose stream has work from here on
 int take_steps(Group* g, long long n) {
+  if (n <= 0) return GBMD_OK;
   const bool al = alone(g->device, g->stream);
   enqueued(g->device, g->stream);
   return enqueue_steps(g, n, al);

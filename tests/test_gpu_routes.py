@@ -116,3 +116,18 @@ def test_a_system_beside_work_on_another_stream_takes_no_launch_of_the_whole_chi
         assert np.array_equal(x, y)
     a.close()
     b.close()
+
+
+def test_a_call_of_no_steps_leaves_its_stream_idle():
+    import torch
+    streams = [torch.cuda.Stream() for _ in range(2)]
+    w = wl.lj_fluid(20000, 0.84, 1.2, seed=772)
+    a, b = (gbmd.System.from_workload(w, stream=x.cuda_stream) for x in streams)
+    for s in (a, b):
+        s.sync()
+    a.step(0)
+    start = b.info()["kernel_launches"]
+    b.step(64)
+    assert b.info()["kernel_launches"] - start == 1
+    a.close()
+    b.close()
